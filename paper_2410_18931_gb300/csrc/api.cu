@@ -84,17 +84,18 @@ wsr_status make_views(const wsr_camera* cams, int32_t n_cams, const wsr_tiles* t
 }
 
 struct WsLayout {
-    size_t cursor, block_sums, order, buckets, bg_tiles, total;
+    size_t cursor, block_sums, order, buckets, bg_tiles, bin_base, total;
 };
 
-// The tile order of the persistent schedule is only part of its layout.
-WsLayout ws_layout(const Views& vs) {
+// The tile order of the persistent schedule is only part of its layout; the binning's rows of counters per
+// block (bin_base) come last and are left out of the static scratch.
+WsLayout ws_layout(const Views& vs, bool with_base = true) {
     WsLayout L;
     const size_t nb = (size_t)(vs.total_tiles + kScanTile - 1) / kScanTile;
     L.cursor = kWsHeader;
     L.block_sums = L.cursor + align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
     L.total = L.block_sums + align256(sizeof(unsigned long long) * (nb + 1));
-    L.order = L.buckets = L.bg_tiles = 0;
+    L.order = L.buckets = L.bg_tiles = L.bin_base = 0;
     if (vs.schedule == WSR_SCHEDULE_PERSISTENT) {
         L.order = L.total;
         L.buckets = L.order + align256(sizeof(unsigned) * (size_t)vs.total_tiles);
@@ -104,6 +105,12 @@ WsLayout ws_layout(const Views& vs) {
         L.bg_tiles = L.total;
         L.total = L.bg_tiles + align256(4 * sizeof(float) * (size_t)vs.total_tiles);
     }
+    if (!with_base) return L;
+    int t_max = 0;
+    for (int v = 0; v < vs.n; ++v) t_max = vs.v[v].tiles_x * vs.v[v].tiles_y > t_max ? vs.v[v].tiles_x * vs.v[v].tiles_y
+                                                                                     : t_max;
+    L.bin_base = L.total;
+    L.total += align256(sizeof(unsigned) * (size_t)vs.total_tiles * (size_t)bin_blocks_per_view(vs.n, t_max));
     return L;
 }
 
@@ -264,15 +271,18 @@ wsr_status wsr_project(const wsr_gaussians* g, const wsr_camera* cams, int32_t n
     return cuda_status(launch_project(gp, vs, wd, records, (cudaStream_t)stream));
 }
 
+// The binning's rows of counters per block in a caller's workspace (nullptr: none in this layout).
+static unsigned* bin_base(const WsLayout& L, void* workspace) {
+    return L.bin_base != 0 && L.total > L.bin_base ? (unsigned*)((char*)workspace + L.bin_base) : nullptr;
+}
+
 static wsr_status bin_count_impl(const float* records, int64_t n, const Views& vs, uint32_t* tile_offsets,
-                                 unsigned long long capacity, void* workspace, cudaStream_t s) {
-    const WsLayout L = ws_layout(vs);
+                                 unsigned long long capacity, void* workspace, const WsLayout& L, cudaStream_t s) {
     char* ws = (char*)workspace;
     WsHeader* hdr = (WsHeader*)ws;
     unsigned* cursor = (unsigned*)(ws + L.cursor);
     unsigned* bsum = (unsigned*)(ws + L.block_sums);
-    WSR_CUDA(cudaMemsetAsync(&hdr->err, 0, sizeof(int), s));
-    WSR_CUDA(launch_bin_count(records, n, vs, cursor, s));
+    WSR_CUDA(launch_bin_count(records, n, vs, cursor, bin_base(L, workspace), s));
     const bool persistent = vs.schedule == WSR_SCHEDULE_PERSISTENT;
     WSR_CUDA(launch_scan(vs, cursor, bsum, tile_offsets, capacity, hdr, (unsigned*)(ws + L.buckets),
                          persistent ? (unsigned*)(ws + L.order) : nullptr, s));
@@ -289,7 +299,7 @@ wsr_status wsr_bin_count(const float* records, int64_t n, const wsr_camera* cams
     if (n < 0 || (n > 0 && (!records || !aligned16(records))) || !tile_offsets) return WSR_ERR_INVALID_ARG;
     if (!aligned4(tile_offsets)) return WSR_ERR_INVALID_ARG;
     if ((unsigned long long)n * (unsigned long long)n_cams > 0xffffffffull) return WSR_ERR_INVALID_ARG;
-    return bin_count_impl(records, n, vs, tile_offsets, ~0ull, workspace, (cudaStream_t)stream);
+    return bin_count_impl(records, n, vs, tile_offsets, ~0ull, workspace, ws_layout(vs), (cudaStream_t)stream);
 }
 
 wsr_status wsr_bin(const float* records, int64_t n, const wsr_camera* cams, int32_t n_cams, const wsr_tiles* tiles,
@@ -304,10 +314,10 @@ wsr_status wsr_bin(const float* records, int64_t n, const wsr_camera* cams, int3
     if (!aligned4(tile_offsets) || !aligned4(tile_list) || !aligned8(total_dev)) return WSR_ERR_INVALID_ARG;
     if ((unsigned long long)n * (unsigned long long)n_cams > 0xffffffffull) return WSR_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, workspace, s));
     const WsLayout L = ws_layout(vs);
+    WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, workspace, L, s));
     char* ws = (char*)workspace;
-    WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), tile_list, list_capacity,
+    WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), bin_base(L, ws), tile_list, list_capacity,
                                 (WsHeader*)ws, s));
     if (vs.det) WSR_CUDA(launch_sort_segments(vs, tile_offsets, tile_list, (WsHeader*)ws, s));
     if (total_dev)
@@ -333,11 +343,11 @@ wsr_status wsr_bin_static(const float* records, int64_t n, const wsr_camera* cam
     WSR_TRY(static_scratch(s, &scratch));
     Views vb = vs;                 // the binning's part of the layout (no backward regions)
     vb.det = 0;
-    if (ws_layout(vb).total > kStaticBytes) return WSR_ERR_UNSUPPORTED;
-    WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, scratch, s));
-    const WsLayout L = ws_layout(vs);
+    const WsLayout L = ws_layout(vb, false);
+    if (L.total > kStaticBytes) return WSR_ERR_UNSUPPORTED;
+    WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, scratch, L, s));
     char* ws = (char*)scratch;
-    WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), tile_list, list_capacity,
+    WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), nullptr, tile_list, list_capacity,
                                 (WsHeader*)ws, s));
     if (vs.det) WSR_CUDA(launch_sort_segments(vs, tile_offsets, tile_list, (WsHeader*)ws, s));
     if (total_dev)
