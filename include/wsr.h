@@ -132,8 +132,7 @@ enum {
  * the render schedule and the backward's Gaussians per block.  With
  * WSR_SCHEDULE_PERSISTENT, wsr_bin also orders the tiles by decreasing
  * instance count (a bucketed longest-first order kept in the workspace) and
- * the render calls launch one block per resident slot (wsr_render_fwd: at
- * most 16 warps per SM, the forward's fastest grid) that takes tiles from
+ * the render calls launch one block per resident slot that takes tiles from
  * that order through a counter in the workspace; the same workspace and tiles
  * must then be passed to wsr_bin and the renderers.  `chunk` is how many of a
  * tile's Gaussians one block of wsr_render_bwd takes at a time: 0 for the
@@ -456,9 +455,10 @@ wsr_status wsr_bin_static(const float* records, int64_t n, const wsr_camera* cam
  * written to count_dev [3] (device uint64, overwritten, 8-byte aligned):
  *   [0] (pixel, Gaussian) pairs with q <= 9, i.e. the terms of the sums of
  *       Eq. 7 (the algorithmic work of both render kernels);
- *   [1] (pixel, Gaussian) slots wsr_render_fwd evaluates: for each Gaussian of
- *       a tile, the pixels of every warp whose region of the tile its footprint
- *       reaches (the forward tests q at each of them);
+ *   [1] (pixel, Gaussian) slots wsr_render_fwd evaluates: it walks the
+ *       Gaussians that reach an 8x8 region of a tile four at a time, so 256
+ *       slots per round of four (of each batch of the tile's list), the last
+ *       round's idle quarters included; 64 per Gaussian in 8x8 tiles;
  *   [2] (pixel, Gaussian) slots wsr_render_bwd evaluates: for each Gaussian
  *       of a tile, the rows from its first span to its last, each of tile
  *       width columns, or of half the tile width when none of its row spans

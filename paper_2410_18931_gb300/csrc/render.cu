@@ -1,11 +1,11 @@
 // Per-pixel Weighted Sum Rendering, forward and backward (Eq. 7).
 //
 // One thread block per tile (or, with the persistent schedule, one per
-// resident slot taking tiles longest first).  Each warp of the block streams
-// the tile's Gaussian list (unordered: Eq. 7 is a sum) through shared memory
-// on its own, 32 records at a time, keeping those whose footprint reaches its
-// rows; every thread owns a 2x2 block of pixels (two columns share each
-// paired float2 FP32 instruction) and accumulates, in FP32 registers,
+// resident slot taking tiles longest first).  A warp takes an 8x8 region of
+// the tile and walks the Gaussians of the tile's list (unordered: Eq. 7 is a
+// sum) that reach it, a quarter warp per Gaussian; every thread owns 2x4
+// pixels (two columns share each paired float2 FP32 instruction) and
+// accumulates, in FP32 registers,
 //     N += (c u w) e,   D += (u w) e,   e = exp(-q/2) = 2^(-q'),   q <= 9
 // with q' = q log2(e)/2 evaluated from the record's sum of squares
 // q' = (qs dy + qw dx)^2 + qd dx^2, which has no cancellation even for
@@ -42,17 +42,6 @@ template <int CH>
 struct BwdThreads {
     static constexpr int value = CH < 128 ? 2 * CH : 256;
 };
-
-// Asynchronous 16-byte global-to-shared copies (both addresses 16-byte aligned).
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 
 // A lane count as a type, to instantiate one walk of the backward per group size.
 template <int N>
@@ -128,127 +117,181 @@ struct TileShape {
     static_assert(TH % PPT == 0 && NT % 32 == 0, "whole warps");
 };
 
-// Forward tile shape: each thread owns a PX x 2 block of pixels (PX = 2 or 1),
-// so two horizontally adjacent pixels share one paired (float2) FP32 op.
-template <int TW, int TH, int PX>
+// Forward.  A tile is cut into 8x8 regions, one warp each, and its list into S slices, each walked by a group of
+// one warp per region.  The warps of a group stage a batch together, each thread one record: the walk constants
+// into shared memory and, per region, whether the footprint reaches it.  Each warp then lists its region's
+// Gaussians and walks them four at a time, one per quarter warp: eight threads with 2x4 pixels each cover the
+// region, so the walk constants and the terms of a column pair are read and formed once for eight pixels, and
+// the quarters' sums are added once per tile.
+//   It is bound by the FP32 pipe (its paired instructions issue every 2.4 cycles from distinct registers, not
+// every 2) and by the shared loads beside them.  16x16 tiles at 1M Gaussians and 1920x1080, persistent: 457 us
+// with a warp per 16x8 pixels, 2x2 pixels per thread and a Gaussian per warp (1.96 pixel slots per pair, each
+// warp staging the whole list); 414 us with that split and quarter warps on 8x8 regions; 363 us with the shared
+// staging and a warp per region.  One block per tile: 566 -> 399 us, 95 -> 60 us for 200k at 1280x720.
+//   20 warps per SM (at most 96 registers a thread): 363 us against 367 at 16, 379 at 24 and 389 at 28.
+constexpr int kFwdWarpsPerSM = 20;
+
+template <int TW, int TH>
 struct FwdShape {
-    static constexpr int PY = 2;
-    static constexpr int BX = TW / PX;                  // thread columns
-    static constexpr int NT = (TW / PX) * (TH / PY);    // threads per block
-    static constexpr int NW = NT / 32;
-    static_assert(NT % 32 == 0 && 32 % BX == 0, "whole warps of whole thread rows");
-    // first and last pixel row (within the tile) of warp w
-    __host__ __device__ static constexpr int row_lo(int w) { return (32 * w / BX) * PY; }
-    __host__ __device__ static constexpr int row_hi(int w) { return ((32 * w + 31) / BX) * PY + PY - 1; }
+    static constexpr int RX = TW / 8, RY = TH / 8, NR = RX * RY;
+    static_assert(TW % 8 == 0 && TH % 8 == 0 && NR <= 4, "whole regions");
 };
 
-template <int TW, int TH, int PX>
+// Which of the tile's 8x8 regions a footprint q' <= kQMax can reach, one bit each (row by row); (gx, gy) is the
+// tile's first pixel centre less the mean.  Eight pixel rows cut the ellipse in a convex part whose x-extent
+// [x_l, x_r] has a closed form (as in the binning: x(dy) = (-B' dy +- sqrt(A' QM - det' dy^2)) / A' at the row
+// of the band nearest the ellipse's rightmost and leftmost point); a region is reached when that extent,
+// widened far beyond its rounding, meets the region's pixel-centre columns.  Every comparison is "not outside":
+// NaN counts as reached.
+template <int RX, int RY>
+__device__ __forceinline__ unsigned regions_hit(const float4 a, const float qd, const float gx, const float gy) {
+    const float QM = kQMax * 1.0001f + 1e-4f;
+    const float A = fmaf(a.w, a.w, qd), ia = rcp_approx(A), det = qd * a.z * a.z, aq = A * QM;
+    const float dxm = sqrt_approx(QM * rcp_approx(qd));         // half-width of the ellipse
+    const float dys = -(a.w * rcp_approx(a.z)) * dxm;           // dy of its rightmost point
+    const float slope = a.z * a.w * ia, margin = fminf(2e-3f * dxm, 1e6f) + 0.01f;
+    unsigned hit = 0u;
+#pragma unroll
+    for (int b = 0; b < RY; ++b) {
+        const float ya = gy + (float)(8 * b), yb = ya + 7.0f;   // the band's pixel-centre rows
+        const float dn = fminf(fmaxf(0.0f, ya), yb);
+        const float dr = fminf(fmaxf(dys, ya), yb), dl = fminf(fmaxf(-dys, ya), yb);
+        const float xr = fmaf(-slope, dr, sqrt_approx(fmaxf(fmaf(-det * dr, dr, aq), 0.0f)) * ia) + margin;
+        const float xl = fmaf(-slope, dl, -sqrt_approx(fmaxf(fmaf(-det * dl, dl, aq), 0.0f)) * ia) - margin;
+        const bool out = det * dn * dn > aq * 1.001f;
+#pragma unroll
+        for (int c = 0; c < RX; ++c)
+            if (!(out || xl > gx + (float)(8 * c + 7) || xr < gx + (float)(8 * c))) hit |= 1u << (b * RX + c);
+    }
+    return hit;
+}
+
+// A group's shared memory: two batches of 32 list entries per warp, and each warp's list of the batch's
+// Gaussians that reach its region.  Walk constants, 48 bytes per Gaussian: (qs, qw, r_0, qd),
+// (qd g_x^2, 2 qd g_x, c_r u w, c_g u w), (c_b u w, u w), with g the tile's first pixel centre less the mean and
+// r_0 = qs g_y + qw g_x.  The last entry lies outside every pixel's cutoff.
+template <int NR>
+struct FwdStage {
+    float4 g[2][32 * NR + 1][3];
+    unsigned hits[2][NR][NR];                       // per region: which of each warp's 32 entries reach it
+    unsigned short list[NR][4][8 * NR + 2];         // per region and quarter warp: byte offsets into g
+};
+
+template <int TW, int TH, int S>
 __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restrict__ rec,
                                          const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
                                          const Views& vs, const float* __restrict__ wparams,
                                          float* __restrict__ out_rgb, float* __restrict__ out_den) {
-    using S = FwdShape<TW, TH, PX>;
-    constexpr int NW = S::NW;
-    // per warp, the Gaussians of its current batch that reach its rows
-    __shared__ float4 s0[NW][32];   // qs, qw, c_r u w, c_g u w
-    __shared__ float2 s2[NW][32];   // c_b u w, u w
-    __shared__ float4 s3[NW][32];   // at the tile's first pixel centre: r, qd dx^2, 2 qd dx; and qd
-    __shared__ float4 sraw[NW][2][32][3];   // per warp, two batches of records in flight (cp.async)
+    using F = FwdShape<TW, TH>;
+    constexpr int RX = F::RX, NR = F::NR, BATCH = 32 * NR;
+    union GroupMem {
+        FwdStage<NR> st;
+        float4 px[TW * TH];             // the slice's sums, at the end
+    };
+    __shared__ __align__(16) unsigned char s_mem[S][sizeof(GroupMem)];
 
+    // The slice's batches of list entries, each thread staging one; the next batch's records are loaded while
+    // this one is walked, and the list entries of the one after that.
+    const unsigned start = offsets[tile], end = offsets[tile + 1];
+    const float wB = __ldg(wparams + 2);
+    const float cB0 = __ldg(wparams + 3) * wB, cB1 = __ldg(wparams + 4) * wB, cB2 = __ldg(wparams + 5) * wB;
     const TileCoord tc = tile_coord(vs, tile);
     const View& V = vs.v[tc.v];
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int x0 = tc.tx * TW + (tid % S::BX) * PX;
-    const int y0 = tc.ty * TH + (tid / S::BX) * S::PY;
-    // offsets of the block's pixels from the tile's first pixel (PX == 1: the first column only, its two
-    // rows paired instead)
-    const float2 ox = f2((float)(x0 - tc.tx * TW), (float)(x0 - tc.tx * TW + 1));
-    const float oy0 = (float)(y0 - tc.ty * TH), oy1 = oy0 + 1.0f;
-    // the warp's pixel-centre rectangle
-    const float xl = (float)(tc.tx * TW) + 0.5f, xh = xl + (float)(TW - 1);
-    const float yl = (float)(tc.ty * TH + S::row_lo(w)) + 0.5f, yh = (float)(tc.ty * TH + S::row_hi(w)) + 0.5f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = lane >> 3, o8 = lane & 7;
+    const int w = warp % NR, slice = warp / NR;     // the warp's region, and its group
+    const int x_org = tc.tx * TW, y_org = tc.ty * TH;
+    FwdStage<NR>& st = reinterpret_cast<GroupMem*>(s_mem[slice])->st;
+    auto group_sync = [&] {
+        if constexpr (NR == 1) __syncwarp();
+        else if constexpr (S == 1) __syncthreads();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + slice), "n"(32 * NR) : "memory");
+    };
+    // a thread's 2x4 pixels (columns, rows) of the region, as offsets from the tile's first pixel
+    const float2 ox = f2((float)(8 * (w % RX) + 2 * (o8 & 3)), (float)(8 * (w % RX) + 2 * (o8 & 3) + 1));
+    const float oy0 = (float)(8 * (w / RX) + 4 * (o8 >> 2));
 
-    // accumulators per pixel (column c, row r): (N_r, N_g) and (N_b, D)
-    float2 rg[2][2], bd[2][2];
+    // accumulators per pixel (row r, column c): (N_r, N_g) and (N_b, D)
+    float2 rg[4][2], bd[4][2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 2; ++c) rg[r][c] = bd[r][c] = f2(0.f, 0.f);
 
-    // Each warp takes the tile's list 32 Gaussians at a time on its own (no block barrier): a lane
-    // takes one record and, with several warps per tile, tests whether the footprint reaches a pixel
-    // centre of the warp's rows (exact ellipse-rectangle test); the hits are compacted and walked.
-    // The next batch's records are copied into shared memory (cp.async) while the warp walks this one.
-    const unsigned start = offsets[tile], end = offsets[tile + 1];
-    unsigned nidx = start + lane < end ? list[start + lane] : 0u;       // the next batch's record index
-    auto fetch = [&](unsigned b, int buf) {
-        if (b + lane < end) {
+    if (w == 0 && lane < 2) {
+        st.g[lane][BATCH][0] = make_float4(0.f, 0.f, 1e4f, 0.f);
+        st.g[lane][BATCH][1] = st.g[lane][BATCH][2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    unsigned base = start + (unsigned)(BATCH * slice);
+    const int me = 32 * w + lane;
+    unsigned nidx = base + me < end ? list[base + me] : 0u;
+    float4 na, nb;
+    float ncb;
+    auto fetch = [&](unsigned b) {
+        na = nb = make_float4(0.f, 0.f, 0.f, 0.f);
+        ncb = 0.f;
+        if (b + me < end) {
             const float4* p = rec + 3ull * nidx;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) cp_async16(&sraw[w][buf][lane][q], p + q);
+            na = __ldg(p);
+            nb = __ldg(p + 1);
+            ncb = __ldg(reinterpret_cast<const float*>(p + 2));
         }
-        cp_async_commit();
-        nidx = b + 32 + lane < end ? list[b + 32 + lane] : 0u;
+        nidx = b + BATCH * S + me < end ? list[b + BATCH * S + me] : 0u;
     };
-    fetch(start, 0);
+    fetch(base);
     int buf = 0;
-    for (unsigned base = start; base < end; base += 32, buf ^= 1) {
-        const int cnt = (int)min(32u, end - base);
-        fetch(base + 32, buf ^ 1);                      // an empty group past the end
-        cp_async_wait<1>();                             // this batch's copies have landed
-        __syncwarp();
-        bool hit = false;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        float cb = 0.f;
-        if (lane < cnt) {
-            a = sraw[w][buf][lane][0];
-            b = sraw[w][buf][lane][1];
-            cb = sraw[w][buf][lane][2].x;
-            hit = NW == 1 || footprint_hits(a.x, a.y, a.z, a.w, b.x, xl, xh, yl, yh);
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, hit);
-        const int nj = __popc(bal);
-        __syncwarp();                                   // the previous batch's walk is done with the arrays
-        if (hit) {
-            const int k = __popc(bal & ((1u << lane) - 1u));
-            s0[w][k] = make_float4(a.z, a.w, b.z, b.w);
-            s2[w][k] = f2(cb, b.y);
-            const float gx = (float)(tc.tx * TW) + 0.5f - a.x, gy = (float)(tc.ty * TH) + 0.5f - a.y;
-            s3[w][k] = make_float4(fmaf(a.z, gy, a.w * gx), b.x * gx * gx, 2.0f * b.x * gx, b.x);
-        }
-        __syncwarp();
-#pragma unroll 8
-        for (int k = 0; k < nj; ++k) {
-            const float4 g = s0[w][k];
-            const float2 cbuw = s2[w][k];
-            const float4 t = s3[w][k];
-            const float qs = g.x, qw = g.y;
-            const float2 crg = f2(g.z, g.w);
-            // q' = r^2 + qd dx^2 with dx = g_x + o_x: qd dx^2 = qd g_x^2 + o_x (2 qd g_x + o_x qd) and
-            // r = r_0 + qs o_y + qw o_x from the values at the tile's first pixel centre
-            if constexpr (PX == 1) {
-                // one column, its two rows paired: the same dx, so the same qd dx^2
-                const float P1 = fmaf(ox.x, fmaf(ox.x, t.w, t.z), t.y);
-                const float base = fmaf(qw, ox.x, t.x);
-                const float2 rr = __ffma2_rn(f2(qs, qs), f2(oy0, oy1), f2(base, base));
-                const float2 q = __ffma2_rn(rr, rr, f2(P1, P1));
-                if (q.x <= kQMax) {
-                    const float e = ex2_approx(-q.x);
-                    rg[0][0] = __ffma2_rn(crg, f2(e, e), rg[0][0]);
-                    bd[0][0] = __ffma2_rn(cbuw, f2(e, e), bd[0][0]);
-                }
-                if (q.y <= kQMax) {
-                    const float e = ex2_approx(-q.y);
-                    rg[1][0] = __ffma2_rn(crg, f2(e, e), rg[1][0]);
-                    bd[1][0] = __ffma2_rn(cbuw, f2(e, e), bd[1][0]);
-                }
-                continue;
-            }
-            const float2 P = __ffma2_rn(ox, __ffma2_rn(ox, f2(t.w, t.w), f2(t.z, t.z)), f2(t.y, t.y));
-            const float rys[2] = {fmaf(qs, oy0, t.x), fmaf(qs, oy1, t.x)};
+    for (; base < end; base += BATCH * S, buf ^= 1) {
+        {
+            const float4 a = na, b = nb;
+            const float gx = (float)x_org + 0.5f - a.x, gy = (float)y_org + 0.5f - a.y;
+            st.g[buf][me][0] = make_float4(a.z, a.w, fmaf(a.z, gy, a.w * gx), b.x);
+            st.g[buf][me][1] = make_float4(b.x * gx * gx, 2.0f * b.x * gx, b.z, b.w);
+            *reinterpret_cast<float2*>(&st.g[buf][me][2]) = f2(ncb, b.y);
+            const unsigned hit = base + me < end ? regions_hit<RX, F::RY>(a, b.x, gx, gy) : 0u;
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const float2 rr = __ffma2_rn(f2(qw, qw), ox, f2(rys[r], rys[r]));
+            for (int k = 0; k < NR; ++k) {
+                const unsigned bal = __ballot_sync(0xffffffffu, (hit >> k) & 1u);
+                if (lane == 0) st.hits[buf][k][w] = bal;
+            }
+        }
+        fetch(base + BATCH * S);
+        // The batch is staged, and every warp has walked the one before: the buffer written next is free
+        group_sync();
+        // the region's Gaussians by turns to the four quarter warps; the last round is filled with the entry
+        // that lies outside
+        int n = 0;
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            const unsigned bal = st.hits[buf][w][k];
+            const int pos = n + __popc(bal & ((1u << lane) - 1u));
+            if ((bal >> lane) & 1u) st.list[w][pos & 3][pos >> 2] = (unsigned short)((32 * k + lane) * 48);
+            n += __popc(bal);
+        }
+        if (lane < 3) st.list[w][(n + lane) & 3][(n + lane) >> 2] = (unsigned short)(BATCH * 48);
+        __syncwarp();
+        const char* const gbase = reinterpret_cast<const char*>(st.g[buf]);
+        const unsigned short* const lk = st.list[w][quarter];
+        const int nj = (n + 3) >> 2;
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
+            const float4* g = reinterpret_cast<const float4*>(gbase + lk[j]);
+            const float4 u = g[0], t = g[1];
+            const float2 cbuw = *reinterpret_cast<const float2*>(g + 2);
+            const float2 crg = f2(t.z, t.w);
+            // q' = r^2 + qd dx^2 with dx = g_x + o_x: qd dx^2 = qd g_x^2 + o_x (2 qd g_x + o_x qd) and
+            // r = r_0 + qs o_y + qw o_x from the values at the tile's first pixel centre (8-wide tiles
+            // add the two products the other way round)
+            const float2 P = __ffma2_rn(ox, __ffma2_rn(ox, f2(u.w, u.w), f2(t.y, t.y)), f2(t.x, t.x));
+            const float2 rx = __ffma2_rn(f2(u.y, u.y), ox, f2(u.z, u.z));       // TW == 8 only
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float oy = oy0 + (float)r;
+                float2 rr;
+                if constexpr (TW == 8) {
+                    rr = __ffma2_rn(f2(u.x, u.x), f2(oy, oy), rx);
+                } else {
+                    const float ry = fmaf(u.x, oy, u.z);
+                    rr = __ffma2_rn(f2(u.y, u.y), ox, f2(ry, ry));
+                }
                 const float2 q = __ffma2_rn(rr, rr, P);
                 if (q.x <= kQMax) {
                     const float e = ex2_approx(-q.x);
@@ -262,25 +305,68 @@ __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restric
                 }
             }
         }
+        __syncwarp();                                   // the list is read: the next batch's may be written
     }
 
-    const float wB = __ldg(wparams + 2);
-    const float cB0 = __ldg(wparams + 3) * wB, cB1 = __ldg(wparams + 4) * wB, cB2 = __ldg(wparams + 5) * wB;
+    // The quarter warps' sums: a lane keeps row `quarter` of its 2x4 pixels (two exchanges, each handing over
+    // half of what is left)
+    const bool up = quarter & 2, odd = quarter & 1;
+    auto pass = [&](float lo, float hi, bool keep_hi, int mask) {
+        const float mine = keep_hi ? hi : lo, give = keep_hi ? lo : hi;
+        return mine + __shfl_xor_sync(0xffffffffu, give, mask);
+    };
+    float4 sum[2];
+    sum[0] = sum[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (start != end)
 #pragma unroll
-    for (int r = 0; r < 2; ++r)
+    for (int c = 0; c < 2; ++c) {
+        float o[4];
 #pragma unroll
-        for (int c = 0; c < PX; ++c) {
-            const int x = x0 + c, y = y0 + r;
-            if (x < V.W && y < V.H) {
-                const long long pix = V.pix_base + (long long)y * V.W + x;
-                const float D = wB + bd[r][c].y;
-                const float inv = 1.0f / D;
-                out_rgb[3 * pix + 0] = (cB0 + rg[r][c].x) * inv;
-                out_rgb[3 * pix + 1] = (cB1 + rg[r][c].y) * inv;
-                out_rgb[3 * pix + 2] = (cB2 + bd[r][c].x) * inv;
-                out_den[pix] = D;
-            }
+        for (int e = 0; e < 4; ++e) {
+            auto val = [&](int r) {
+                const float2 x = e < 2 ? rg[r][c] : bd[r][c];
+                return e & 1 ? x.y : x.x;
+            };
+            o[e] = pass(pass(val(0), val(2), up, 16), pass(val(1), val(3), up, 16), odd, 8);
         }
+        sum[c] = make_float4(o[0], o[1], o[2], o[3]);
+    }
+    const int ly = 8 * (w / RX) + 4 * (o8 >> 2) + quarter, lx = 8 * (w % RX) + 2 * (o8 & 3);
+    if (S > 1 && start != end) {
+        // the slices' sums, added by the first group in their order
+        if (slice > 0) {
+            group_sync();                               // the stage is read: it may hold the sums
+            float4* const px = reinterpret_cast<GroupMem*>(s_mem[slice])->px;
+            px[32 * w + lane] = sum[0];
+            px[32 * w + lane + 32 * NR] = sum[1];
+        }
+        __syncthreads();
+        if (slice > 0) return;                          // (back to the tile loop)
+#pragma unroll
+        for (int k = 1; k < S; ++k)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float4 o = reinterpret_cast<const GroupMem*>(s_mem[k])->px[32 * w + lane + 32 * NR * c];
+                sum[c].x += o.x;
+                sum[c].y += o.y;
+                sum[c].z += o.z;
+                sum[c].w += o.w;
+            }
+    }
+    if (S > 1 && slice > 0) return;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int x = x_org + lx + c, y = y_org + ly;
+        if (x < V.W && y < V.H) {
+            const long long pix = V.pix_base + (long long)y * V.W + x;
+            const float D = wB + sum[c].w;
+            const float inv = 1.0f / D;
+            out_rgb[3 * pix + 0] = (cB0 + sum[c].x) * inv;
+            out_rgb[3 * pix + 1] = (cB1 + sum[c].y) * inv;
+            out_rgb[3 * pix + 2] = (cB2 + sum[c].z) * inv;
+            out_den[pix] = D;
+        }
+    }
 }
 
 // Persistent schedule: blocks take tiles order[0..n) through *counter.
@@ -302,14 +388,14 @@ __device__ __forceinline__ void for_each_tile(const unsigned* __restrict__ order
     }
 }
 
-template <int TW, int TH, int PX>
-__global__ void __launch_bounds__(FwdShape<TW, TH, PX>::NT)
+template <int TW, int TH, int S>
+__global__ void __launch_bounds__(32 * S * FwdShape<TW, TH>::NR, kFwdWarpsPerSM / (S * FwdShape<TW, TH>::NR))
     k_render_fwd(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
                  const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
                  float* __restrict__ out_rgb, float* __restrict__ out_den, const unsigned* __restrict__ order,
                  unsigned* __restrict__ counter) {
     for_each_tile(order, counter, vs.total_tiles, [&](int tile) {
-        fwd_tile<TW, TH, PX>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den);
+        fwd_tile<TW, TH, S>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den);
     });
 }
 
@@ -701,35 +787,40 @@ __global__ void __launch_bounds__(256) k_det_bg_reduce(const float* __restrict__
 }
 
 // Grid of a launch: one block per tile, or, persistent, as many blocks as
-// fit on the device at once, up to max_warps_per_sm warps per SM.
+// fit on the device at once.
 template <typename K>
-unsigned grid_for(K kernel, int threads, const Views& vs, const Sched& sched, int max_warps_per_sm = 64) {
+unsigned grid_for(K kernel, int threads, const Views& vs, const Sched& sched) {
     if (!sched.order) return (unsigned)vs.total_tiles;
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
-    per_sm = min(per_sm, max(1, max_warps_per_sm * 32 / threads));
     return (unsigned)min(max(1, sms * max(per_sm, 1)), vs.total_tiles);
 }
 
-// The forward's persistent grid holds 16 warps per SM (8 blocks of 16x16 tiles), not the 28 that its
-// registers allow: at 1M Gaussians and 1920x1080 it ran in 0.49 ms at 16 warps against 0.51 at 12,
-// 0.55 at 20 and 0.58 at 28.
-constexpr int kFwdWarpsPerSM = 16;
+constexpr int kFwdSliceTiles = 608;     // four per SM
 
-template <int TW, int TH, int PX>
-cudaError_t fwd_t(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
+template <int TW, int TH, int S>
+cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
-    constexpr int NT = FwdShape<TW, TH, PX>::NT;
-    const unsigned grid = grid_for(k_render_fwd<TW, TH, PX>, NT, vs, sched, kFwdWarpsPerSM);
+    constexpr int NT = 32 * S * FwdShape<TW, TH>::NR;
+    const unsigned grid = grid_for(k_render_fwd<TW, TH, S>, NT, vs, sched);
     if (sched.order) {
         cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
     }
-    k_render_fwd<TW, TH, PX><<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb,
-                                                 den, sched.order, sched.counter);
+    k_render_fwd<TW, TH, S><<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb, den,
+                                                sched.order, sched.counter);
     return cudaGetLastError();
+}
+
+template <int TW, int TH>
+cudaError_t fwd_t(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
+                  float* rgb, float* den, Sched sched, cudaStream_t s) {
+    // Two slices where the tiles alone leave the SMs idle: 14.4 -> 10.4 us at 240 tiles, 14.5 -> 13.7 at 475
+    // (40k Gaussians), 14.4 -> 15.1 at 920, 39 -> 70 at 8160.
+    return vs.total_tiles <= kFwdSliceTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
+                                            : fwd_s<TW, TH, 1>(rec, off, list, vs, w, rgb, den, sched, s);
 }
 
 template <int TW, int TH, int CH>
@@ -762,21 +853,23 @@ cudaError_t bwd_t(const float* rec, const unsigned* off, const unsigned* list, c
 //   [0] (pixel, Gaussian) pairs inside the cutoff, i.e. the algorithmic work
 //       (q' from each pixel's own dx, dy; the renderers may decide pairs
 //       within rounding of the cutoff differently);
-//   [1] the (pixel, Gaussian) slots the forward evaluates: for every Gaussian
-//       of a tile, the pixels of each warp whose region its footprint reaches
-//       (the forward's per-warp test; all the tile's pixel slots with one warp);
+//   [1] the (pixel, Gaussian) slots the forward evaluates: per batch of a
+//       tile's list and 8x8 region, rounds of four Gaussians that reach the
+//       region (its own test), 256 slots each; 64 per Gaussian in 8x8 tiles;
 //   [2] the backward's pixel slots (per tile instance, the rows from the first
 //       to the last with a span, TW columns each, or TW / 2 when no span is
 //       longer than TW / 2 pixels), from the backward's own span arithmetic.
-template <int TW, int TH, int PPT, int PX>
+template <int TW, int TH, int PPT>
 __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
     k_count_pairs(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
                   const unsigned* __restrict__ list, const Views vs, unsigned long long* __restrict__ count) {
     using S = TileShape<TW, TH, PPT>;
-    using F = FwdShape<TW, TH, PX>;
     constexpr int NT = S::NT;
+    using F = FwdShape<TW, TH>;
+    static_assert(NT == 32 * F::NR, "the forward's batches");
     __shared__ float4 s0[NT];
     __shared__ float s1[NT];
+    __shared__ unsigned s_n[F::NR];
     const int tile = blockIdx.x;
     const TileCoord tc = tile_coord(vs, tile);
     const View& V = vs.v[tc.v];
@@ -793,24 +886,15 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
     for (unsigned base = start; base < end; base += NT) {
         const int cnt = (int)min((unsigned)NT, end - base);
         __syncthreads();
+        unsigned hit = 0u;
+        if (tid < F::NR) s_n[tid] = 0u;
         if (tid < cnt) {
             const float4* p = rec + 3ull * list[base + tid];
             const float4 a = __ldg(p);
             const float qd = __ldg(reinterpret_cast<const float*>(p + 1));
             s0[tid] = a;
             s1[tid] = qd;
-            // the forward's slots: 32 threads x PX x 2 pixels per warp whose rows the footprint reaches
-            if constexpr (F::NW > 1) {
-                const float xl = (float)x_org + 0.5f, xh = xl + (float)(TW - 1);
-#pragma unroll
-                for (int w = 0; w < F::NW; ++w) {
-                    const float yl = (float)(y_org + F::row_lo(w)) + 0.5f;
-                    const float yh = (float)(y_org + F::row_hi(w)) + 0.5f;
-                    if (footprint_hits(a.x, a.y, a.z, a.w, qd, xl, xh, yl, yh)) cnt_fwd += 32ull * PX * 2;
-                }
-            } else {
-                cnt_fwd += (unsigned long long)F::NT * PX * 2;
-            }
+            hit = regions_hit<F::RX, F::RY>(a, qd, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y);
             // the backward's pixel slots: the rows from its first span to its last, TW columns each, or
             // TW / 2 when no span is longer than TW / 2 pixels
             const RowSpans rs(a, qd, QM);
@@ -827,6 +911,14 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
             if (r_hi >= r_lo) cnt_bwd += (unsigned long long)(r_hi - r_lo + 1) * (2 * umax > TW / 2 ? TW : TW / 2);
         }
         __syncthreads();
+#pragma unroll
+        for (int k = 0; k < F::NR; ++k) {
+            const unsigned bal = __ballot_sync(0xffffffffu, (hit >> k) & 1u);
+            if ((tid & 31) == 0 && bal) atomicAdd(&s_n[k], (unsigned)__popc(bal));
+        }
+        __syncthreads();
+        // the forward's rounds over this batch: 256 slots each (one region per tile: 64 per Gaussian)
+        if (tid < F::NR) cnt_fwd += F::NR > 1 ? 256ull * ((s_n[tid] + 3u) >> 2) : 64ull * s_n[tid];
         if (x >= V.W) continue;
         for (int j = 0; j < cnt; ++j) {
             const float4 a = s0[j];
@@ -893,10 +985,10 @@ __global__ void __launch_bounds__(256) k_loss_l1(const float* __restrict__ rgb, 
 cudaError_t launch_render_fwd(const float* rec, const unsigned* off, const unsigned* list, const Views& vs,
                               WeightDev w, float* rgb, float* den, Sched sc, cudaStream_t s) {
     if (vs.total_tiles == 0) return cudaSuccess;
-    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16, 2>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8, 1>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8, 2>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8, 2>(rec, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16>(rec, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8>(rec, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8>(rec, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8>(rec, off, list, vs, w, rgb, den, sc, s);
     return cudaErrorInvalidValue;
 }
 
@@ -939,11 +1031,10 @@ cudaError_t launch_count_pairs(const float* rec, const unsigned* off, const unsi
     cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(unsigned long long), s);
     if (e != cudaSuccess || vs.total_tiles == 0) return e;
     const float4* r = reinterpret_cast<const float4*>(rec);
-    // the forward's pixels per thread (PX) as launch_render_fwd picks them
-    if (vs.tile_w == 16 && vs.tile_h == 16) k_count_pairs<16, 16, 2, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 8 && vs.tile_h == 8) k_count_pairs<8, 8, 2, 1><<<vs.total_tiles, 32, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 32 && vs.tile_h == 8) k_count_pairs<32, 8, 2, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 16 && vs.tile_h == 8) k_count_pairs<16, 8, 2, 2><<<vs.total_tiles, 64, 0, s>>>(r, off, list, vs, count);
+    if (vs.tile_w == 16 && vs.tile_h == 16) k_count_pairs<16, 16, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
+    else if (vs.tile_w == 8 && vs.tile_h == 8) k_count_pairs<8, 8, 2><<<vs.total_tiles, 32, 0, s>>>(r, off, list, vs, count);
+    else if (vs.tile_w == 32 && vs.tile_h == 8) k_count_pairs<32, 8, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
+    else if (vs.tile_w == 16 && vs.tile_h == 8) k_count_pairs<16, 8, 2><<<vs.total_tiles, 64, 0, s>>>(r, off, list, vs, count);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
