@@ -460,9 +460,8 @@ wsr_status wsr_bin_static(const float* records, int64_t n, const wsr_camera* cam
  *       slots per round of four (of each batch of the tile's list), the last
  *       round's idle quarters included; 64 per Gaussian in 8x8 tiles;
  *   [2] (pixel, Gaussian) slots wsr_render_bwd evaluates: for each Gaussian
- *       of a tile, the rows from its first span to its last, each of tile
- *       width columns, or of half the tile width when none of its row spans
- *       is longer than that.
+ *       of a tile, the rows that its footprint reaches, each of tile width
+ *       columns, or of half the tile width when no row needs more.
  * Arguments as for wsr_render_fwd.  Not part of a timed step.
  */
 wsr_status wsr_count_pairs(const float* records, int64_t n, const uint32_t* tile_offsets,

@@ -49,64 +49,44 @@ struct Lanes {
     static constexpr int value = N;
 };
 
-// The backward's pixel spans of one record on the rows of a tile: on row y the
-// footprint q' <= QM is mu_x + c(dy) +- h(dy) with the conic entries
-// A' = qw^2 + qd, B' = qs qw, C' = qs^2, det' = A' C' - B'^2 = qd qs^2:
-// c = -B' dy / A', h = sqrt(A' QM - det' dy^2) / A' (no cancellation anywhere),
-// widened by 0.02 pixel.  `row` gives the span of a local row as
-// (first column, rounded down to even) | (column pairs << 8): the pairs from
-// that even column that hold the span (a padding pixel at either end lies
-// outside the footprint or in the tile's zero column).
-struct RowSpans {
-    float Ap, hb, det, ia, ext, apqm, hbia;
-    __device__ __forceinline__ RowSpans(const float4 a, const float qd, const float QM) {
-        Ap = fmaf(a.w, a.w, qd);
-        hb = a.z * a.w;
-        det = qd * a.z * a.z;
-        ia = rcp_approx(Ap);
-        apqm = Ap * QM;
-        hbia = hb * ia;
-        // rows the footprint can reach: |dy| <= sqrt(A' QM / det'), with a pixel of slack
-        ext = fminf(sqrt_approx(fmaxf(Ap * QM * rcp_approx(det), 0.0f)), 1e6f) + 1.0f;
+// The part of a footprint q' <= QM inside a tile, as the backward walks it.  On row dy the footprint is
+// dx = -(B'/A') dy +- sqrt(QM / A' - (det'/A'^2) dy^2) with A' = qw^2 + qd, B' = qs qw, det' = qd qs^2 (no
+// cancellation); on column dx it is dy = (-qw dx +- sqrt(QM - qd dx^2)) / qs.  `rows` gives the tile's rows that
+// it can reach between the tile's first and last columns (from the second form, at the columns of the tile
+// nearest its highest and lowest points) and whether a row can need more than half the tile's width.  Both
+// are widened far beyond their rounding; NaN widens them to the whole tile.
+struct Footprint {
+    float h0, h1, slope;                // half-width^2 = h0 - h1 dy^2, centre = -slope dy
+    __device__ __forceinline__ Footprint(const float4 a, const float qd) {
+        const float QM = kQMax * 1.0001f + 1e-4f;
+        const float ia = rcp_approx(fmaf(a.w, a.w, qd));
+        slope = a.z * a.w * ia;
+        h0 = QM * ia;
+        h1 = qd * a.z * a.z * ia * ia;
     }
-    // local rows [lo, hi] of the block [first, first + count) that the footprint can reach
-    __device__ __forceinline__ void rows(const float4 a, int y_org, int first, int count, int& lo, int& hi) const {
-        lo = max(first, (int)floorf(a.y - ext - 0.5f) - y_org);
-        hi = min(first + count - 1, (int)ceilf(a.y + ext - 0.5f) - y_org);
-    }
-    __device__ __forceinline__ unsigned short row(const float4 a, const float QM, int x_org, int y_org, int x_lim,
-                                                  int ly) const {
-        const float dy = (float)(y_org + ly) + 0.5f - a.y;
-        const float d4 = fmaf(-det * dy, dy, Ap * QM);
-        if (d4 < 0.0f) return 0;
-        const float h = sqrt_approx(d4) * ia;
-        const float cx = a.x - hb * dy * ia;
-        const float fx0 = fmaxf(ceilf(cx - h - 0.52f), (float)x_org);
-        const float fx1 = fminf(floorf(cx + h - 0.48f), (float)(x_org + x_lim - 1));
-        if (!(fx0 <= fx1)) return 0;
-        const int xs = (int)fx0 - x_org, len = (int)fx1 - (int)fx0 + 1, xe = xs & ~1;
-        return (unsigned short)(xe | (((xs - xe + len + 1) >> 1) << 8));    // even start, column pairs
-    }
-    // the spans of local rows ly and ly + 1 (low and high half), two rows per paired FP32 op
-    __device__ __forceinline__ unsigned row2(const float4 a, int x_org, int y_org, int x_lim, int ly) const {
-        const float dy0 = (float)(y_org + ly) + 0.5f - a.y;
-        const float2 dy = f2(dy0, dy0 + 1.0f);
-        const float2 d4 = __ffma2_rn(__fmul2_rn(f2(-det, -det), dy), dy, f2(apqm, apqm));
-        const float2 h = __fmul2_rn(f2(sqrt_approx(fmaxf(d4.x, 0.0f)), sqrt_approx(fmaxf(d4.y, 0.0f))), f2(ia, ia));
-        const float2 cx = __ffma2_rn(f2(-hbia, -hbia), dy, f2(a.x, a.x));
-        const float2 l = __fadd2_rn(__ffma2_rn(h, f2(-1.0f, -1.0f), cx), f2(-0.52f, -0.52f));
-        const float2 r = __fadd2_rn(__fadd2_rn(cx, h), f2(-0.48f, -0.48f));
-        const float xlo = (float)x_org, xhi = (float)(x_org + x_lim - 1);
-        unsigned out = 0;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float fx0 = fmaxf(ceilf(k ? l.y : l.x), xlo), fx1 = fminf(floorf(k ? r.y : r.x), xhi);
-            if ((k ? d4.y : d4.x) >= 0.0f && fx0 <= fx1) {
-                const int xs = (int)fx0 - x_org, len = (int)fx1 - (int)fx0 + 1, xe = xs & ~1;
-                out |= (unsigned)(xe | (((xs - xe + len + 1) >> 1) << 8)) << (16 * k);
-            }
-        }
-        return out;
+    // (gx, gy): the tile's first pixel centre less the mean; x_lim, y_lim: its pixels inside the image
+    template <int TW>
+    __device__ __forceinline__ void rows(const float4 a, const float qd, const float gx, const float gy, const int x_lim,
+                                         const int y_lim, int& first, int& count, bool& wide) const {
+        const float QM = kQMax * 1.0001f + 1e-4f;
+        const float iqs = rcp_approx(a.z), xm = sqrt_approx(QM * rcp_approx(qd));       // half-width of the box
+        const float xt = -a.w * xm * sqrt_approx(rcp_approx(fmaf(a.w, a.w, qd)));       // dx of the highest point
+        const float xl = gx, xr = gx + (float)(x_lim - 1);
+        const float x1 = fminf(fmaxf(xt, xl), xr), x0 = fminf(fmaxf(-xt, xl), xr);
+        const float y1 = fmaf(-a.w, x1, sqrt_approx(fmaxf(fmaf(-qd * x1, x1, QM), 0.0f))) * iqs;
+        const float y0 = fmaf(-a.w, x0, -sqrt_approx(fmaxf(fmaf(-qd * x0, x0, QM), 0.0f))) * iqs;
+        const float margin = fmaf(1e-3f, fabsf(y1) + fabsf(y0), 0.02f);
+        int lo = 0, hi = y_lim - 1;
+        if (y0 - margin - gy > 0.0f) lo = (int)fminf(ceilf(y0 - margin - gy), 64.0f);
+        if (y1 + margin - gy < (float)hi) hi = (int)fmaxf(floorf(y1 + margin - gy), -1.0f);
+        first = min(lo, y_lim - 1);
+        count = max(hi - lo + 1, 0);
+        // narrow: the widest row has at most TW / 2 - 1 pixel centres (one more may go before an even first
+        // column), or the whole box lies in one half of the tile
+        const float yc = fminf(fmaxf(0.0f, gy + (float)lo), gy + (float)hi);
+        const float h = sqrt_approx(fmaxf(fmaf(-h1 * yc, yc, h0), 0.0f));
+        wide = !(2.0f * h < (float)(TW / 2 - 1) - 0.1f || xm < gx + (float)(TW / 2) - 0.1f ||
+                 -xm > gx + (float)(TW / 2 - 1) + 0.1f);
     }
 };
 
@@ -411,14 +391,11 @@ __device__ __forceinline__ float warp_sum(float v) {
 // pairs, two float4 planes (x0, x1, y0, y1) and (z0, z1, w0, w1), with zero
 // pairs past the tile's right edge as far as a lane reads.  For each chunk of
 // CH Gaussians of the tile:
-//   A. two threads per Gaussian compute, for their half of the tile's rows
-//      (two rows per paired op), the span of pixels whose centre can lie
-//      inside the footprint (the roots of q(dx) = 9 on each row, widened
-//      slightly), kept as its first column rounded down to even and a number
-//      of column pairs, and the first and last rows with a span, and take
-//      the Gaussian's rank in its bucket of the sort below;
-//   B. the chunk's Gaussians are ordered wide ones first (a row span longer
-//      than TW / 2 pixels), each class by its number of rows, longest first
+//   A. a thread per Gaussian finds the rows of the tile that its footprint
+//      reaches and whether a row may need more than TW / 2 pixels (closed
+//      forms, Footprint), and takes its rank in its bucket of the sort below;
+//   B. the chunk's Gaussians are ordered wide ones first (more than TW / 2
+//      pixels on a row), each class by its number of rows, longest first
 //      (a counting sort: the buckets' starts from one warp suffix scan); each
 //      warp takes the next Gaussians of a class whenever it is free (a shared
 //      counter per class), so that the groups of a warp walk for the same
@@ -427,10 +404,11 @@ __device__ __forceinline__ float warp_sum(float v) {
 //      its rows one per step, L = TW / (2 M) for the wide class and TW / (4 M)
 //      for the narrow one (whose spans all fit in 2 M L columns), M = 4 column
 //      pairs per lane and row (2 for 8-pixel-wide tiles); lane k takes column
-//      pairs start / 2 + k + m L (m < M) of the row, so the lanes of a group
-//      read consecutive entries of each plane, 2 M pixels per step from one
-//      decode of the row's span, every quantity of a column pair in one
-//      paired FP32 op.  The nine record terms stay in registers until
+//      pairs start / 2 + k + m L (m < M) of the row, start being the first
+//      column the footprint can reach there, rounded down to even, so the
+//      lanes of a group read consecutive entries of each plane, 2 M pixels
+//      per step from one start, every quantity of a column pair in one paired
+//      FP32 op.  The nine record terms stay in registers until
 //      the Gaussian's last row; then log2(L) shuffle steps sum them over the
 //      group and its first lane adds them to the Gaussian's global record (in
 //      the deterministic mode: as fixed point, in units that a per-Gaussian
@@ -443,25 +421,32 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Gaussian's peak there) may be counted by one and not the other.
 // Gaussians per chunk: CH, a template parameter (64, 128, 256 or 512); threads
 // per block: BwdThreads<CH> (2 CH up to 256).
-template <int TW, int TH, int CH>
+//   It is bound by the shared-memory data path (76% busy: two 16-byte loads per
+// column pair and lane, a quarter of the wavefronts bank conflicts) and the FP32
+// pipe (63%).  1M Gaussians at 1920x1080, 512 per chunk, persistent: 1008 us and
+// 7.9e8 warp instructions when step A found every row's span (two threads per
+// Gaussian, a table of spans in shared memory), 931 us and 6.7e8 with the rows in
+// closed form and a row's start formed as it is walked; three blocks per SM at 80
+// registers, without spills, took 960 us.
+constexpr float kMagic = 12582912.0f;       // 1.5 x 2^23
+
+template <int TW, int TH, int CH, bool DET>
 __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restrict__ rec,
                                          const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
                                          const Views& vs, const float* __restrict__ wparams,
                                          const float* __restrict__ out_rgb, const float* __restrict__ out_den,
                                          const float* __restrict__ grad_rgb, float* __restrict__ grec,
-                                         float* __restrict__ gw, const int pass, float* __restrict__ bg_tiles,
+                                         float* __restrict__ gw, float* __restrict__ bg_tiles,
                                          const unsigned* __restrict__ det_pmax) {
     constexpr int NT = BwdThreads<CH>::value;
     constexpr int NW = NT / 32;
-    constexpr int PASSES = 2 * CH / NT;                // step A: (Gaussian, half) items per thread
     // pixel-table row pitch in column pairs: the row's TW / 2 pairs, then zero pairs up to the farthest pair a
     // lane reads (start / 2 + k + m L <= (TW / 2 - 1) + (TW / 2 - 1)), so no index needs a clamp; odd, so that
     // the rows start in different banks
     constexpr int PP = TW - 1;
-    constexpr int HR = TH / 2;                          // rows per thread in step A
     constexpr int NB = TH + 1;                          // row counts 0 .. TH
     constexpr int NK = 2 * NB;                          // sort keys: narrow 0 .. TH, wide NB .. NB + TH
-    static_assert(PASSES * NT == 2 * CH && TH % 4 == 0 && TW % 8 == 0 && TW <= 64 && CH <= 512 && NK <= NT, "layout");
+    static_assert(CH % 32 == 0 && TW % 8 == 0 && TW <= 64 && CH <= 512 && NK <= NT, "layout");
     constexpr int M = TW >= 16 ? 4 : 2;                 // column pairs per lane and row in step C
     // per pixel: G/D (3), -(G.C)/D, stored per column pair as (x0, x1, y0, y1) and (z0, z1, w0, w1)
     __shared__ float4 spA[PP * TH];
@@ -470,9 +455,8 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     __shared__ float4 s1[CH];                   // qd, u w, c_r u w, c_g u w
     __shared__ float2 s2[CH];                   // c_b u w, u w
     __shared__ unsigned sidx[CH];
-    __shared__ unsigned short sspan[CH][TH];    // per row: even first column | column pairs << 8
-    __shared__ unsigned char sfirst[CH];        // first row with a span
-    __shared__ unsigned char snst[CH];          // rows from there to the last row with a span
+    __shared__ unsigned char sfirst[CH];        // first row of the tile that the footprint reaches
+    __shared__ unsigned char snst[CH];          // rows from there to the last one
     __shared__ unsigned char skey[CH];          // sort key: rows, plus NB when wide
     __shared__ unsigned short srank[CH];        // rank among the chunk's Gaussians of the same key
     __shared__ unsigned short sord[CH];         // the chunk's Gaussians: wide ones first, most rows first
@@ -488,7 +472,7 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     const int y_lim = min(TH, V.H - y_org);
     const float wB = __ldg(wparams + 2);
     const float cB0 = __ldg(wparams + 3), cB1 = __ldg(wparams + 4), cB2 = __ldg(wparams + 5);
-    const float pmax = pass != 0 ? __int_as_float(*det_pmax) : 0.0f;    // deterministic mode
+    const float pmax = DET ? __int_as_float(*det_pmax) : 0.0f;    // deterministic mode
 
     float bg[4] = {0.f, 0.f, 0.f, 0.f};
     for (int p = tid; p < 2 * PP * TH; p += NT) {
@@ -518,56 +502,32 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
         if (lane == 0) sbg[c][warp] = t;
     }
 
-    const float QM = kQMax * 1.0001f + 1e-4f;
     const unsigned start = offsets[tile], end = offsets[tile + 1];
     if (tid < NK) shist[tid] = 0u;
     for (unsigned base = start; base < end; base += CH) {
         const int cnt = (int)min((unsigned)CH, end - base);
         __syncthreads();                                // the previous chunk is done with shared memory
-        // ---- A: record, spans of half the rows of a Gaussian per item, first and last rows ----
+        // ---- A: record, rows and class of a Gaussian per thread ----
 #pragma unroll 1
-        for (int ps = 0; ps < PASSES; ++ps) {
-            const int u = tid + ps * NT;
-            const int gj = u >> 1, half = u & 1;
-            unsigned rows = 0u;                         // bit ly: row ly has a span
-            unsigned umax = 0u;                         // the most column pairs of a row's span
-            if (gj < cnt) {
-                const unsigned r = list[base + gj];
-                const float4* pr = rec + 3ull * r;
-                const float4 a = __ldg(pr);
-                const float4 b = __ldg(pr + 1);
-                if (half == 0) {
-                    const float cb = __ldg(reinterpret_cast<const float*>(pr + 2));
-                    s0[gj] = a;
-                    s1[gj] = b;
-                    s2[gj] = f2(cb, b.y);
-                    sidx[gj] = r;
-                }
-                const RowSpans rs(a, b.x, QM);
-#pragma unroll
-                for (int k = 0; k < HR; k += 2) {
-                    const int ly = half * HR + k;
-                    // rows the footprint does not reach have no span (no root: the square root's argument is
-                    // negative); rows past the image's last have none either
-                    unsigned sp2 = rs.row2(a, x_org, y_org, x_lim, ly);
-                    if (ly + 1 >= y_lim) sp2 = ly < y_lim ? sp2 & 0x0000ffffu : 0u;
-                    *reinterpret_cast<unsigned*>(&sspan[gj][ly]) = sp2;
-                    rows |= ((sp2 & 0x0000ff00u) ? 1u : 0u) << ly;
-                    rows |= ((sp2 & 0xff000000u) ? 2u : 0u) << ly;
-                    umax = max(umax, max((sp2 >> 8) & 0xffu, sp2 >> 24));
-                }
-            }
-            rows |= __shfl_xor_sync(0xffffffffu, rows, 1);           // the two halves of a Gaussian
-            umax = max(umax, __shfl_xor_sync(0xffffffffu, umax, 1));
-            const int row_lo = rows ? __ffs((int)rows) - 1 : TH, row_hi = rows ? 31 - __clz((int)rows) : -1;
-            if (gj < cnt && half == 0) {
-                const int nst = row_hi >= row_lo ? row_hi - row_lo + 1 : 0;
-                const int key = nst + (2 * (int)umax > TW / 2 ? NB : 0);    // wide: a span longer than TW / 2 pixels
-                sfirst[gj] = (unsigned char)max(row_lo, 0);
-                snst[gj] = (unsigned char)nst;
-                skey[gj] = (unsigned char)key;
-                srank[gj] = (unsigned short)atomicAdd(&shist[key], 1u);
-            }
+        for (int gj = tid; gj < cnt; gj += NT) {
+            const unsigned r = list[base + gj];
+            const float4* pr = rec + 3ull * r;
+            const float4 a = __ldg(pr);
+            const float4 b = __ldg(pr + 1);
+            const float cb = __ldg(reinterpret_cast<const float*>(pr + 2));
+            s0[gj] = a;
+            s1[gj] = b;
+            s2[gj] = f2(cb, b.y);
+            sidx[gj] = r;
+            int first, nst;
+            bool wide;
+            Footprint(a, b.x).rows<TW>(a, b.x, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y, x_lim, y_lim,
+                                       first, nst, wide);
+            const int key = nst + (wide ? NB : 0);
+            sfirst[gj] = (unsigned char)first;
+            snst[gj] = (unsigned char)nst;
+            skey[gj] = (unsigned char)key;
+            srank[gj] = (unsigned short)atomicAdd(&shist[key], 1u);
         }
         if (tid < 2) snext[tid] = 0u;
         __syncthreads();
@@ -629,23 +589,26 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
                 // footprint's small along-axis terms (dx) are not rounded away under its large r terms.
                 float2 gr = f2(0.f, 0.f), gg = gr, gb = gr, gu = gr;
                 float2 srr = f2(0.f, 0.f), srx = srr, sxx = srr, sr = srr, sx = srr;
-                // dx of this lane's two column pairs (2 (k + m L), +1) from the row's even first column, less
-                // that column
+                // dx of this lane's first column pair (2 k, 2 k + 1) from the row's even first column, less that column
                 const float2 gxb = __fadd2_rn(f2((float)(2 * gk), (float)(2 * gk + 1)), gx2);
-                for (int st = 0; st < steps; ++st) {
-                    const int ly = r0 + st;
-                    const unsigned sp = sspan[j][ly];
-                    const int xe = (int)(sp & 0xffu);                           // even first column
-                    const int pb = ly * PP + (xe >> 1) + gk;
-                    const float xsf = (float)xe;
-                    const float rb = qs * ((float)ly + gy0);                     // qs dy
+                const Footprint fp(a, b.x);
+                const float left = -gx0 - 0.025f;                               // columns, with a little slack
+                int row = r0 * PP + gk - __float_as_int(kMagic);
+                const float yend = (float)(r0 + steps);
+                for (float yf = (float)r0; yf < yend; row += PP, yf += 1.0f) {
+                    const float dy = yf + gy0, rb = qs * dy;
+                    // the row's first column v (not beyond the last pair), rounded up and then down to even:
+                    // round(v / 2), by adding a number whose last bit weighs one
+                    const float v = fmaf(-fp.slope, dy, left) - sqrt_approx(fmaxf(fmaf(-fp.h1 * dy, dy, fp.h0), 0.0f));
+                    const float w = fmaf(fminf(fmaxf(v, 0.0f), (float)(TW - 2)), 0.5f, kMagic);
+                    const int pb = row + __float_as_int(w);
+                    const float xsf = fmaf(w, 2.0f, -2.0f * kMagic);
                     const float2 xb = __fadd2_rn(f2(xsf, xsf), gxb);             // dx of the lane's first pair
                     const float2 rb2 = f2(rb, rb);
 #pragma unroll
                     for (int m = 0; m < M; ++m) {
-                        // Columns outside the span evaluate q > 9 (the span holds every pixel centre of the row
-                        // with q' <= kQMax, with a margin), so the cutoff test zeroes them; pairs past the tile
-                        // read zero pairs.  No per-pixel validity mask is needed.
+                        // Columns outside the footprint evaluate q > 9, so the cutoff test zeroes them; pairs past
+                        // the tile and rows past the image read zero pairs.  No per-pixel mask is needed.
                         const int pi = pb + m * L;
                         const float4 A = spA[pi], B = spB[pi];          // (x0, x1, y0, y1), (z0, z1, w0, w1)
                         const float2 dx = m == 0 ? xb : __fadd2_rn(xb, f2((float)(2 * m * L), (float)(2 * m * L)));
@@ -681,7 +644,7 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
 #pragma unroll
                     for (int c = 0; c < 9; ++c) vals[c] += __shfl_xor_sync(0xffffffffu, vals[c], off);
                 if (act && gk == 0 && steps > 0) {
-                    if (pass == 0) {
+                    if constexpr (!DET) {
                         float4* o = reinterpret_cast<float4*>(grec + (size_t)WSR_GRAD_RECORD_FLOATS * sidx[j]);
                         atomicAdd(o, make_float4(vals[0], vals[1], vals[2], vals[3]));
                         atomicAdd(o + 1, make_float4(vals[4], vals[5], vals[6], vals[7]));
@@ -694,6 +657,7 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
                         // pixel-table entry at most pmax, |r| <= sqrt(QM), |dx| <= hx inside the cutoff.
                         float* o = grec + (size_t)kDetRecordFloats * sidx[j];
                         int* mag = reinterpret_cast<int*>(o + 18);
+                        constexpr float QM = kQMax * 1.0001f + 1e-4f;
                         const float qd = b.x, hx = sqrtf(QM / qd);
                         const float hy = sqrtf(QM * fmaf(a.w, a.w, qd) / (qd * a.z * a.z));
                         const float npx = fminf((2.0f * hx + 2.0f) * (2.0f * hy + 2.0f), 1e12f);
@@ -724,7 +688,7 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     if (tid < 4) {
         float t = 0.0f;
         for (int w = 0; w < NW; ++w) t += sbg[tid][w];
-        if (pass == 0) {
+        if constexpr (!DET) {
             if (t != 0.0f) atomicAdd(gw + 2 + tid, t);
         } else {
             bg_tiles[4 * (size_t)tile + tid] = t;      // summed in tile order afterwards
@@ -732,18 +696,18 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     }
 }
 
-template <int TW, int TH, int CH>
+template <int TW, int TH, int CH, bool DET>
 __global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::value)
     k_render_bwd(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
                  const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
                  const float* __restrict__ out_rgb, const float* __restrict__ out_den,
                  const float* __restrict__ grad_rgb, float* __restrict__ grec, float* __restrict__ gw,
-                 const int pass, float* __restrict__ bg_tiles, const unsigned* __restrict__ det_pmax,
+                 float* __restrict__ bg_tiles, const unsigned* __restrict__ det_pmax,
                  const unsigned* __restrict__ order,
                  unsigned* __restrict__ counter) {
     for_each_tile(order, counter, vs.total_tiles, [&](int tile) {
-        bwd_tile<TW, TH, CH>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den, grad_rgb, grec, gw, pass,
-                             bg_tiles, det_pmax);
+        bwd_tile<TW, TH, CH, DET>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den, grad_rgb, grec, gw,
+                                  bg_tiles, det_pmax);
     });
 }
 
@@ -828,13 +792,14 @@ cudaError_t bwd_chunk(const float* rec, const unsigned* off, const unsigned* lis
                       const float* rgb, const float* den, const float* grgb, float* grec, float* gw, int pass,
                       float* bg_tiles, const unsigned* det_pmax, Sched sched, cudaStream_t s) {
     constexpr int NT = BwdThreads<CH>::value;
-    const unsigned grid = grid_for(k_render_bwd<TW, TH, CH>, NT, vs, sched);
+    auto kernel = pass == 0 ? k_render_bwd<TW, TH, CH, false> : k_render_bwd<TW, TH, CH, true>;
+    const unsigned grid = grid_for(kernel, NT, vs, sched);
     if (sched.order) {
         cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
     }
-    k_render_bwd<TW, TH, CH><<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params,
-                                                     rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax,
+    kernel<<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params,
+                                                     rgb, den, grgb, grec, gw, bg_tiles, det_pmax,
                                                      sched.order, sched.counter);
     return cudaGetLastError();
 }
@@ -856,9 +821,9 @@ cudaError_t bwd_t(const float* rec, const unsigned* off, const unsigned* list, c
 //   [1] the (pixel, Gaussian) slots the forward evaluates: per batch of a
 //       tile's list and 8x8 region, rounds of four Gaussians that reach the
 //       region (its own test), 256 slots each; 64 per Gaussian in 8x8 tiles;
-//   [2] the backward's pixel slots (per tile instance, the rows from the first
-//       to the last with a span, TW columns each, or TW / 2 when no span is
-//       longer than TW / 2 pixels), from the backward's own span arithmetic.
+//   [2] the backward's pixel slots (per tile instance, the rows its footprint
+//       reaches, TW columns each, or TW / 2 when no row needs more), from the
+//       backward's own arithmetic.
 template <int TW, int TH, int PPT>
 __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
     k_count_pairs(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
@@ -880,7 +845,6 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
     const float px = (float)x + 0.5f;
     const int x_org = tc.tx * TW, y_org = tc.ty * TH;
     const int x_lim = min(TW, V.W - x_org), y_lim = min(TH, V.H - y_org);
-    const float QM = kQMax * 1.0001f + 1e-4f;
     unsigned long long cnt_pairs = 0, cnt_fwd = 0, cnt_bwd = 0;
     const unsigned start = offsets[tile], end = offsets[tile + 1];
     for (unsigned base = start; base < end; base += NT) {
@@ -895,20 +859,12 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
             s0[tid] = a;
             s1[tid] = qd;
             hit = regions_hit<F::RX, F::RY>(a, qd, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y);
-            // the backward's pixel slots: the rows from its first span to its last, TW columns each, or
-            // TW / 2 when no span is longer than TW / 2 pixels
-            const RowSpans rs(a, qd, QM);
-            int lo, hi, r_lo = TH, r_hi = -1, umax = 0;
-            rs.rows(a, y_org, 0, y_lim, lo, hi);
-            for (int r = lo; r <= hi; ++r) {
-                const int u = rs.row(a, QM, x_org, y_org, x_lim, r) >> 8;
-                if (u) {
-                    r_lo = min(r_lo, r);
-                    r_hi = max(r_hi, r);
-                    umax = max(umax, u);
-                }
-            }
-            if (r_hi >= r_lo) cnt_bwd += (unsigned long long)(r_hi - r_lo + 1) * (2 * umax > TW / 2 ? TW : TW / 2);
+            // the backward's pixel slots: the rows its footprint reaches, TW or TW / 2 columns each
+            int first, nst;
+            bool wide;
+            Footprint(a, qd).rows<TW>(a, qd, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y, x_lim, y_lim, first,
+                                      nst, wide);
+            cnt_bwd += (unsigned long long)(nst * (wide ? TW : TW / 2));
         }
         __syncthreads();
 #pragma unroll
