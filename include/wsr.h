@@ -123,7 +123,7 @@ typedef struct {
 
 /* Work schedule of the render kernels. */
 enum {
-    WSR_SCHEDULE_TILE_BLOCKS = 0,  /* one thread block per tile */
+    WSR_SCHEDULE_TILE_BLOCKS = 0,  /* the forward: one thread block per tile */
     WSR_SCHEDULE_PERSISTENT = 1    /* one block per SM slot, tiles taken heaviest first */
 };
 
@@ -132,14 +132,15 @@ enum {
  * the render schedule and the backward's Gaussians per block.  With
  * WSR_SCHEDULE_PERSISTENT, wsr_bin also orders the tiles by decreasing
  * instance count (a bucketed longest-first order kept in the workspace) and
- * the render calls launch one block per resident slot that takes tiles from
+ * wsr_render_fwd launches one block per resident slot that takes tiles from
  * that order through a counter in the workspace; the same workspace and tiles
- * must then be passed to wsr_bin and the renderers.  `chunk` is how many of a
- * tile's Gaussians one block of wsr_render_bwd takes at a time: 0 for the
- * default 128 (blocks of 256 threads), 64 (blocks of 128 threads, twice as
- * many resident), 256 or 512 (blocks of 256 threads, fewer barriers per
- * Gaussian); other values return WSR_ERR_UNSUPPORTED.  It changes the schedule only, not the result
- * beyond rounding order.
+ * must then be passed to wsr_bin and the renderers.  The backward always takes
+ * tiles that way (it forms the order itself for the other schedule) and splits
+ * the longest lists over blocks.  `chunk` is how many of a tile's Gaussians a
+ * block of wsr_render_bwd takes at a time: 64 (blocks of 128 threads), 128, 256
+ * or 512 (blocks of 256 threads), or 0 for the default, 512 (128 for views of
+ * at most 608 tiles); other values return WSR_ERR_UNSUPPORTED.  It changes the
+ * schedule only, not the result beyond rounding order.
  *
  * `deterministic` = 1 makes every result bitwise reproducible from run to run
  * for the same inputs and tiles (0, the default, lets the order of atomics
@@ -162,7 +163,7 @@ enum {
 typedef struct {
     int32_t tile_w, tile_h;
     int32_t schedule;            /* WSR_SCHEDULE_* */
-    int32_t chunk;               /* Gaussians per backward block: 0 (128), 64, 256, 512 */
+    int32_t chunk;               /* Gaussians per backward chunk: 0 (default), 64, 128, 256, 512 */
     int32_t deterministic;       /* 0, or 1: bitwise-reproducible results */
 } wsr_tiles;
 

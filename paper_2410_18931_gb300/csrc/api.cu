@@ -26,7 +26,7 @@ bool aligned8(const void* p) { return ((uintptr_t)p & 7u) == 0; }
 // Builds the per-view constant table.  Returns WSR_OK or the argument error.
 wsr_status make_views(const wsr_camera* cams, int32_t n_cams, const wsr_tiles* tiles, Views* vs) {
     if (!cams || n_cams < 1 || n_cams > WSR_MAX_VIEWS) return WSR_ERR_INVALID_ARG;
-    int tw = 16, th = 16, sched = WSR_SCHEDULE_TILE_BLOCKS, chunk = 128, det = 0;
+    int tw = 16, th = 16, sched = WSR_SCHEDULE_TILE_BLOCKS, chunk = 0, det = 0;
     if (tiles) {
         if (tiles->chunk < 0) return WSR_ERR_INVALID_ARG;
         if (tiles->deterministic != 0 && tiles->deterministic != 1) return WSR_ERR_INVALID_ARG;
@@ -39,7 +39,7 @@ wsr_status make_views(const wsr_camera* cams, int32_t n_cams, const wsr_tiles* t
         tw = tiles->tile_w;
         th = tiles->tile_h;
         sched = tiles->schedule;
-        chunk = tiles->chunk ? tiles->chunk : 128;
+        chunk = tiles->chunk;
         det = tiles->deterministic;
     }
     memset(vs, 0, sizeof(Views));
@@ -84,28 +84,28 @@ wsr_status make_views(const wsr_camera* cams, int32_t n_cams, const wsr_tiles* t
 }
 
 struct WsLayout {
-    size_t cursor, block_sums, order, buckets, bg_tiles, bin_base, total;
+    size_t cursor, block_sums, order, buckets, bg_tiles, bwd_work, bin_base, total;
 };
 
-// The tile order of the persistent schedule is only part of its layout; the binning's rows of counters per
-// block (bin_base) come last and are left out of the static scratch.
-WsLayout ws_layout(const Views& vs, bool with_base = true) {
+// What only a caller's workspace holds is left out of the static scratch (render = false): the tile order (and
+// its buckets), which the persistent schedule's binning writes and the backward forms otherwise, the backward's
+// counters, the deterministic mode's background terms and the binning's rows of counters per block.
+WsLayout ws_layout(const Views& vs, bool render = true) {
     WsLayout L;
     const size_t nb = (size_t)(vs.total_tiles + kScanTile - 1) / kScanTile;
     L.cursor = kWsHeader;
     L.block_sums = L.cursor + align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
     L.total = L.block_sums + align256(sizeof(unsigned long long) * (nb + 1));
-    L.order = L.buckets = L.bg_tiles = L.bin_base = 0;
-    if (vs.schedule == WSR_SCHEDULE_PERSISTENT) {
-        L.order = L.total;
-        L.buckets = L.order + align256(sizeof(unsigned) * (size_t)vs.total_tiles);
-        L.total = L.buckets + align256(sizeof(unsigned) * 66);
-    }
+    L.order = L.buckets = L.bg_tiles = L.bwd_work = L.bin_base = 0;
+    if (!render) return L;
+    L.order = L.total;
+    L.buckets = L.order + align256(sizeof(unsigned) * (size_t)vs.total_tiles);
+    L.bwd_work = L.buckets + align256(sizeof(unsigned) * 66);
+    L.total = L.bwd_work + align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
     if (vs.det) {
         L.bg_tiles = L.total;
         L.total = L.bg_tiles + align256(4 * sizeof(float) * (size_t)vs.total_tiles);
     }
-    if (!with_base) return L;
     int t_max = 0;
     for (int v = 0; v < vs.n; ++v) t_max = vs.v[v].tiles_x * vs.v[v].tiles_y > t_max ? vs.v[v].tiles_x * vs.v[v].tiles_y
                                                                                      : t_max;
@@ -114,12 +114,12 @@ WsLayout ws_layout(const Views& vs, bool with_base = true) {
     return L;
 }
 
-Sched sched_of(const Views& vs, void* workspace, int which) {
+Sched sched_of(const Views& vs, void* workspace) {
     Sched sc{nullptr, nullptr};
     if (vs.schedule == WSR_SCHEDULE_PERSISTENT) {
         const WsLayout L = ws_layout(vs);
         sc.order = (const unsigned*)((char*)workspace + L.order);
-        sc.counter = &((WsHeader*)workspace)->work[which];
+        sc.counter = &((WsHeader*)workspace)->work[0];
     }
     return sc;
 }
@@ -341,9 +341,7 @@ wsr_status wsr_bin_static(const float* records, int64_t n, const wsr_camera* cam
     cudaStream_t s = (cudaStream_t)stream;
     void* scratch = nullptr;
     WSR_TRY(static_scratch(s, &scratch));
-    Views vb = vs;                 // the binning's part of the layout (no backward regions)
-    vb.det = 0;
-    const WsLayout L = ws_layout(vb, false);
+    const WsLayout L = ws_layout(vs, false);       // the binning's part
     if (L.total > kStaticBytes) return WSR_ERR_UNSUPPORTED;
     WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, scratch, L, s));
     char* ws = (char*)scratch;
@@ -383,7 +381,7 @@ wsr_status wsr_render_fwd(const float* records, int64_t n, const uint32_t* tile_
         !aligned4(out_den))
         return WSR_ERR_INVALID_ARG;
     return cuda_status(launch_render_fwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den,
-                                         sched_of(vs, workspace, 0), (cudaStream_t)stream));
+                                         sched_of(vs, workspace), (cudaStream_t)stream));
 }
 
 wsr_status wsr_render_bwd_tiles(const float* records, int64_t n, const uint32_t* tile_offsets,
@@ -409,17 +407,23 @@ wsr_status wsr_render_bwd_tiles(const float* records, int64_t n, const uint32_t*
     WSR_CUDA(cudaMemsetAsync(hdr->gw, 0, sizeof hdr->gw, s));
     const size_t rec_floats = vs.det ? WSR_GRAD_RECORD_FLOATS_DET : WSR_GRAD_RECORD_FLOATS;
     if (n > 0) WSR_CUDA(cudaMemsetAsync(grad_records, 0, sizeof(float) * rec_floats * (size_t)n * n_cams, s));
+    const WsLayout L = ws_layout(vs);
+    char* const ws = (char*)workspace;
+    // the binning leaves the tile order only for the persistent schedule
+    BwdSched sched{vs.total_tiles > kFewTiles ? (const unsigned*)(ws + L.order) : nullptr, (unsigned*)(ws + L.bwd_work)};
+    if (vs.schedule != WSR_SCHEDULE_PERSISTENT && sched.order)
+        WSR_CUDA(launch_tile_order(vs, tile_offsets, (unsigned*)(ws + L.buckets), (unsigned*)(ws + L.order), s));
     if (!vs.det) {
         WSR_CUDA(launch_render_bwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den, grad_rgb, grad_records,
-                                   hdr->gw, 0, nullptr, nullptr, sched_of(vs, workspace, 1), s));
+                                   hdr->gw, false, nullptr, nullptr, sched, s));
         return WSR_OK;
     }
     // deterministic: the largest pixel term over the image, then the record terms as exact fixed-point sums
     // in units that a per-Gaussian bound fixes; the background terms per tile, then summed in tile order
-    float* bg_tiles = (float*)((char*)workspace + ws_layout(vs).bg_tiles);
+    float* bg_tiles = (float*)(ws + L.bg_tiles);
     WSR_CUDA(launch_det_pmax(out_rgb, out_den, grad_rgb, vs.total_pix, &hdr->det_pmax, s));
     WSR_CUDA(launch_render_bwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den, grad_rgb, grad_records,
-                               hdr->gw, 1, bg_tiles, &hdr->det_pmax, sched_of(vs, workspace, 1), s));
+                               hdr->gw, true, bg_tiles, &hdr->det_pmax, sched, s));
     WSR_CUDA(launch_det_bg_reduce(bg_tiles, vs.total_tiles, hdr->gw, s));
     return WSR_OK;
 }

@@ -447,7 +447,8 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_small(unsigned* __res
 // as I rows of 32, the rows' shuffles independent of one another, and ranks a tile among its warp's tiles of the
 // same bucket by matching lanes, so that neither pass over the tiles queues on a bucket's counter.  It is bound by
 // the latency of its chain of loads, shuffles and three barriers: 12 -> 6 us for 8160 tiles with the order.
-template <int I>
+// With SCAN false it only orders the tiles of given offsets.
+template <int I, bool SCAN>
 __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __restrict__ cursor, int n,
                                                                 unsigned* __restrict__ offsets,
                                                                 unsigned long long capacity, WsHeader* hdr,
@@ -461,7 +462,10 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
     const int t0 = warp * 32 * I + lane;
     unsigned c[I], rank[I];
 #pragma unroll
-    for (int r = 0; r < I; ++r) c[r] = t0 + 32 * r < n ? cursor[t0 + 32 * r] : 0u;
+    for (int r = 0; r < I; ++r) {
+        const int t = t0 + 32 * r;
+        c[r] = t >= n ? 0u : SCAN ? cursor[t] : offsets[t + 1] - offsets[t];
+    }
     if (order) {
         s_hist[warp][lane] = 0u;
         if (lane == 0) s_hist[warp][32] = 0u;
@@ -478,46 +482,50 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
             rank[r] = h + __popc(same & below);
         }
     }
-    unsigned long long inc[I], sum = 0;
+    if constexpr (SCAN) {
+        unsigned long long inc[I], sum = 0;
 #pragma unroll
-    for (int r = 0; r < I; ++r) inc[r] = c[r];
+        for (int r = 0; r < I; ++r) inc[r] = c[r];
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1)
+        for (int off = 1; off < 32; off <<= 1)
+#pragma unroll
+            for (int r = 0; r < I; ++r) {
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, inc[r], off);
+                if (lane >= off) inc[r] += y;
+            }
 #pragma unroll
         for (int r = 0; r < I; ++r) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, inc[r], off);
-            if (lane >= off) inc[r] += y;
+            const unsigned long long row = __shfl_sync(0xffffffffu, inc[r], 31);
+            inc[r] += sum - c[r];                   // exclusive within the warp's tiles
+            sum += row;
         }
+        if (lane == 0) s_sum[warp] = sum;
+        __syncthreads();
+        unsigned long long x = s_sum[lane], scan = x;
 #pragma unroll
-    for (int r = 0; r < I; ++r) {
-        const unsigned long long row = __shfl_sync(0xffffffffu, inc[r], 31);
-        inc[r] += sum - c[r];                   // exclusive within the warp's tiles
-        sum += row;
-    }
-    if (lane == 0) s_sum[warp] = sum;
-    __syncthreads();
-    unsigned long long x = s_sum[lane], scan = x;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, scan, off);
-        if (lane >= off) scan += y;
-    }
-    const unsigned long long tot = __shfl_sync(0xffffffffu, scan, 31);
-    const unsigned long long first = __shfl_sync(0xffffffffu, scan - x, warp);
-#pragma unroll
-    for (int r = 0; r < I; ++r) {
-        const int t = t0 + 32 * r;
-        const unsigned long long run = first + inc[r];
-        const unsigned o = (unsigned)(run < lim ? run : lim);
-        if (t < n) {
-            offsets[t] = o;
-            cursor[t] = o;                      // the scatter's cursor starts at the tile's offset
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, scan, off);
+            if (lane >= off) scan += y;
         }
-    }
-    if (threadIdx.x == 0) {
-        offsets[n] = (unsigned)(tot < lim ? tot : lim);
-        hdr->total = tot;
-        hdr->err = tot > lim ? WSR_ERR_CAPACITY : 0;        // a binning starts from no error
+        const unsigned long long tot = __shfl_sync(0xffffffffu, scan, 31);
+        const unsigned long long first = __shfl_sync(0xffffffffu, scan - x, warp);
+#pragma unroll
+        for (int r = 0; r < I; ++r) {
+            const int t = t0 + 32 * r;
+            const unsigned long long run = first + inc[r];
+            const unsigned o = (unsigned)(run < lim ? run : lim);
+            if (t < n) {
+                offsets[t] = o;
+                cursor[t] = o;                      // the scatter's cursor starts at the tile's offset
+            }
+        }
+        if (threadIdx.x == 0) {
+            offsets[n] = (unsigned)(tot < lim ? tot : lim);
+            hdr->total = tot;
+            hdr->err = tot > lim ? WSR_ERR_CAPACITY : 0;        // a binning starts from no error
+        }
+    } else {
+        __syncthreads();
     }
     if (!order) return;
     // warp b takes bucket b (warp 0 also bucket 32), a lane per warp's count; then warp 0 the buckets
@@ -625,8 +633,15 @@ __global__ void __launch_bounds__(512) k_sort_segments(const unsigned* __restric
 cudaError_t launch_tile_order(const Views& vs, const unsigned* offsets, unsigned* buckets, unsigned* order,
                               cudaStream_t s) {
     const int n = vs.total_tiles;
+    unsigned* const off = const_cast<unsigned*>(offsets);       // read only
+    if (n <= 16 * kScanBlock) {
+        if (n <= 4 * kScanBlock) k_scan_order_rows<4, false><<<1, kScanBlock, 0, s>>>(nullptr, n, off, 0, nullptr, order);
+        else if (n <= 8 * kScanBlock) k_scan_order_rows<8, false><<<1, kScanBlock, 0, s>>>(nullptr, n, off, 0, nullptr, order);
+        else k_scan_order_rows<16, false><<<1, kScanBlock, 0, s>>>(nullptr, n, off, 0, nullptr, order);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(buckets, 0, sizeof(unsigned) * 33, s);
-    if (e != cudaSuccess || n == 0) return e;
+    if (e != cudaSuccess) return e;
     const int nb = min((n + 255) / 256, 1024);
     k_order_hist<<<nb, 256, 0, s>>>(offsets, n, buckets);
     k_order_scan<<<1, 32, 0, s>>>(buckets);
@@ -698,10 +713,10 @@ cudaError_t launch_scan(const Views& vs, unsigned* cursor, unsigned* block_sums,
                         cudaStream_t s) {
     const int n = vs.total_tiles;
     if (n <= 16 * kScanBlock) {
-        if (n <= kScanBlock) k_scan_order_rows<1><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
-        else if (n <= 4 * kScanBlock) k_scan_order_rows<4><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
-        else if (n <= 8 * kScanBlock) k_scan_order_rows<8><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
-        else k_scan_order_rows<16><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
+        if (n <= kScanBlock) k_scan_order_rows<1, true><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
+        else if (n <= 4 * kScanBlock) k_scan_order_rows<4, true><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
+        else if (n <= 8 * kScanBlock) k_scan_order_rows<8, true><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
+        else k_scan_order_rows<16, true><<<1, kScanBlock, 0, s>>>(cursor, n, offsets, capacity, hdr, order);
         return cudaGetLastError();
     }
     if (n <= kSmallScanTiles) {

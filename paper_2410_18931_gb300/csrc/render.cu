@@ -43,10 +43,11 @@ struct BwdThreads {
     static constexpr int value = CH < 128 ? 2 * CH : 256;
 };
 
-// A lane count as a type, to instantiate one walk of the backward per group size.
-template <int N>
+// Lane counts as a type, to instantiate one walk of the backward per group shape: lanes across a row's column
+// pairs, and rows walked side by side.
+template <int N, int R>
 struct Lanes {
-    static constexpr int value = N;
+    static constexpr int value = N, rows = R;
 };
 
 // The part of a footprint q' <= QM inside a tile, as the backward walks it.  On row dy the footprint is
@@ -429,15 +430,33 @@ __device__ __forceinline__ float warp_sum(float v) {
 // closed form and a row's start formed as it is walked; three blocks per SM at 80
 // registers, without spills, took 960 us.
 constexpr float kMagic = 12582912.0f;       // 1.5 x 2^23
+// Up to this many Gaussians of a class in a chunk are walked by twice the lanes, two rows side by side, so that more
+// warps have some: 915 -> 905 us at 1M Gaussians and 1920x1080, 84 -> 80 us at 150k and 979x543 (more lanes for
+// larger classes cost more bank conflicts than they save: 1111 us with two rows throughout).
+constexpr int kFewWalk = 64;
+// Chunks per part of a tile's list (1 for few tiles): claiming each chunk on its own costs 20 us at 1M Gaussians.
+constexpr unsigned kPartChunks = 4;
+constexpr int kHelpTiles = 1024;            // tiles whose chunks idle blocks look for (a power of two)
 
+// Schedule: as many blocks as fit on the device take the tiles through *counter (in the order given, longest first,
+// or as they are numbered).  A tile's list is cut into parts of part_chunks chunks; those of a tile with several are
+// handed out one by one (parts[tile], zero at the start), and a block that finds no tile left looks for parts nobody
+// has taken among the first tiles of the order, picking its tile at random among those that have any, so that the
+// longest lists do not hold up the end.  Nothing waits for another block: a part is done by whoever takes it, and the
+// block that took the tile itself takes parts until none is left.
+//   Measured against a block per tile and chunks of 128, and against the longest-first order with 512: 1301 and
+// 931 -> 905 us at 1M Gaussians and 1920x1080, 187 and 135 -> 128 us for 200k at 1280x720, 58 -> 22 us for 5000 at
+// 200x120 (104 tiles).  Taking the next tile while one is walked made it slower, 35 us at 1M: a block then holds a
+// tile that others could start.
 template <int TW, int TH, int CH, bool DET>
-__device__ __forceinline__ void bwd_tile(const int tile, const float4* __restrict__ rec,
-                                         const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
-                                         const Views& vs, const float* __restrict__ wparams,
-                                         const float* __restrict__ out_rgb, const float* __restrict__ out_den,
-                                         const float* __restrict__ grad_rgb, float* __restrict__ grec,
-                                         float* __restrict__ gw, float* __restrict__ bg_tiles,
-                                         const unsigned* __restrict__ det_pmax) {
+__global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::value)
+    k_render_bwd(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
+                 const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
+                 const float* __restrict__ out_rgb, const float* __restrict__ out_den,
+                 const float* __restrict__ grad_rgb, float* __restrict__ grec, float* __restrict__ gw,
+                 float* __restrict__ bg_tiles, const unsigned* __restrict__ det_pmax,
+                 const unsigned* __restrict__ order, unsigned* __restrict__ counter, unsigned* __restrict__ parts,
+                 const unsigned part_chunks) {
     constexpr int NT = BwdThreads<CH>::value;
     constexpr int NW = NT / 32;
     // pixel-table row pitch in column pairs: the row's TW / 2 pairs, then zero pairs up to the farthest pair a
@@ -447,6 +466,7 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     constexpr int NB = TH + 1;                          // row counts 0 .. TH
     constexpr int NK = 2 * NB;                          // sort keys: narrow 0 .. TH, wide NB .. NB + TH
     static_assert(CH % 32 == 0 && TW % 8 == 0 && TW <= 64 && CH <= 512 && NK <= NT, "layout");
+    static_assert((TW * TH) % NT == 0 || NT % (TW * TH) == 0, "whole pixels per thread");
     constexpr int M = TW >= 16 ? 4 : 2;                 // column pairs per lane and row in step C
     // per pixel: G/D (3), -(G.C)/D, stored per column pair as (x0, x1, y0, y1) and (z0, z1, w0, w1)
     __shared__ float4 spA[PP * TH];
@@ -462,253 +482,296 @@ __device__ __forceinline__ void bwd_tile(const int tile, const float4* __restric
     __shared__ unsigned short sord[CH];         // the chunk's Gaussians: wide ones first, most rows first
     __shared__ unsigned shist[NK];
     __shared__ unsigned snext[2];               // per class: the next position of the order a warp takes
-    __shared__ float sbg[4][NW];
+    __shared__ float4 sbg[NW];                  // background terms per warp
+    __shared__ int4 s_cur;                      // the tile (-1: none left) and its ends
+    __shared__ unsigned s_part;
 
-    const TileCoord tc = tile_coord(vs, tile);
-    const View& V = vs.v[tc.v];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int x_org = tc.tx * TW, y_org = tc.ty * TH;
-    const int x_lim = min(TW, V.W - x_org);    // pixels of the tile inside the image
-    const int y_lim = min(TH, V.H - y_org);
+    const int n = vs.total_tiles;
     const float wB = __ldg(wparams + 2);
-    const float cB0 = __ldg(wparams + 3), cB1 = __ldg(wparams + 4), cB2 = __ldg(wparams + 5);
     const float pmax = DET ? __int_as_float(*det_pmax) : 0.0f;    // deterministic mode
-
-    float bg[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int p = tid; p < 2 * PP * TH; p += NT) {
-        const int ly = p / (2 * PP), lx = p - ly * (2 * PP);
-        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (lx < x_lim && ly < y_lim) {
-            const long long pix = V.pix_base + (long long)(y_org + ly) * V.W + x_org + lx;
-            const float inv = 1.0f / out_den[pix];
-            const float G0 = grad_rgb[3 * pix], G1 = grad_rgb[3 * pix + 1], G2 = grad_rgb[3 * pix + 2];
-            const float C0 = out_rgb[3 * pix], C1 = out_rgb[3 * pix + 1], C2 = out_rgb[3 * pix + 2];
-            f = make_float4(G0 * inv, G1 * inv, G2 * inv, -(G0 * C0 + G1 * C1 + G2 * C2) * inv);
-            // dL/dw_B = G.(c_B - C)/D,  dL/dc_B = G w_B / D
-            bg[0] += f.x * cB0 + f.y * cB1 + f.z * cB2 + f.w;
-            bg[1] += f.x * wB;
-            bg[2] += f.y * wB;
-            bg[3] += f.z * wB;
+    auto load_item = [&](unsigned item) {
+        int t = -1;
+        unsigned a = 0u, b = 0u;
+        if (item < (unsigned)n) {
+            t = order ? (int)order[item] : (int)item;
+            a = offsets[t];
+            b = offsets[t + 1];
         }
-        const int pi = 4 * (ly * PP + (lx >> 1)) + (lx & 1);
-        reinterpret_cast<float*>(spA)[pi] = f.x;
-        reinterpret_cast<float*>(spA)[pi + 2] = f.y;
-        reinterpret_cast<float*>(spB)[pi] = f.z;
-        reinterpret_cast<float*>(spB)[pi + 2] = f.w;
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float t = warp_sum(bg[c]);
-        if (lane == 0) sbg[c][warp] = t;
-    }
-
-    const unsigned start = offsets[tile], end = offsets[tile + 1];
+        s_cur = make_int4(t, (int)a, (int)b, 0);
+    };
+    if (tid == 0) load_item(atomicAdd(counter, 1u));
     if (tid < NK) shist[tid] = 0u;
-    for (unsigned base = start; base < end; base += CH) {
-        const int cnt = (int)min((unsigned)CH, end - base);
-        __syncthreads();                                // the previous chunk is done with shared memory
-        // ---- A: record, rows and class of a Gaussian per thread ----
-#pragma unroll 1
-        for (int gj = tid; gj < cnt; gj += NT) {
-            const unsigned r = list[base + gj];
-            const float4* pr = rec + 3ull * r;
-            const float4 a = __ldg(pr);
-            const float4 b = __ldg(pr + 1);
-            const float cb = __ldg(reinterpret_cast<const float*>(pr + 2));
-            s0[gj] = a;
-            s1[gj] = b;
-            s2[gj] = f2(cb, b.y);
-            sidx[gj] = r;
-            int first, nst;
-            bool wide;
-            Footprint(a, b.x).rows<TW>(a, b.x, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y, x_lim, y_lim,
-                                       first, nst, wide);
-            const int key = nst + (wide ? NB : 0);
-            sfirst[gj] = (unsigned char)first;
-            snst[gj] = (unsigned char)nst;
-            skey[gj] = (unsigned char)key;
-            srank[gj] = (unsigned short)atomicAdd(&shist[key], 1u);
+    for (int p = tid; p < PP * TH; p += NT) spA[p] = spB[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+
+    for (;;) {
+        int tile = s_cur.x;
+        unsigned start = (unsigned)s_cur.y, end = (unsigned)s_cur.z;
+        const bool first = tile >= 0;                   // this block took the tile: it sums its background terms
+        if (first) {
+        } else {
+            __syncthreads();
+            if (tid == 0) s_part = 0u;
+            __syncthreads();
+            unsigned best = 0u;                         // a random number and the position, 0: none
+            for (int pos = tid; pos < min(n, kHelpTiles); pos += NT) {
+                const unsigned t = order ? order[pos] : (unsigned)pos;
+                const unsigned np = (offsets[t + 1] - offsets[t] + CH * part_chunks - 1) / (CH * part_chunks);
+                if (np > 1 && __ldcg(parts + t) < np) {
+                    const unsigned h = ((unsigned)pos * 2654435761u ^ (blockIdx.x + 1u) * 2246822519u) * 3266489917u;
+                    best = max(best, (h & ~(unsigned)(kHelpTiles - 1)) | (unsigned)pos | (unsigned)kHelpTiles);
+                }
+            }
+            best = __reduce_max_sync(0xffffffffu, best);
+            if (lane == 0 && best) atomicMax(&s_part, best);
+            __syncthreads();
+            best = s_part;
+            if (best == 0u) break;
+            __syncthreads();                            // s_part is read: the parts below write it again
+            best &= (unsigned)(kHelpTiles - 1);
+            tile = order ? (int)order[best] : (int)best;
+            start = offsets[tile];
+            end = offsets[tile + 1];
         }
-        if (tid < 2) snext[tid] = 0u;
-        __syncthreads();
-        // ---- B: the chunk's order, wide first, most rows first: each warp forms the buckets' starts (the
-        // counts of all larger keys, a suffix scan over the NK <= 64 keys held two per lane), and a
-        // Gaussian's position is its bucket's start plus its rank in the bucket ----
-        const unsigned h0 = lane < NK ? shist[lane] : 0u, h1 = lane + 32 < NK ? shist[lane + 32] : 0u;
-        unsigned s0i = h0, s1i = h1;                    // inclusive suffix sums of keys lane and lane + 32
+        const TileCoord tc = tile_coord(vs, tile);
+        const View& V = vs.v[tc.v];
+        const int x_org = tc.tx * TW, y_org = tc.ty * TH;
+        const int x_lim = min(TW, V.W - x_org);         // pixels of the tile inside the image
+        const int y_lim = min(TH, V.H - y_org);
+
+        const unsigned per_part = CH * part_chunks, n_parts = (end - start + per_part - 1) / per_part;
+        float4 bg = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned y0 = __shfl_down_sync(0xffffffffu, s0i, off), y1 = __shfl_down_sync(0xffffffffu, s1i, off);
-            if (lane + off < 32) {
-                s0i += y0;
-                s1i += y1;
+        for (int k = 0; k < (TW * TH > NT ? TW * TH / NT : 1); ++k) {
+            const int p = tid + k * NT, ly = p / TW, lx = p - ly * TW;
+            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lx < x_lim && ly < y_lim) {
+                const long long pix = V.pix_base + (long long)(y_org + ly) * V.W + x_org + lx;
+                const float inv = 1.0f / out_den[pix];
+                const float G0 = grad_rgb[3 * pix], G1 = grad_rgb[3 * pix + 1], G2 = grad_rgb[3 * pix + 2];
+                const float C0 = out_rgb[3 * pix], C1 = out_rgb[3 * pix + 1], C2 = out_rgb[3 * pix + 2];
+                f = make_float4(G0 * inv, G1 * inv, G2 * inv, -(G0 * C0 + G1 * C1 + G2 * C2) * inv);
+                // dL/dw_B = G.(c_B - C)/D,  dL/dc_B = G w_B / D
+                bg.x += f.x * __ldg(wparams + 3) + f.y * __ldg(wparams + 4) + f.z * __ldg(wparams + 5) + f.w;
+                bg.y += f.x * wB;
+                bg.z += f.y * wB;
+                bg.w += f.z * wB;
+            }
+            if (TW * TH >= NT || p < TW * TH) {
+                const int pi = 4 * (ly * PP + (lx >> 1)) + (lx & 1);
+                reinterpret_cast<float*>(spA)[pi] = f.x;
+                reinterpret_cast<float*>(spA)[pi + 2] = f.y;
+                reinterpret_cast<float*>(spB)[pi] = f.z;
+                reinterpret_cast<float*>(spB)[pi + 2] = f.w;
             }
         }
-        s0i += __shfl_sync(0xffffffffu, s1i, 0);        // keys 32.. lie above every key of the first half
-        const unsigned start0 = s0i - h0, start1 = s1i - h1;
-        const int nwide = (int)__shfl_sync(0xffffffffu, s0i, NB);   // Gaussians with keys NB and up: the wide
-        static_assert(NB < 32, "the wide class starts in the first half of the keys");
-        for (int g0 = warp * 32; g0 < cnt; g0 += NT) {
-            const int gj = g0 + lane;
-            const int key = gj < cnt ? (int)skey[gj] : 0;
-            const unsigned a0 = __shfl_sync(0xffffffffu, start0, key & 31);
-            const unsigned a1 = __shfl_sync(0xffffffffu, start1, key & 31);
-            if (gj < cnt) sord[(key < 32 ? a0 : a1) + srank[gj]] = (unsigned short)gj;
+        if (first) {
+            bg = make_float4(warp_sum(bg.x), warp_sum(bg.y), warp_sum(bg.z), warp_sum(bg.w));
+            if (lane == 0) sbg[warp] = bg;
         }
-        __syncthreads();
-        if (tid < NK) shist[tid] = 0u;                  // for the next chunk (step C does not read it)
-        // ---- C: a group per Gaussian; each warp takes the next 32 / L Gaussians of a class ----
-        auto walk = [&](auto lanes, const int lo, const int hi, unsigned* next) {
-            constexpr int L = decltype(lanes)::value;
-            constexpr int GW = 32 / L;                  // groups per warp
-            const int grp = lane / L, gk = lane % L;    // group and lane within the group
-            for (;;) {
-                unsigned at0 = 0;
-                if (lane == 0) at0 = atomicAdd(next, (unsigned)GW);
-                at0 = __shfl_sync(0xffffffffu, at0, 0);
-                if (lo + (int)at0 >= hi) break;
-                const int so = lo + (int)at0 + grp;
-                const bool act = so < hi;
-                const int j = act ? (int)sord[so] : 0;
-                const int steps = act ? (int)snst[j] : 0;
-                const int r0 = act ? (int)sfirst[j] : 0;
-                const float4 a = s0[j], b = s1[j];
-                const float2 c2 = s2[j];
-                const float gx0 = (float)x_org + 0.5f - a.x;                 // dx of column 0
-                const float gy0 = (float)y_org + 0.5f - a.y;                 // dy of row 0
-                const float qs = a.z;
-                const float2 qw2 = f2(a.w, a.w), qd2 = f2(b.x, b.x), gx2 = f2(gx0, gx0);
-                // dL/dq' = e (P . cw) with cw = -ln2 u w (c, 1): the walk uses the colour c = (c u w) / (u w)
-                // (in both halves of a pair) and applies the factor -ln2 u w to the moments once, after it
-                const float iuw = c2.y != 0.0f ? 1.0f / c2.y : 0.0f;
-                const float2 ccr = f2(b.z * iuw, b.z * iuw), ccg = f2(b.w * iuw, b.w * iuw);
-                const float2 ccb = f2(c2.x * iuw, c2.x * iuw);
-                // accumulators, each over the two pixels of a column pair: d/d(c u w) per channel, d/d(u w);
-                // and the moments of gq = dL/dq' in the record's own frame (r = qs dy + qw dx, dx):
-                // sum gq r^2, sum gq r dx, sum gq dx^2, sum gq r, sum gq dx.  Kept apart, a thin
-                // footprint's small along-axis terms (dx) are not rounded away under its large r terms.
-                float2 gr = f2(0.f, 0.f), gg = gr, gb = gr, gu = gr;
-                float2 srr = f2(0.f, 0.f), srx = srr, sxx = srr, sr = srr, sx = srr;
-                // dx of this lane's first column pair (2 k, 2 k + 1) from the row's even first column, less that column
-                const float2 gxb = __fadd2_rn(f2((float)(2 * gk), (float)(2 * gk + 1)), gx2);
-                const Footprint fp(a, b.x);
-                const float left = -gx0 - 0.025f;                               // columns, with a little slack
-                int row = r0 * PP + gk - __float_as_int(kMagic);
-                const float yend = (float)(r0 + steps);
-                for (float yf = (float)r0; yf < yend; row += PP, yf += 1.0f) {
-                    const float dy = yf + gy0, rb = qs * dy;
-                    // the row's first column v (not beyond the last pair), rounded up and then down to even:
-                    // round(v / 2), by adding a number whose last bit weighs one
-                    const float v = fmaf(-fp.slope, dy, left) - sqrt_approx(fmaxf(fmaf(-fp.h1 * dy, dy, fp.h0), 0.0f));
-                    const float w = fmaf(fminf(fmaxf(v, 0.0f), (float)(TW - 2)), 0.5f, kMagic);
-                    const int pb = row + __float_as_int(w);
-                    const float xsf = fmaf(w, 2.0f, -2.0f * kMagic);
-                    const float2 xb = __fadd2_rn(f2(xsf, xsf), gxb);             // dx of the lane's first pair
-                    const float2 rb2 = f2(rb, rb);
+        for (unsigned part = 0;; ++part) {
+            if (n_parts > 1) {
+                if (tid == 0) s_part = atomicAdd(parts + tile, 1u);
+                __syncthreads();
+                part = s_part;
+            }
+            if (part >= n_parts) break;
+            const unsigned part_end = min(end, start + (part + 1) * per_part);
+            for (unsigned base = start + part * per_part; base < part_end; base += CH) {
+                const int cnt = (int)min((unsigned)CH, part_end - base);
+                // ---- A: record, rows and class of a Gaussian per thread ----
+#pragma unroll 1
+                for (int gj = tid; gj < cnt; gj += NT) {
+                    const unsigned r = list[base + gj];
+                    const float4* pr = rec + 3ull * r;
+                    const float4 a = __ldg(pr), b = __ldg(pr + 1);
+                    const float cb = __ldg(reinterpret_cast<const float*>(pr + 2));
+                    s0[gj] = a;
+                    s1[gj] = b;
+                    s2[gj] = f2(cb, b.y);
+                    sidx[gj] = r;
+                    int row, nst;
+                    bool wide;
+                    Footprint(a, b.x).rows<TW>(a, b.x, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y, x_lim, y_lim,
+                                               row, nst, wide);
+                    const int key = nst + (wide ? NB : 0);
+                    sfirst[gj] = (unsigned char)row;
+                    snst[gj] = (unsigned char)nst;
+                    skey[gj] = (unsigned char)key;
+                    srank[gj] = (unsigned short)atomicAdd(&shist[key], 1u);
+                }
+                if (tid < 2) snext[tid] = 0u;
+                __syncthreads();
+                // ---- B: the chunk's order, wide first, most rows first: each warp forms the buckets' starts (the
+                // counts of all larger keys, a suffix scan over the NK <= 64 keys held two per lane), and a
+                // Gaussian's position is its bucket's start plus its rank in the bucket ----
+                const unsigned h0 = lane < NK ? shist[lane] : 0u, h1 = lane + 32 < NK ? shist[lane + 32] : 0u;
+                unsigned s0i = h0, s1i = h1;                    // inclusive suffix sums of keys lane and lane + 32
 #pragma unroll
-                    for (int m = 0; m < M; ++m) {
-                        // Columns outside the footprint evaluate q > 9, so the cutoff test zeroes them; pairs past
-                        // the tile and rows past the image read zero pairs.  No per-pixel mask is needed.
-                        const int pi = pb + m * L;
-                        const float4 A = spA[pi], B = spB[pi];          // (x0, x1, y0, y1), (z0, z1, w0, w1)
-                        const float2 dx = m == 0 ? xb : __fadd2_rn(xb, f2((float)(2 * m * L), (float)(2 * m * L)));
-                        const float2 rr = __ffma2_rn(qw2, dx, rb2);
-                        const float2 q = __ffma2_rn(rr, rr, __fmul2_rn(__fmul2_rn(qd2, dx), dx));
-                        const float2 e = f2(ex2_approx(q.x <= kQMax ? -q.x : -256.0f),      // 2^-256 flushes to 0
-                                            ex2_approx(q.y <= kQMax ? -q.y : -256.0f));
-                        // d/d(c u w) and d/d(u w) at fixed c u w
-                        gr = __ffma2_rn(f2(A.x, A.y), e, gr);
-                        gg = __ffma2_rn(f2(A.z, A.w), e, gg);
-                        gb = __ffma2_rn(f2(B.x, B.y), e, gb);
-                        gu = __ffma2_rn(f2(B.z, B.w), e, gu);
-                        // dL/dq' per pixel, less the factor -ln2 u w: e * (P_w + c . P_rgb)
-                        const float2 pc = __ffma2_rn(f2(B.x, B.y), ccb, __ffma2_rn(f2(A.z, A.w), ccg,
-                                                     __ffma2_rn(f2(A.x, A.y), ccr, f2(B.z, B.w))));
-                        const float2 gq = __fmul2_rn(e, pc);
-                        const float2 tr = __fmul2_rn(gq, rr), tx = __fmul2_rn(gq, dx);
-                        srr = __ffma2_rn(tr, rr, srr);
-                        srx = __ffma2_rn(tr, dx, srx);
-                        sxx = __ffma2_rn(tx, dx, sxx);
-                        sr = __fadd2_rn(sr, tr);
-                        sx = __fadd2_rn(sx, tx);
+                for (int off = 1; off < 32; off <<= 1) {
+                    const unsigned y0 = __shfl_down_sync(0xffffffffu, s0i, off), y1 = __shfl_down_sync(0xffffffffu, s1i, off);
+                    if (lane + off < 32) {
+                        s0i += y0;
+                        s1i += y1;
                     }
                 }
-                // the group's sums: record order sum gq r, sum gq dx, sum gq r^2, sum gq r dx, sum gq dx^2,
-                // d/d(u w), d/d(c u w)
-                const float fq = -kLn2 * c2.y;
-                float vals[9] = {fq * (sr.x + sr.y), fq * (sx.x + sx.y), fq * (srr.x + srr.y), fq * (srx.x + srx.y),
-                                 fq * (sxx.x + sxx.y), gu.x + gu.y, gr.x + gr.y, gg.x + gg.y, gb.x + gb.y};
-                __syncwarp();
+                s0i += __shfl_sync(0xffffffffu, s1i, 0);        // keys 32.. lie above every key of the first half
+                const unsigned start0 = s0i - h0, start1 = s1i - h1;
+                const int nwide = (int)__shfl_sync(0xffffffffu, s0i, NB);   // Gaussians with keys NB and up: the wide
+                static_assert(NB < 32, "the wide class starts in the first half of the keys");
+                for (int g0 = warp * 32; g0 < cnt; g0 += NT) {
+                    const int gj = g0 + lane;
+                    const int key = gj < cnt ? (int)skey[gj] : 0;
+                    const unsigned a0 = __shfl_sync(0xffffffffu, start0, key & 31);
+                    const unsigned a1 = __shfl_sync(0xffffffffu, start1, key & 31);
+                    if (gj < cnt) sord[(key < 32 ? a0 : a1) + srank[gj]] = (unsigned short)gj;
+                }
+                __syncthreads();
+                if (tid < NK) shist[tid] = 0u;                  // for the next chunk (step C does not read it)
+                // ---- C: a group per Gaussian; each warp takes the next 32 / L Gaussians of a class ----
+                auto walk = [&](auto lanes, const int lo, const int hi, unsigned* next) {
+                    constexpr int L = decltype(lanes)::value, RP = decltype(lanes)::rows, LT = L * RP;
+                    constexpr int GW = 32 / LT;                 // groups per warp
+                    const int grp = lane / LT, gk = lane % L, rp = lane % LT / L;    // group, column lane and row lane
+                    for (;;) {
+                        unsigned at0 = 0;
+                        if (lane == 0) at0 = atomicAdd(next, (unsigned)GW);
+                        at0 = __shfl_sync(0xffffffffu, at0, 0);
+                        if (lo + (int)at0 >= hi) break;
+                        const int so = lo + (int)at0 + grp;
+                        const bool act = so < hi;
+                        const int j = act ? (int)sord[so] : 0;
+                        const int steps = act ? (int)snst[j] : 0;
+                        const int r0 = act ? (int)sfirst[j] : 0;
+                        const float4 a = s0[j], b = s1[j];
+                        const float2 c2 = s2[j];
+                        const float gx0 = (float)x_org + 0.5f - a.x;                 // dx of column 0
+                        const float gy0 = (float)y_org + 0.5f - a.y;                 // dy of row 0
+                        const float qs = a.z;
+                        const float2 qw2 = f2(a.w, a.w), qd2 = f2(b.x, b.x), gx2 = f2(gx0, gx0);
+                        // dL/dq' = e (P . cw) with cw = -ln2 u w (c, 1): the walk uses the colour c = (c u w) / (u w)
+                        // (in both halves of a pair) and applies the factor -ln2 u w to the moments once, after it
+                        const float iuw = c2.y != 0.0f ? 1.0f / c2.y : 0.0f;
+                        const float2 ccr = f2(b.z * iuw, b.z * iuw), ccg = f2(b.w * iuw, b.w * iuw);
+                        const float2 ccb = f2(c2.x * iuw, c2.x * iuw);
+                        // accumulators, each over the two pixels of a column pair: d/d(c u w) per channel, d/d(u w);
+                        // and the moments of gq = dL/dq' in the record's own frame (r = qs dy + qw dx, dx):
+                        // sum gq r^2, sum gq r dx, sum gq dx^2, sum gq r, sum gq dx.  Kept apart, a thin
+                        // footprint's small along-axis terms (dx) are not rounded away under its large r terms.
+                        float2 gr = f2(0.f, 0.f), gg = gr, gb = gr, gu = gr;
+                        float2 srr = f2(0.f, 0.f), srx = srr, sxx = srr, sr = srr, sx = srr;
+                        // dx of this lane's first column pair (2 k, 2 k + 1) from the row's even first column, less that column
+                        const float2 gxb = __fadd2_rn(f2((float)(2 * gk), (float)(2 * gk + 1)), gx2);
+                        const Footprint fp(a, b.x);
+                        const float left = -gx0 - 0.025f;                               // columns, with a little slack
+                        int row = (r0 + rp) * PP + gk - __float_as_int(kMagic);
+                        const float yend = (float)(r0 + steps);
+                        for (float yf = (float)(r0 + rp); yf < yend; row += RP * PP, yf += (float)RP) {
+                            const float dy = yf + gy0, rb = qs * dy;
+                            // the row's first column v (not beyond the last pair), rounded up and then down to even:
+                            // round(v / 2), by adding a number whose last bit weighs one
+                            const float v = fmaf(-fp.slope, dy, left) - sqrt_approx(fmaxf(fmaf(-fp.h1 * dy, dy, fp.h0), 0.0f));
+                            const float w = fmaf(fminf(fmaxf(v, 0.0f), (float)(TW - 2)), 0.5f, kMagic);
+                            const int pb = row + __float_as_int(w);
+                            const float xsf = fmaf(w, 2.0f, -2.0f * kMagic);
+                            const float2 xb = __fadd2_rn(f2(xsf, xsf), gxb);             // dx of the lane's first pair
+                            const float2 rb2 = f2(rb, rb);
 #pragma unroll
-                for (int off = L / 2; off > 0; off >>= 1)
+                            for (int m = 0; m < M; ++m) {
+                                // Columns outside the footprint evaluate q > 9, so the cutoff test zeroes them; pairs past
+                                // the tile and rows past the image read zero pairs.  No per-pixel mask is needed.
+                                const int pi = pb + m * L;
+                                const float4 A = spA[pi], B = spB[pi];          // (x0, x1, y0, y1), (z0, z1, w0, w1)
+                                const float2 dx = m == 0 ? xb : __fadd2_rn(xb, f2((float)(2 * m * L), (float)(2 * m * L)));
+                                const float2 rr = __ffma2_rn(qw2, dx, rb2);
+                                const float2 q = __ffma2_rn(rr, rr, __fmul2_rn(__fmul2_rn(qd2, dx), dx));
+                                const float2 e = f2(ex2_approx(q.x <= kQMax ? -q.x : -256.0f),      // 2^-256 flushes to 0
+                                                    ex2_approx(q.y <= kQMax ? -q.y : -256.0f));
+                                // d/d(c u w) and d/d(u w) at fixed c u w
+                                gr = __ffma2_rn(f2(A.x, A.y), e, gr);
+                                gg = __ffma2_rn(f2(A.z, A.w), e, gg);
+                                gb = __ffma2_rn(f2(B.x, B.y), e, gb);
+                                gu = __ffma2_rn(f2(B.z, B.w), e, gu);
+                                // dL/dq' per pixel, less the factor -ln2 u w: e * (P_w + c . P_rgb)
+                                const float2 pc = __ffma2_rn(f2(B.x, B.y), ccb, __ffma2_rn(f2(A.z, A.w), ccg,
+                                                             __ffma2_rn(f2(A.x, A.y), ccr, f2(B.z, B.w))));
+                                const float2 gq = __fmul2_rn(e, pc);
+                                const float2 tr = __fmul2_rn(gq, rr), tx = __fmul2_rn(gq, dx);
+                                srr = __ffma2_rn(tr, rr, srr);
+                                srx = __ffma2_rn(tr, dx, srx);
+                                sxx = __ffma2_rn(tx, dx, sxx);
+                                sr = __fadd2_rn(sr, tr);
+                                sx = __fadd2_rn(sx, tx);
+                            }
+                        }
+                        // the group's sums: record order sum gq r, sum gq dx, sum gq r^2, sum gq r dx, sum gq dx^2,
+                        // d/d(u w), d/d(c u w)
+                        const float fq = -kLn2 * c2.y;
+                        float vals[9] = {fq * (sr.x + sr.y), fq * (sx.x + sx.y), fq * (srr.x + srr.y), fq * (srx.x + srx.y),
+                                         fq * (sxx.x + sxx.y), gu.x + gu.y, gr.x + gr.y, gg.x + gg.y, gb.x + gb.y};
+                        __syncwarp();
 #pragma unroll
-                    for (int c = 0; c < 9; ++c) vals[c] += __shfl_xor_sync(0xffffffffu, vals[c], off);
-                if (act && gk == 0 && steps > 0) {
-                    if constexpr (!DET) {
-                        float4* o = reinterpret_cast<float4*>(grec + (size_t)WSR_GRAD_RECORD_FLOATS * sidx[j]);
-                        atomicAdd(o, make_float4(vals[0], vals[1], vals[2], vals[3]));
-                        atomicAdd(o + 1, make_float4(vals[4], vals[5], vals[6], vals[7]));
-                        atomicAdd(reinterpret_cast<float*>(o + 2), vals[8]);
-                    } else {
-                        // deterministic mode: a 128-byte record holds 9 int64 sums, then the 9 bounds (float
-                        // bits) that fix their units.  A term's bound caps the sum of its absolute pixel
-                        // terms over the whole footprint, the same in every tile of the Gaussian: at most
-                        // (2 hx + 2)(2 hy + 2) pixels (hx, hy its half-extents), each with e <= 1, every
-                        // pixel-table entry at most pmax, |r| <= sqrt(QM), |dx| <= hx inside the cutoff.
-                        float* o = grec + (size_t)kDetRecordFloats * sidx[j];
-                        int* mag = reinterpret_cast<int*>(o + 18);
-                        constexpr float QM = kQMax * 1.0001f + 1e-4f;
-                        const float qd = b.x, hx = sqrtf(QM / qd);
-                        const float hy = sqrtf(QM * fmaf(a.w, a.w, qd) / (qd * a.z * a.z));
-                        const float npx = fminf((2.0f * hx + 2.0f) * (2.0f * hy + 2.0f), 1e12f);
-                        const float gqm = pmax * kLn2 * 1.0001f * (fabsf(b.z) + fabsf(b.w) + fabsf(c2.x) + fabsf(b.y));
-                        const float sq = sqrtf(QM);
-                        const float bound[9] = {npx * gqm * sq, npx * gqm * hx, npx * gqm * QM, npx * gqm * sq * hx,
-                                                npx * gqm * hx * hx, npx * pmax, npx * pmax, npx * pmax, npx * pmax};
-                        unsigned long long* sum = reinterpret_cast<unsigned long long*>(o);
+                        for (int off = LT / 2; off > 0; off >>= 1)
 #pragma unroll
-                        for (int c = 0; c < 9; ++c) {
-                            const float m = fminf(bound[c], 1e30f);
-                            mag[c] = __float_as_int(m);     // every tile of the Gaussian writes the same value
-                            if (m > 0.0f) {
-                                int e;
-                                frexpf(m, &e);              // m < 2^e
-                                const long long q = __double2ll_rn(ldexp((double)vals[c], kDetBits - e));
-                                atomicAdd(sum + c, (unsigned long long)q);
+                            for (int c = 0; c < 9; ++c) vals[c] += __shfl_xor_sync(0xffffffffu, vals[c], off);
+                        if (act && lane % LT == 0 && steps > 0) {
+                            if constexpr (!DET) {
+                                float4* o = reinterpret_cast<float4*>(grec + (size_t)WSR_GRAD_RECORD_FLOATS * sidx[j]);
+                                atomicAdd(o, make_float4(vals[0], vals[1], vals[2], vals[3]));
+                                atomicAdd(o + 1, make_float4(vals[4], vals[5], vals[6], vals[7]));
+                                atomicAdd(reinterpret_cast<float*>(o + 2), vals[8]);
+                            } else {
+                                // deterministic mode: a 128-byte record holds 9 int64 sums, then the 9 bounds (float
+                                // bits) that fix their units.  A term's bound caps the sum of its absolute pixel
+                                // terms over the whole footprint, the same in every tile of the Gaussian: at most
+                                // (2 hx + 2)(2 hy + 2) pixels (hx, hy its half-extents), each with e <= 1, every
+                                // pixel-table entry at most pmax, |r| <= sqrt(QM), |dx| <= hx inside the cutoff.
+                                float* o = grec + (size_t)kDetRecordFloats * sidx[j];
+                                int* mag = reinterpret_cast<int*>(o + 18);
+                                constexpr float QM = kQMax * 1.0001f + 1e-4f;
+                                const float qd = b.x, hx = sqrtf(QM / qd);
+                                const float hy = sqrtf(QM * fmaf(a.w, a.w, qd) / (qd * a.z * a.z));
+                                const float npx = fminf((2.0f * hx + 2.0f) * (2.0f * hy + 2.0f), 1e12f);
+                                const float gqm = pmax * kLn2 * 1.0001f * (fabsf(b.z) + fabsf(b.w) + fabsf(c2.x) + fabsf(b.y));
+                                const float sq = sqrtf(QM);
+                                const float bound[9] = {npx * gqm * sq, npx * gqm * hx, npx * gqm * QM, npx * gqm * sq * hx,
+                                                        npx * gqm * hx * hx, npx * pmax, npx * pmax, npx * pmax, npx * pmax};
+                                unsigned long long* sum = reinterpret_cast<unsigned long long*>(o);
+#pragma unroll
+                                for (int c = 0; c < 9; ++c) {
+                                    const float m = fminf(bound[c], 1e30f);
+                                    mag[c] = __float_as_int(m);     // every tile of the Gaussian writes the same value
+                                    if (m > 0.0f) {
+                                        int e;
+                                        frexpf(m, &e);              // m < 2^e
+                                        const long long q = __double2ll_rn(ldexp((double)vals[c], kDetBits - e));
+                                        atomicAdd(sum + c, (unsigned long long)q);
+                                    }
+                                }
                             }
                         }
                     }
-                }
+                };
+                // few Gaussians: more lanes each, so that every warp has some
+                if (nwide > kFewWalk) walk(Lanes<TW / (2 * M), 1>(), 0, nwide, &snext[0]);        // the wide class
+                else walk(Lanes<TW / (2 * M), 2>(), 0, nwide, &snext[0]);
+                if (cnt - nwide > kFewWalk) walk(Lanes<TW / (4 * M), 1>(), nwide, cnt, &snext[1]);   // the narrow class
+                else walk(Lanes<TW / (4 * M), 2>(), nwide, cnt, &snext[1]);
+                __syncthreads();                                // this chunk is done with shared memory
             }
-        };
-        walk(Lanes<TW / (2 * M)>(), 0, nwide, &snext[0]);        // the wide class
-        walk(Lanes<TW / (4 * M)>(), nwide, cnt, &snext[1]);      // the narrow class
-    }
-    __syncthreads();
-    if (tid < 4) {
-        float t = 0.0f;
-        for (int w = 0; w < NW; ++w) t += sbg[tid][w];
-        if constexpr (!DET) {
-            if (t != 0.0f) atomicAdd(gw + 2 + tid, t);
-        } else {
-            bg_tiles[4 * (size_t)tile + tid] = t;      // summed in tile order afterwards
         }
+        if (n_parts == 0) __syncthreads();                      // every thread has read s_cur, sbg is written
+        if (first && tid == 0) load_item(atomicAdd(counter, 1u));
+        if (first && tid >= 32 && tid < 36) {
+            const int c = tid - 32;
+            float t = 0.0f;
+            for (int w = 0; w < NW; ++w) t += reinterpret_cast<const float*>(&sbg[w])[c];
+            if constexpr (DET) bg_tiles[4 * (size_t)tile + c] = t;      // summed in tile order afterwards
+            else if (t != 0.0f) atomicAdd(gw + 2 + c, t);
+        }
+        __syncthreads();                                        // s_cur is written, s_part and sbg read
     }
-}
-
-template <int TW, int TH, int CH, bool DET>
-__global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::value)
-    k_render_bwd(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
-                 const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
-                 const float* __restrict__ out_rgb, const float* __restrict__ out_den,
-                 const float* __restrict__ grad_rgb, float* __restrict__ grec, float* __restrict__ gw,
-                 float* __restrict__ bg_tiles, const unsigned* __restrict__ det_pmax,
-                 const unsigned* __restrict__ order,
-                 unsigned* __restrict__ counter) {
-    for_each_tile(order, counter, vs.total_tiles, [&](int tile) {
-        bwd_tile<TW, TH, CH, DET>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den, grad_rgb, grec, gw,
-                                  bg_tiles, det_pmax);
-    });
 }
 
 // Deterministic mode: the largest magnitude of the backward's pixel terms, G / D per channel and
@@ -762,8 +825,6 @@ unsigned grid_for(K kernel, int threads, const Views& vs, const Sched& sched) {
     return (unsigned)min(max(1, sms * max(per_sm, 1)), vs.total_tiles);
 }
 
-constexpr int kFwdSliceTiles = 608;     // four per SM
-
 template <int TW, int TH, int S>
 cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
@@ -783,35 +844,38 @@ cudaError_t fwd_t(const float* rec, const unsigned* off, const unsigned* list, c
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
     // Two slices where the tiles alone leave the SMs idle: 14.4 -> 10.4 us at 240 tiles, 14.5 -> 13.7 at 475
     // (40k Gaussians), 14.4 -> 15.1 at 920, 39 -> 70 at 8160.
-    return vs.total_tiles <= kFwdSliceTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
+    return vs.total_tiles <= kFewTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
                                             : fwd_s<TW, TH, 1>(rec, off, list, vs, w, rgb, den, sched, s);
 }
 
 template <int TW, int TH, int CH>
 cudaError_t bwd_chunk(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
-                      const float* rgb, const float* den, const float* grgb, float* grec, float* gw, int pass,
-                      float* bg_tiles, const unsigned* det_pmax, Sched sched, cudaStream_t s) {
+                      const float* rgb, const float* den, const float* grgb, float* grec, float* gw, bool det,
+                      float* bg_tiles, const unsigned* det_pmax, const BwdSched& sched, cudaStream_t s) {
     constexpr int NT = BwdThreads<CH>::value;
-    auto kernel = pass == 0 ? k_render_bwd<TW, TH, CH, false> : k_render_bwd<TW, TH, CH, true>;
-    const unsigned grid = grid_for(kernel, NT, vs, sched);
-    if (sched.order) {
-        cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
-        if (e != cudaSuccess) return e;
-    }
-    kernel<<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params,
-                                                     rgb, den, grgb, grec, gw, bg_tiles, det_pmax,
-                                                     sched.order, sched.counter);
+    auto kernel = det ? k_render_bwd<TW, TH, CH, true> : k_render_bwd<TW, TH, CH, false>;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0);
+    const long long most = (long long)max(sms, 1) * max(per_sm, 1), want = 4ll * vs.total_tiles;
+    cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned) * ((size_t)vs.total_tiles + 1), s);
+    if (e != cudaSuccess) return e;
+    kernel<<<(unsigned)min(most, want), NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb,
+                                                    den, grgb, grec, gw, bg_tiles, det_pmax, sched.order,
+                                                    sched.counter, sched.counter + 1,
+                                                    vs.total_tiles <= kFewTiles ? 1u : kPartChunks);
     return cudaGetLastError();
 }
 
 template <int TW, int TH>
 cudaError_t bwd_t(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
-                  const float* rgb, const float* den, const float* grgb, float* grec, float* gw, int pass,
-                  float* bg_tiles, const unsigned* det_pmax, Sched sched, cudaStream_t s) {
-    const int ch = vs.chunk;
+                  const float* rgb, const float* den, const float* grgb, float* grec, float* gw, bool det,
+                  float* bg_tiles, const unsigned* det_pmax, const BwdSched& sched, cudaStream_t s) {
+    const int ch = vs.chunk ? vs.chunk : vs.total_tiles <= kFewTiles ? 128 : 512;
     auto k = ch == 64 ? bwd_chunk<TW, TH, 64> : ch == 256 ? bwd_chunk<TW, TH, 256>
                                               : ch == 512 ? bwd_chunk<TW, TH, 512> : bwd_chunk<TW, TH, 128>;
-    return k(rec, off, list, vs, w, rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax, sched, s);
+    return k(rec, off, list, vs, w, rgb, den, grgb, grec, gw, det, bg_tiles, det_pmax, sched, s);
 }
 
 // Diagnostic: the work of the render kernels, three counts added to count[0..2]:
@@ -950,17 +1014,17 @@ cudaError_t launch_render_fwd(const float* rec, const unsigned* off, const unsig
 
 cudaError_t launch_render_bwd(const float* rec, const unsigned* off, const unsigned* list, const Views& vs,
                               WeightDev w, const float* rgb, const float* den, const float* grgb, float* grec,
-                              float* gw, int pass, float* bg_tiles, const unsigned* det_pmax, Sched sc,
+                              float* gw, bool det, float* bg_tiles, const unsigned* det_pmax, const BwdSched& sc,
                               cudaStream_t s) {
     if (vs.total_tiles == 0) return cudaSuccess;
     if (vs.tile_w == 16 && vs.tile_h == 16)
-        return bwd_t<16, 16>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax, sc, s);
+        return bwd_t<16, 16>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, det, bg_tiles, det_pmax, sc, s);
     if (vs.tile_w == 8 && vs.tile_h == 8)
-        return bwd_t<8, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax, sc, s);
+        return bwd_t<8, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, det, bg_tiles, det_pmax, sc, s);
     if (vs.tile_w == 32 && vs.tile_h == 8)
-        return bwd_t<32, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax, sc, s);
+        return bwd_t<32, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, det, bg_tiles, det_pmax, sc, s);
     if (vs.tile_w == 16 && vs.tile_h == 8)
-        return bwd_t<16, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, pass, bg_tiles, det_pmax, sc, s);
+        return bwd_t<16, 8>(rec, off, list, vs, w, rgb, den, grgb, grec, gw, det, bg_tiles, det_pmax, sc, s);
     return cudaErrorInvalidValue;
 }
 

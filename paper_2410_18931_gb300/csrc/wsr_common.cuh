@@ -40,14 +40,16 @@ struct Views {
     int total_tiles;
     long long total_pix;
     int schedule;         // WSR_SCHEDULE_*
-    int chunk;            // Gaussians per block of the backward (64 or 128)
+    int chunk;            // Gaussians per chunk of the backward (0: by the number of tiles)
     int det;              // deterministic mode (wsr_tiles.deterministic)
     View v[WSR_MAX_VIEWS];
 };
 
 // Workspace layout: [header 8 KB][cursor: total_tiles + 1 u32][block sums]
-//                   [tile order: total_tiles u32][order buckets: 64 u32]
+//                   [tile order: total_tiles u32][order buckets: 66 u32]
+//                   [backward: counter and chunks taken per tile, total_tiles + 1 u32]
 //                   [deterministic mode: background terms per tile, 4 floats]
+//                   [binning: a row of counters per block of k_bin_local]
 // The header's first 256 bytes are the struct below; in deterministic mode the
 // projection backward keeps its per-block sigma/beta sums after it.
 struct WsHeader {
@@ -55,7 +57,7 @@ struct WsHeader {
     int pad0;
     float gw[8];               // gradient accumulators of sigma, beta, w_B, c_B (6 used)
     unsigned long long total;  // tile instances counted by the last binning
-    unsigned int work[4];      // persistent-schedule counters: [0] forward, [1] backward
+    unsigned int work[4];      // [0] the forward's persistent-schedule counter
     unsigned int det_pmax;     // deterministic mode: the largest |pixel term| G/D, (G.C)/D (float bits)
 };
 

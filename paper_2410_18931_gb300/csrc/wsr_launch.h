@@ -67,7 +67,11 @@ cudaError_t launch_bin_scatter(const float* records, long long n, const Views& v
 cudaError_t launch_sort_segments(const Views& vs, const unsigned* tile_offsets, unsigned* tile_list,
                                  WsHeader* hdr, cudaStream_t s);
 
-// Work distribution of a render launch: order == nullptr means one block per
+// Views of at most this many tiles (four per SM) leave SMs idle with a block per tile: the forward then splits each
+// tile's list in two, and the backward takes smaller chunks and needs no order.
+constexpr int kFewTiles = 608;
+
+// Work distribution of a forward launch: order == nullptr means one block per
 // tile; otherwise a persistent grid takes tiles order[0..total) via *counter
 // (reset by the launcher).
 struct Sched {
@@ -78,15 +82,26 @@ struct Sched {
 cudaError_t launch_render_fwd(const float* records, const unsigned* tile_offsets,
                               const unsigned* tile_list, const Views& vs, WeightDev w,
                               float* out_rgb, float* out_den, Sched sched, cudaStream_t s);
-// pass 0: float atomics into WSR_GRAD_RECORD_FLOATS records and grad_wparams.  Deterministic mode
-// (pass 1, WSR_GRAD_RECORD_FLOATS_DET records): the record terms added as fixed point in units set by
-// a per-Gaussian bound from *det_pmax (launch_det_pmax first), each tile's background terms stored in
-// bg_tiles[4 tile + c].
+
+// The longest-first tile order of a binning's offsets (`buckets`: 66 words of scratch).
+cudaError_t launch_tile_order(const Views& vs, const unsigned* tile_offsets, unsigned* buckets, unsigned* order,
+                              cudaStream_t s);
+
+// Work distribution of a backward launch: the tile order (nullptr: as numbered), and total_tiles + 1 words that the
+// launcher clears: the counter of tiles taken, then each tile's counter of chunks taken.
+struct BwdSched {
+    const unsigned* order;
+    unsigned* counter;
+};
+
+// Float atomics into WSR_GRAD_RECORD_FLOATS records and grad_wparams; or (det, the deterministic mode,
+// WSR_GRAD_RECORD_FLOATS_DET records) the record terms added as fixed point in units set by a per-Gaussian bound from
+// *det_pmax (launch_det_pmax first), each tile's background terms stored in bg_tiles[4 tile + c].
 cudaError_t launch_render_bwd(const float* records, const unsigned* tile_offsets,
                               const unsigned* tile_list, const Views& vs, WeightDev w,
                               const float* out_rgb, const float* out_den, const float* grad_rgb,
-                              float* grad_records, float* grad_wparams, int pass, float* bg_tiles,
-                              const unsigned* det_pmax, Sched sched, cudaStream_t s);
+                              float* grad_records, float* grad_wparams, bool det, float* bg_tiles,
+                              const unsigned* det_pmax, const BwdSched& sched, cudaStream_t s);
 // deterministic mode: grad_wparams[2..5] = the tiles' background terms summed in tile order
 cudaError_t launch_det_pmax(const float* out_rgb, const float* out_den, const float* grad_rgb, long long npix,
                             unsigned* pmax, cudaStream_t s);

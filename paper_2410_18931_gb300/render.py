@@ -98,6 +98,9 @@ class Renderer:
         else:
             self.bin_kernels = 5 + (3 if persistent else 0)
         self.bin_kernels += 1 if self.deterministic else 0
+        # kernels the backward launches to order the tiles when the binning has not (the per-tile schedule): none for
+        # few tiles, one up to 16384, else three
+        self.order_kernels = 0 if persistent or self.num_tiles <= 608 else 1 if self.num_tiles <= 16384 else 3
         self.num_pix = int(self.lib.wsr_num_pixels(self.cams_c, self.n_cams))
         ws = int(self.lib.wsr_workspace_size(self.cams_c, self.n_cams, ctypes.byref(self.tiles_c)))
         if self.num_tiles <= 0 or ws == 0:

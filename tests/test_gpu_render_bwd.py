@@ -48,3 +48,34 @@ def test_backward_rows_and_classes(kind, tile, chunk):
             continue                             # a sphere has no orientation: the gradient is zero
         ex = grad_excess(out[k].cpu().numpy(), env, k)
         assert ex <= GRAD_TOL, (k, ex)
+
+
+@pytest.mark.parametrize("n,size", [(5000, (64, 48)), (4097, (64, 48)), (9000, (480, 352)), (9000, (16 * 41, 240))])
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("chunk", [0, 128, 512])
+def test_split_lists_give_the_gradients_of_one_block_per_list(n, size, persistent, chunk):
+    """Most of the Gaussians on one tile, so that its list has many parts (few tiles: a chunk each; more: four), taken
+    by several blocks: the gradients are the deterministic mode's (exact integer sums) up to FP32 rounding."""
+    import torch
+
+    from paper_2410_18931_gb300 import Gaussians, Renderer
+    sc = ws.random_scene(n, 7, sh_degree=0, vd_opacity=False, box=0.02, log_scale_mu=-5.0, log_scale_sd=0.4)
+    sc.means[::50] *= 60.0                       # a few elsewhere
+    cam = ws.look_at((0.0, 0.0, -3.0), width=size[0], height=size[1])
+    cam.cx, cam.cy = 24.0, 24.0                  # the cluster in the middle of the second tile
+    cam = cam.rounded()
+    w = ws.default_weight(ws.EXP)
+    g = Gaussians.from_scene(sc)
+    wpar = torch.tensor(w.as_array(), device="cuda")
+    G = torch.tensor(np.random.default_rng(3).normal(size=(size[0] * size[1], 3)).astype(np.float32), device="cuda")
+    outs = []
+    for det in (False, True):
+        r = Renderer([cam], tile=(16, 16), chunk=chunk, persistent=persistent, deterministic=det)
+        st = r.forward(g, w.kind, wpar, check=not det)           # the list may be too long for the mode's sort
+        r.wsr_check()
+        outs.append(r.backward(g, w.kind, wpar, st, G))
+        longest = int(torch.diff(st.tile_offsets).max())
+    assert longest > 2048
+    for k in (*KEYS, "weight_params"):
+        a, b = outs[0][k].double(), outs[1][k].double()
+        assert float((a - b).abs().max()) <= 1e-4 * max(float(b.abs().max()), 1e-12), k
