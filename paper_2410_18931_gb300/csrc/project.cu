@@ -22,6 +22,8 @@
 // dilation terms): a sum of squares with no cancellation.  For strongly
 // anisotropic footprints (det < 1e-3 a c) the conic is recomputed in FP64
 // from the same rows.
+#include <mutex>
+
 #include "wsr_launch.h"
 
 namespace wsr {
@@ -235,52 +237,211 @@ __device__ __forceinline__ void store_n(float* __restrict__ p, const float* v) {
     }
 }
 
-// ONE: a single view.  Its SH and opacity-SH gradients are final as soon as
-// they are formed, so they are stored there and neither they nor the SH
-// coefficients stay live through the geometry chain (about 60 registers
-// fewer: three blocks of 128 per SM instead of two).
+// A block's SH rows in shared memory: R floats per Gaussian, P apart.  Rows that are whole float4s are padded so
+// that a row per lane falls on distinct banks; other rows (odd lengths do already) lie as in global memory.
+template <int R>
+struct Rows {
+    static constexpr int P = R % 4 ? R : (R / 4 + 1) % 2 ? R + 4 : (R / 4) % 2 ? R : R + 8;
+    static_assert(R % 4 || (P / 4) % 2, "an odd number of float4s apart");
+};
+
+// Whether rows of R stored as T lie in shared memory as they are stored (else as floats): halfs in whole 16 bytes.
+template <int R, typename T>
+constexpr bool kRawHalfs = sizeof(T) == 2 && R % 8 == 0;
+
+// A thread's own row as floats: 16 bytes at a time where the rows are padded for it.
+template <int R, typename T>
+__device__ __forceinline__ void row_get(const float* __restrict__ row, float (&v)[R]) {
+    if constexpr (kRawHalfs<R, T>) {
+#pragma unroll
+        for (int c = 0; c < R / 8; ++c) {
+            const uint4 x = reinterpret_cast<const uint4*>(row)[c];
+            const T* e = reinterpret_cast<const T*>(&x);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[8 * c + j] = to_f(e[j]);
+        }
+    } else if constexpr (R % 4 == 0) {
+#pragma unroll
+        for (int c = 0; c < R / 4; ++c) {
+            const float4 x = reinterpret_cast<const float4*>(row)[c];
+            v[4 * c] = x.x, v[4 * c + 1] = x.y, v[4 * c + 2] = x.z, v[4 * c + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < R; ++e) v[e] = row[e];
+    }
+}
+template <int R>
+__device__ __forceinline__ void row_put(float* __restrict__ row, const float (&v)[R]) {
+    if constexpr (R % 4 == 0) {
+#pragma unroll
+        for (int c = 0; c < R / 4; ++c)
+            reinterpret_cast<float4*>(row)[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < R; ++e) row[e] = v[e];
+    }
+}
+
+// Rows [0, cnt) of R consecutive T each from global memory (16-byte aligned) to shared memory, consecutive lanes on
+// consecutive 16 bytes; asynchronous copies where nothing is converted.
+template <int R, typename T>
+__device__ __forceinline__ void rows_in(float* __restrict__ sm, const T* __restrict__ g, const int cnt) {
+    constexpr int PER = 16 / (int)sizeof(T), P = Rows<R>::P;
+    constexpr bool RAW = sizeof(T) == 4 || kRawHalfs<R, T>;
+    const int total = cnt * R, whole = total / PER;
+    if constexpr (RAW) {
+        for (int c = threadIdx.x; c < whole; c += blockDim.x) {
+            float* const o = sm + (sizeof(T) == 4 ? P == R ? 4 * c : 4 * c / R * P + 4 * c % R
+                                                  : 8 * c / R * P + 8 * c % R / 2);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(o)),
+                         "l"(reinterpret_cast<const uint4*>(g) + c) : "memory");
+        }
+        // (rows of halfs are whole 16 bytes: nothing is left over)
+        for (int k = whole * PER + threadIdx.x; k < total; k += blockDim.x) sm[k / R * P + k % R] = to_f(g[k]);
+    } else {
+#pragma unroll 4
+        for (int c = threadIdx.x; c < whole; c += blockDim.x) {
+            const uint4 u = __ldg(reinterpret_cast<const uint4*>(g) + c);
+            const T* e = reinterpret_cast<const T*>(&u);
+#pragma unroll
+            for (int j = 0; j < PER; ++j) sm[(c * PER + j) / R * P + (c * PER + j) % R] = to_f(e[j]);
+        }
+        for (int k = whole * PER + threadIdx.x; k < total; k += blockDim.x) sm[k / R * P + k % R] = to_f(g[k]);
+    }
+}
+
+// The way back, floats: 16 bytes per lane when the output allows it (only its elements' alignment is asked for).
+template <int R>
+__device__ __forceinline__ void rows_out(float* __restrict__ g, const float* __restrict__ sm, const int cnt) {
+    constexpr int P = Rows<R>::P;
+    const int total = cnt * R, whole = (reinterpret_cast<uintptr_t>(g) & 15u) ? 0 : total / 4;
+#pragma unroll 4
+    for (int c = threadIdx.x; c < whole; c += blockDim.x)
+        reinterpret_cast<float4*>(g)[c] = *reinterpret_cast<const float4*>(sm + (P == R ? 4 * c : 4 * c / R * P + 4 * c % R));
+    for (int k = 4 * whole + threadIdx.x; k < total; k += blockDim.x) g[k] = sm[k / R * P + k % R];
+}
+
+// From degree 2 up the SH coefficients and their gradients go through shared memory, a row per thread there and 16
+// bytes per lane in global memory: a row per thread in global memory puts each lane of an access on a line of its
+// own, and the lines, not the bytes, bound the kernel.  Neither then stays in registers.  The copies in and the
+// gradient record's loads are all in flight at once (with a round of loads at a time the kernel took 200 us).
+// ONE: a single view, whose SH gradients are final as soon as they are formed and take the coefficients' place;
+// several views add theirs in rows beside them.  Below degree 2 the rows are short and stay in registers.
+//   One view, 1M Gaussians of degree 3 with view-dependent opacity: 138 -> 117 us (636 MB, 80% of the copy rate);
+// 400k of degree 2: 82 -> 37 us (rows of 27 floats took 4-byte accesses); six views of 300k, degree 2: 128 -> 84 us.
+// Blocks per SM: at degree 3 four, for five the registers spill (136 us).
 template <int DEG, bool VD, bool RED, bool ONE>
-__global__ void __launch_bounds__(128, ONE ? 3 : 1) k_project_bwd(const GaussPtrs g, const Views vs, const WeightDev wd,
-                                                     const float* __restrict__ grec, const wsr_grads out,
-                                                     float* __restrict__ det_sb) {
-    constexpr int K = (DEG + 1) * (DEG + 1);
+__global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) : (DEG == 3 ? 3 : DEG == 2 ? 4 : 1))
+    k_project_bwd(const GaussPtrs g, const Views vs, const WeightDev wd, const float* __restrict__ grec,
+                  const wsr_grads out, float* __restrict__ det_sb) {
+    using sq_t = typename Store<RED>::sq_t;
+    using sh_t = typename Store<RED>::sh_t;
+    constexpr int K = (DEG + 1) * (DEG + 1), KA = VD ? K : 1;
+    constexpr bool ROWS = DEG >= 2;
+    constexpr int PH = Rows<3 * K>::P, PA = Rows<KA>::P;
+    extern __shared__ __align__(16) float s_rows[];
+    float* const s_h = s_rows;                                  // coefficients, or (ONE) at the end gradients
+    float* const s_a = s_h + 128 * PH;                          // opacity likewise
+    float* const s_gh = ONE ? s_h : s_a + 128 * PA;             // gradients
+    float* const s_ga = ONE ? s_a : s_gh + 128 * PH;
     float gsig = 0.0f, gbeta = 0.0f;
+    const float sigma = __ldg(wd.params + 0), beta = __ldg(wd.params + 1);
     // det_sb != nullptr: deterministic mode (fixed-point records, a bounded grid striding over the
     // Gaussians, sigma/beta summed per block in a fixed order into det_sb)
-    auto body = [&](const long long i) {
-        Params<DEG, VD, RED> P;
-        load_params<DEG, VD, RED>(g, i, wd.kind, P);
-        const float sigma = __ldg(wd.params + 0), beta = __ldg(wd.params + 1);
-        float qn[4], qlen, Rg[9], s[3];
-        rot_scale(P.q, P.ls, qn, qlen, Rg, s);
+    for (long long i0 = 128ll * blockIdx.x; i0 < g.n; i0 += 128ll * gridDim.x) {
+        const int cnt = (int)min(128ll, g.n - i0);
+        const long long i = i0 + threadIdx.x;
+        const bool mine = (int)threadIdx.x < cnt;
+        float p[3] = {0.f, 0.f, 0.f}, ls[3] = {0.f, 0.f, 0.f}, q[4] = {1.f, 0.f, 0.f, 0.f}, lcv = 0.0f;
+        if (mine) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) p[k] = __ldg(g.means + 3 * i + k);
+            load_n<sq_t, 3>(reinterpret_cast<const sq_t*>(g.log_scales) + 3 * i, ls);
+            load_n<sq_t, 4>(reinterpret_cast<const sq_t*>(g.quats) + 4 * i, q);
+            if (wd.kind == WSR_WEIGHT_LC) lcv = __ldg(g.lc_v + i);
+        }
+        float rh[ROWS ? 1 : 3 * K], ra_[ROWS ? 1 : KA];             // short rows, in registers
+        float rgh[ROWS ? 1 : 3 * K], rga[ROWS ? 1 : KA];
+        if constexpr (ROWS) {
+            rows_in<3 * K>(s_h, reinterpret_cast<const sh_t*>(g.sh) + 3ll * K * i0, cnt);
+            rows_in<KA>(s_a, reinterpret_cast<const sh_t*>(g.opacity) + (long long)KA * i0, cnt);
+        } else if (mine) {
+            load_n<sh_t, 3 * K>(reinterpret_cast<const sh_t*>(g.sh) + 3ll * K * i, rh);
+            load_n<sh_t, KA>(reinterpret_cast<const sh_t*>(g.opacity) + (long long)KA * i, ra_);
+        }
+        float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;       // a gradient record (not the deterministic mode's)
+        float rc = 0.0f;
+        auto load_record = [&](int v) {
+            const float4* r = reinterpret_cast<const float4*>(grec + WSR_GRAD_RECORD_FLOATS * ((long long)v * g.n + i));
+            ra = __ldg(r);
+            rb = __ldg(r + 1);
+            rc = __ldg(reinterpret_cast<const float*>(r + 2));
+        };
+        if (mine && det_sb == nullptr) load_record(0);
+        auto get_h = [&](float (&h)[3 * K], float (&ha)[KA]) {
+            if constexpr (ROWS) {
+                row_get<3 * K, sh_t>(s_h + PH * threadIdx.x, h);
+                row_get<KA, sh_t>(s_a + PA * threadIdx.x, ha);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 3 * K; ++e) h[e] = rh[e];
+#pragma unroll
+                for (int e = 0; e < KA; ++e) ha[e] = ra_[e];
+            }
+        };
+        auto get_g = [&](float (&h)[3 * K], float (&ha)[KA]) {
+            if constexpr (ROWS) {
+                row_get<3 * K, float>(s_gh + PH * threadIdx.x, h);
+                row_get<KA, float>(s_ga + PA * threadIdx.x, ha);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 3 * K; ++e) h[e] = rgh[e];
+#pragma unroll
+                for (int e = 0; e < KA; ++e) ha[e] = rga[e];
+            }
+        };
+        auto put_g = [&](const float (&h)[3 * K], const float (&ha)[KA]) {
+            if constexpr (ROWS) {
+                row_put<3 * K>(s_gh + PH * threadIdx.x, h);
+                row_put<KA>(s_ga + PA * threadIdx.x, ha);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 3 * K; ++e) rgh[e] = h[e];
+#pragma unroll
+                for (int e = 0; e < KA; ++e) rga[e] = ha[e];
+            }
+        };
+        const float zero_h[3 * K] = {}, zero_a[KA] = {};
+        if constexpr (!ONE || !ROWS) put_g(zero_h, zero_a);
+        if constexpr (ROWS) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+        }
 
+        float qn[4], qlen, Rg[9], s[3];
+        rot_scale(q, ls, qn, qlen, Rg, s);
         float gp[3] = {0.f, 0.f, 0.f}, gs[3] = {0.f, 0.f, 0.f}, gR[9];
 #pragma unroll
         for (int e = 0; e < 9; ++e) gR[e] = 0.f;
-        float gH[K * 3];
-#pragma unroll
-        for (int e = 0; e < K * 3; ++e) gH[e] = 0.f;
-        float gHa[VD ? K : 1];
-#pragma unroll
-        for (int e = 0; e < (VD ? K : 1); ++e) gHa[e] = 0.f;
         float glcv = 0.f;
-        bool sh_stored = false;
+        bool sh_done = false;           // ONE: the rows hold the gradients
 
         const int nv = ONE ? 1 : vs.n;
-        for (int v = 0; v < nv; ++v) {
+        for (int v = 0; mine && v < nv; ++v) {
             const View& V = vs.v[v];
+            const float* const gr = grec + (det_sb ? kDetRecordFloats : WSR_GRAD_RECORD_FLOATS) * ((long long)v * g.n + i);
             float g9[9];
             bool any = false;
             if (det_sb == nullptr) {
-                const float* gr = grec + WSR_GRAD_RECORD_FLOATS * ((long long)v * g.n + i);
+                g9[0] = ra.x, g9[1] = ra.y, g9[2] = ra.z, g9[3] = ra.w;
+                g9[4] = rb.x, g9[5] = rb.y, g9[6] = rb.z, g9[7] = rb.w;
+                g9[8] = rc;
+                if (!ONE && v + 1 < nv) load_record(v + 1);         // the next view's, while this one is chained
 #pragma unroll
-                for (int e = 0; e < 9; ++e) {
-                    g9[e] = __ldg(gr + e);
-                    any |= (g9[e] != 0.0f);
-                }
+                for (int e = 0; e < 9; ++e) any |= (g9[e] != 0.0f);
             } else {
                 // 9 int64 sums in units of 2^(e - kDetBits), 2^e above the term's bound (stored beside them)
-                const float* gr = grec + kDetRecordFloats * ((long long)v * g.n + i);
                 const long long* sums = reinterpret_cast<const long long*>(gr);
                 const int* mag = reinterpret_cast<const int*>(gr + 18);
 #pragma unroll
@@ -297,37 +458,34 @@ __global__ void __launch_bounds__(128, ONE ? 3 : 1) k_project_bwd(const GaussPtr
                 }
             }
             if (!any) continue;
-            const float tz0 = V.R[6] * P.p[0] + V.R[7] * P.p[1] + V.R[8] * P.p[2] + V.T[2];
+            const float tz0 = V.R[6] * p[0] + V.R[7] * p[1] + V.R[8] * p[2] + V.T[2];
             if (!(tz0 > V.znear)) continue;
             const float wf = depth_factor(wd.kind, tz0, sigma, beta);
             if (wf == 0.0f) continue;
-            const float w = (wd.kind == WSR_WEIGHT_LC) ? wf * P.lcv : wf;
+            const float w = (wd.kind == WSR_WEIGHT_LC) ? wf * lcv : wf;
             Geom G;
-            geometry(V, Rg, s, P.p[0], P.p[1], P.p[2], G);
+            geometry(V, Rg, s, p[0], p[1], p[2], G);
             const float tx = G.tx, ty = G.ty, tz = G.tz;
 
-            float vx = P.p[0] - V.campos[0], vy = P.p[1] - V.campos[1], vz = P.p[2] - V.campos[2];
+            float vx = p[0] - V.campos[0], vy = p[1] - V.campos[1], vz = p[2] - V.campos[2];
             const float il = rsqrtf(vx * vx + vy * vy + vz * vz);
             const float dx = vx * il, dy = vy * il, dz = vz * il;
             float Y[K];
             sh_basis<DEG>(dx, dy, dz, Y);
-            float raw[3], col[3];
+            float raw[3] = {0.f, 0.f, 0.f}, col[3], u = 0.0f;
+            {
+                float h[3 * K], ha[KA];
+                get_h(h, ha);
 #pragma unroll
-            for (int ch = 0; ch < 3; ++ch) {
-                float r = 0.0f;
+                for (int k = 0; k < K; ++k) {
 #pragma unroll
-                for (int k = 0; k < K; ++k) r += Y[k] * P.H[3 * k + ch];
-                raw[ch] = r;
-                col[ch] = fmaxf(r + 0.5f, 0.0f);
+                    for (int ch = 0; ch < 3; ++ch) raw[ch] += Y[k] * h[3 * k + ch];
+                    if constexpr (VD) u += Y[k] * ha[k];
+                }
+                if constexpr (!VD) u = 1.0f / (1.0f + expf(-ha[0]));
             }
-            float u;
-            if constexpr (VD) {
-                u = 0.0f;
 #pragma unroll
-                for (int k = 0; k < K; ++k) u += Y[k] * P.Ha[k];
-            } else {
-                u = 1.0f / (1.0f + expf(-P.Ha[0]));
-            }
+            for (int ch = 0; ch < 3; ++ch) col[ch] = fmaxf(raw[ch] + 0.5f, 0.0f);
             const float uw = u * w;
 
             // Eq. 7 record terms -> colour, opacity, weight
@@ -338,46 +496,28 @@ __global__ void __launch_bounds__(128, ONE ? 3 : 1) k_project_bwd(const GaussPtr
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) graw[ch] = (raw[ch] + 0.5f > 0.0f) ? gcuw[ch] * uw : 0.0f;
             float wk[K];
-            if constexpr (ONE) {
-                float gHv[K * 3];
+            if constexpr (ROWS) asm volatile("" ::: "memory");      // read the rows again rather than keep them in registers
+            {
+                float h[3 * K], ha[KA];
+                get_h(h, ha);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    gHv[3 * k + 0] = graw[0] * Y[k];
-                    gHv[3 * k + 1] = graw[1] * Y[k];
-                    gHv[3 * k + 2] = graw[2] * Y[k];
-                    wk[k] = graw[0] * P.H[3 * k] + graw[1] * P.H[3 * k + 1] + graw[2] * P.H[3 * k + 2];
+                    wk[k] = graw[0] * h[3 * k] + graw[1] * h[3 * k + 1] + graw[2] * h[3 * k + 2];
+                    if constexpr (VD) wk[k] += gu * ha[k];
                 }
-                if (out.sh) store_n<K * 3>(out.sh + (long long)K * 3 * i, gHv);
-                if constexpr (VD) {
-                    float gHav[K];
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        gHav[k] = gu * Y[k];
-                        wk[k] += gu * P.Ha[k];
-                    }
-                    if (out.opacity) store_n<K>(out.opacity + (long long)K * i, gHav);
-                } else {
-                    if (out.opacity) out.opacity[i] = gu * u * (1.0f - u);
+                if constexpr (!ONE) {
+                    get_g(h, ha);
                 }
-                sh_stored = true;
-            } else {
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    gH[3 * k + 0] += graw[0] * Y[k];
-                    gH[3 * k + 1] += graw[1] * Y[k];
-                    gH[3 * k + 2] += graw[2] * Y[k];
-                    wk[k] = graw[0] * P.H[3 * k] + graw[1] * P.H[3 * k + 1] + graw[2] * P.H[3 * k + 2];
-                }
-                if constexpr (VD) {
 #pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        gHa[k] += gu * Y[k];
-                        wk[k] += gu * P.Ha[k];
-                    }
-                } else {
-                    gHa[0] += gu * u * (1.0f - u);
+                    for (int ch = 0; ch < 3; ++ch) h[3 * k + ch] = (ONE ? 0.0f : h[3 * k + ch]) + graw[ch] * Y[k];
+                    if constexpr (VD) ha[k] = (ONE ? 0.0f : ha[k]) + gu * Y[k];
                 }
+                if constexpr (!VD) ha[0] = (ONE ? 0.0f : ha[0]) + gu * u * (1.0f - u);
+                put_g(h, ha);
             }
+            sh_done = true;
             // direction dir = (p - f)/|p - f|: tangential part of the SH gradient
             float gdx = 0.f, gdy = 0.f, gdz = 0.f;
             sh_grad_dot<DEG>(dx, dy, dz, wk, gdx, gdy, gdz);
@@ -396,8 +536,8 @@ __global__ void __launch_bounds__(128, ONE ? 3 : 1) k_project_bwd(const GaussPtr
             } else if (wd.kind == WSR_WEIGHT_LC) {
                 const float lin = 1.0f - tz / sigma;
                 glcv += gw * lin;
-                gsig += gw * P.lcv * tz / (sigma * sigma);
-                gt[2] += gw * (-P.lcv / sigma);
+                gsig += gw * lcv * tz / (sigma * sigma);
+                gt[2] += gw * (-lcv / sigma);
             }
             // The record holds moments of gq = dL/dq' over the Gaussian's pixels in the sum-of-squares
             // frame of q' = r^2 + qd dx^2, r = qs dy + qw dx (qs, qw, qd exactly as rendered):
@@ -484,27 +624,25 @@ __global__ void __launch_bounds__(128, ONE ? 3 : 1) k_project_bwd(const GaussPtr
 #pragma unroll
         for (int k = 0; k < 3; ++k) gls[k] = gs[k] * s[k];
 
-        if (out.means) { out.means[3 * i] = gp[0]; out.means[3 * i + 1] = gp[1]; out.means[3 * i + 2] = gp[2]; }
-        if (out.log_scales) {
-            out.log_scales[3 * i] = gls[0]; out.log_scales[3 * i + 1] = gls[1]; out.log_scales[3 * i + 2] = gls[2];
-        }
-        if (out.quats) store_n<4>(out.quats + 4 * i, gq);
-        if (!sh_stored) {           // several views, or a single view that added nothing (zeros)
-            if (out.sh) store_n<K * 3>(out.sh + (long long)K * 3 * i, gH);
-            if (out.opacity) {
-                if constexpr (VD) store_n<K>(out.opacity + (long long)K * i, gHa);
-                else out.opacity[i] = gHa[0];
+        if (mine) {
+            if (out.means) { out.means[3 * i] = gp[0]; out.means[3 * i + 1] = gp[1]; out.means[3 * i + 2] = gp[2]; }
+            if (out.log_scales) {
+                out.log_scales[3 * i] = gls[0]; out.log_scales[3 * i + 1] = gls[1]; out.log_scales[3 * i + 2] = gls[2];
+            }
+            if (out.quats) store_n<4>(out.quats + 4 * i, gq);
+            if (out.lc_v) out.lc_v[i] = glcv;
+            if (ONE && ROWS && !sh_done) put_g(zero_h, zero_a);         // a view that added nothing
+            if constexpr (!ROWS) {
+                if (out.sh) store_n<3 * K>(out.sh + 3ll * K * i, rgh);
+                if (out.opacity) store_n<KA>(out.opacity + (long long)KA * i, rga);
             }
         }
-        if (out.lc_v) out.lc_v[i] = glcv;
-    };
-    if (det_sb == nullptr) {
-        const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (i < g.n) body(i);
-    } else {
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.n;
-             i += (long long)gridDim.x * blockDim.x)
-            body(i);
+        if constexpr (ROWS) {
+            __syncthreads();
+            if (out.sh) rows_out<3 * K>(out.sh + 3ll * K * i0, s_gh, cnt);
+            if (out.opacity) rows_out<KA>(out.opacity + (long long)KA * i0, s_ga, cnt);
+            __syncthreads();                // the rows are read
+        }
     }
     // global weight parameters: warp reduce, then one atomic per warp, or (deterministic) the block's sums
     // in warp order
@@ -560,11 +698,27 @@ cudaError_t project_t(const GaussPtrs& g, const Views& vs, WeightDev w, float* r
 template <int DEG, bool VD, bool RED>
 cudaError_t project_bwd_t(const GaussPtrs& g, const Views& vs, WeightDev w, const float* grec,
                           const wsr_grads& out, float* det_sb, cudaStream_t s) {
-    const int bs = 128;
+    constexpr int bs = 128, K = (DEG + 1) * (DEG + 1);
     long long nb = (g.n + bs - 1) / bs;
     if (det_sb && nb > kDetSBBlocks) nb = kDetSBBlocks;    // one sigma/beta slot per block
-    if (vs.n == 1) k_project_bwd<DEG, VD, RED, true><<<(unsigned)nb, bs, 0, s>>>(g, vs, w, grec, out, det_sb);
-    else k_project_bwd<DEG, VD, RED, false><<<(unsigned)nb, bs, 0, s>>>(g, vs, w, grec, out, det_sb);
+    // the shared-memory opt-in is a per-device function attribute: set once per device (thread-safe)
+    constexpr int rows = DEG < 2 ? 0 : sizeof(float) * bs * (Rows<3 * K>::P + Rows<VD ? K : 1>::P);
+    static std::once_flag once[64];
+    static cudaError_t once_err[64];
+    int dev = 0;
+    cudaError_t e0 = cudaGetDevice(&dev);
+    if (e0 != cudaSuccess) return e0;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::call_once(once[dev], [&] {
+        once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, rows);
+        if (once_err[dev] == cudaSuccess)
+            once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, false>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * rows);
+    });
+    if (once_err[dev] != cudaSuccess) return once_err[dev];
+    if (vs.n == 1) k_project_bwd<DEG, VD, RED, true><<<(unsigned)nb, bs, rows, s>>>(g, vs, w, grec, out, det_sb);
+    else k_project_bwd<DEG, VD, RED, false><<<(unsigned)nb, bs, 2 * rows, s>>>(g, vs, w, grec, out, det_sb);
     if (det_sb) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
