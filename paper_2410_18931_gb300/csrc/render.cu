@@ -813,28 +813,32 @@ __global__ void __launch_bounds__(256) k_det_bg_reduce(const float* __restrict__
     }
 }
 
-// Grid of a launch: one block per tile, or, persistent, as many blocks as
-// fit on the device at once.
+// As many blocks as fit on the device at once, kept in `known` (one per kernel).
 template <typename K>
-unsigned grid_for(K kernel, int threads, const Views& vs, const Sched& sched) {
-    if (!sched.order) return (unsigned)vs.total_tiles;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
-    return (unsigned)min(max(1, sms * max(per_sm, 1)), vs.total_tiles);
+cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks) {
+    return known.get(blocks, [&](int dev, int& out) {
+        int sms = 0, per_sm = 0;
+        cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+        out = max(1, sms * max(per_sm, 1));
+        return e;
+    });
 }
 
 template <int TW, int TH, int S>
 cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
     constexpr int NT = 32 * S * FwdShape<TW, TH>::NR;
-    const unsigned grid = grid_for(k_render_fwd<TW, TH, S>, NT, vs, sched);
+    static PerDevice known;
+    int grid = vs.total_tiles;
     if (sched.order) {
-        cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
+        int most = 0;
+        cudaError_t e = resident_blocks(known, k_render_fwd<TW, TH, S>, NT, most);
+        if (e == cudaSuccess) e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
+        grid = min(grid, most);
     }
-    k_render_fwd<TW, TH, S><<<grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb, den,
+    k_render_fwd<TW, TH, S><<<(unsigned)grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb, den,
                                                 sched.order, sched.counter);
     return cudaGetLastError();
 }
@@ -854,14 +858,14 @@ cudaError_t bwd_chunk(const float* rec, const unsigned* off, const unsigned* lis
                       float* bg_tiles, const unsigned* det_pmax, const BwdSched& sched, cudaStream_t s) {
     constexpr int NT = BwdThreads<CH>::value;
     auto kernel = det ? k_render_bwd<TW, TH, CH, true> : k_render_bwd<TW, TH, CH, false>;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NT, 0);
-    const long long most = (long long)max(sms, 1) * max(per_sm, 1), want = 4ll * vs.total_tiles;
-    cudaError_t e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned) * ((size_t)vs.total_tiles + 1), s);
+    static PerDevice known[2];
+    int most = 0;
+    cudaError_t e = resident_blocks(known[det], kernel, NT, most);
     if (e != cudaSuccess) return e;
-    kernel<<<(unsigned)min(most, want), NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb,
+    const long long want = 4ll * vs.total_tiles;
+    e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned) * ((size_t)vs.total_tiles + 1), s);
+    if (e != cudaSuccess) return e;
+    kernel<<<(unsigned)min((long long)most, want), NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb,
                                                     den, grgb, grec, gw, bg_tiles, det_pmax, sched.order,
                                                     sched.counter, sched.counter + 1,
                                                     vs.total_tiles <= kFewTiles ? 1u : kPartChunks);
@@ -1002,6 +1006,13 @@ __global__ void __launch_bounds__(256) k_loss_l1(const float* __restrict__ rgb, 
 
 }  // namespace
 
+cudaError_t sm_count(int& sms) {
+    static PerDevice known;
+    return known.get(sms, [](int dev, int& out) {
+        return cudaDeviceGetAttribute(&out, cudaDevAttrMultiProcessorCount, dev);
+    });
+}
+
 cudaError_t launch_render_fwd(const float* rec, const unsigned* off, const unsigned* list, const Views& vs,
                               WeightDev w, float* rgb, float* den, Sched sc, cudaStream_t s) {
     if (vs.total_tiles == 0) return cudaSuccess;
@@ -1032,9 +1043,8 @@ cudaError_t launch_det_pmax(const float* out_rgb, const float* out_den, const fl
                             unsigned* pmax, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(pmax, 0, sizeof(unsigned), s);
     if (e != cudaSuccess || npix == 0) return e;
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    e = sm_count(sms);
     if (e != cudaSuccess) return e;
     const long long blocks = min((npix + 255) / 256, (long long)sms * 8);
     k_det_pmax<<<(unsigned)blocks, 256, 0, s>>>(out_rgb, out_den, grad_rgb, npix, pmax);
@@ -1063,9 +1073,8 @@ cudaError_t launch_loss_l1(const float* rgb, const float* target, long long coun
                            cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), s);
     if (e != cudaSuccess || count == 0) return e;
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    e = sm_count(sms);
     if (e != cudaSuccess) return e;
     long long nb = (count / 4 + 255) / 256;
     const long long cap = 4ll * sms;

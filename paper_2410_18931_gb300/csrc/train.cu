@@ -388,9 +388,8 @@ cudaError_t launch_adam(float* p, const float* g, float* m, float* v, const Adam
     if (e != cudaSuccess) return e;
     const long long units = G.ubase[G.n];
     if (units == 0) return cudaSuccess;
-    int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0;
+    e = sm_count(sms);
     if (e != cudaSuccess) return e;
     const long long want = (units + 255) / 256;
     const long long cap = (long long)sms * 8;

@@ -1,11 +1,35 @@
 // Host-side launch interface between the C ABI (api.cu) and the kernels.
 #pragma once
 
+#include <atomic>
+
 #include <cuda_runtime.h>
 
 #include "wsr_common.cuh"
 
 namespace wsr {
+
+// What a launcher asks the runtime for once per kernel and device: a number that does not change afterwards (SMs,
+// resident blocks), kept per device (0: not asked yet; two threads may both ask and store the same).
+struct PerDevice {
+    std::atomic<int> value[64] = {};
+    template <typename F>
+    cudaError_t get(int& out, F&& ask) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= 64) return ask(dev, out);
+        out = value[dev].load(std::memory_order_relaxed);
+        if (out == 0) {
+            e = ask(dev, out);
+            if (e == cudaSuccess) value[dev].store(out, std::memory_order_relaxed);
+        }
+        return e;
+    }
+};
+
+// SMs of the current device.
+cudaError_t sm_count(int& sms);
 
 struct GaussPtrs {
     long long n;

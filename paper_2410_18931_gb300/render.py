@@ -18,12 +18,15 @@ _DT = {torch.float32: A.WSR_F32, torch.float16: A.WSR_F16, torch.bfloat16: A.WSR
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """The stream's handle.  The current stream's is asked for directly: a ``torch.cuda.Stream`` made for every call
+    costs 2.9 us against 0.3, and the smallest frames make four or five calls of about 10 us each."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 @dataclass
