@@ -345,6 +345,9 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
     float* const s_a = s_h + 128 * PH;                          // opacity likewise
     float* const s_gh = ONE ? s_h : s_a + 128 * PA;             // gradients
     float* const s_ga = ONE ? s_a : s_gh + 128 * PH;
+    // deterministic mode: a view's records (27 words used of 32), 28 words apart: 67 -> 44 us for 250k Gaussians
+    // against a record per thread in global memory
+    float* const s_det = ROWS ? s_ga + 128 * PA : s_rows;
     float gsig = 0.0f, gbeta = 0.0f;
     const float sigma = __ldg(wd.params + 0), beta = __ldg(wd.params + 1);
     // det_sb != nullptr: deterministic mode (fixed-point records, a bounded grid striding over the
@@ -378,7 +381,16 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
             rb = __ldg(r + 1);
             rc = __ldg(reinterpret_cast<const float*>(r + 2));
         };
-        if (mine && det_sb == nullptr) load_record(0);
+        auto copy_det = [&](int v) {
+            const uint4* from = reinterpret_cast<const uint4*>(grec) + 8ll * ((long long)v * g.n + i0);
+            for (int c = threadIdx.x; c < 7 * cnt; c += 128) {
+                float* const o = s_det + 4 * c;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(o)),
+                             "l"(from + (c / 7 * 8 + c % 7)) : "memory");
+            }
+        };
+        if (det_sb) copy_det(0);
+        else if (mine) load_record(0);
         auto get_h = [&](float (&h)[3 * K], float (&ha)[KA]) {
             if constexpr (ROWS) {
                 row_get<3 * K, sh_t>(s_h + PH * threadIdx.x, h);
@@ -414,7 +426,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
         };
         const float zero_h[3 * K] = {}, zero_a[KA] = {};
         if constexpr (!ONE || !ROWS) put_g(zero_h, zero_a);
-        if constexpr (ROWS) {
+        if (ROWS || det_sb) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
         }
@@ -428,9 +440,15 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
         bool sh_done = false;           // ONE: the rows hold the gradients
 
         const int nv = ONE ? 1 : vs.n;
-        for (int v = 0; mine && v < nv; ++v) {
+        for (int v = 0; v < nv; ++v) {
+            if (det_sb && v > 0) {
+                __syncthreads();                // the last view's records are read
+                copy_det(v);
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncthreads();
+            }
+            if (!mine) continue;
             const View& V = vs.v[v];
-            const float* const gr = grec + (det_sb ? kDetRecordFloats : WSR_GRAD_RECORD_FLOATS) * ((long long)v * g.n + i);
             float g9[9];
             bool any = false;
             if (det_sb == nullptr) {
@@ -442,16 +460,17 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
                 for (int e = 0; e < 9; ++e) any |= (g9[e] != 0.0f);
             } else {
                 // 9 int64 sums in units of 2^(e - kDetBits), 2^e above the term's bound (stored beside them)
+                const float* const gr = s_det + 28 * threadIdx.x;
                 const long long* sums = reinterpret_cast<const long long*>(gr);
                 const int* mag = reinterpret_cast<const int*>(gr + 18);
 #pragma unroll
                 for (int c = 0; c < 9; ++c) {
-                    const float m = __int_as_float(__ldg(mag + c));
+                    const float m = __int_as_float(mag[c]);
                     float val = 0.0f;
                     if (m > 0.0f) {
                         int e;
                         frexpf(m, &e);
-                        val = (float)ldexp((double)__ldg(sums + c), e - kDetBits);
+                        val = ldexpf(__ll2float_rn(sums[c]), e - kDetBits);
                     }
                     g9[c] = val;
                     any |= (val != 0.0f);
@@ -641,8 +660,8 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
             __syncthreads();
             if (out.sh) rows_out<3 * K>(out.sh + 3ll * K * i0, s_gh, cnt);
             if (out.opacity) rows_out<KA>(out.opacity + (long long)KA * i0, s_ga, cnt);
-            __syncthreads();                // the rows are read
         }
+        if (ROWS || det_sb) __syncthreads();    // the rows and records are read
     }
     // global weight parameters: warp reduce, then one atomic per warp, or (deterministic) the block's sums
     // in warp order
@@ -671,18 +690,26 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
 
 // Deterministic mode: the blocks' sigma/beta sums added in block order.
 __global__ void __launch_bounds__(256) k_det_sb_reduce(const float* __restrict__ sb, int nb, float* __restrict__ gw) {
-    __shared__ float part[2][256];
+    __shared__ float part[2][8];
     float a0 = 0.0f, a1 = 0.0f;
     for (int b = threadIdx.x; b < nb; b += 256) {
         a0 += sb[2 * b];
         a1 += sb[2 * b + 1];
     }
-    part[0][threadIdx.x] = a0;
-    part[1][threadIdx.x] = a1;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a0 += __shfl_xor_sync(0xffffffffu, a0, off);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        part[0][threadIdx.x >> 5] = a0;
+        part[1][threadIdx.x >> 5] = a1;
+    }
     __syncthreads();
     if (threadIdx.x < 2) {
         float t = 0.0f;
-        for (int k = 0; k < 256; ++k) t += part[threadIdx.x][k];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t += part[threadIdx.x][k];
         gw[threadIdx.x] = t;
     }
 }
@@ -700,9 +727,12 @@ cudaError_t project_bwd_t(const GaussPtrs& g, const Views& vs, WeightDev w, cons
                           const wsr_grads& out, float* det_sb, cudaStream_t s) {
     constexpr int bs = 128, K = (DEG + 1) * (DEG + 1);
     long long nb = (g.n + bs - 1) / bs;
-    if (det_sb && nb > kDetSBBlocks) nb = kDetSBBlocks;    // one sigma/beta slot per block
+    // one sigma/beta slot per block, and the blocks that fit on the device at once: 608 at four per SM
+    if (det_sb && nb > kDetBlocks) nb = kDetBlocks;
     // the shared-memory opt-in is a per-device function attribute: set once per device (thread-safe)
     constexpr int rows = DEG < 2 ? 0 : sizeof(float) * bs * (Rows<3 * K>::P + Rows<VD ? K : 1>::P);
+    constexpr int det_rows = sizeof(float) * bs * 28;
+    const int more = det_sb ? det_rows : 0;
     static std::once_flag once[64];
     static cudaError_t once_err[64];
     int dev = 0;
@@ -711,14 +741,15 @@ cudaError_t project_bwd_t(const GaussPtrs& g, const Views& vs, WeightDev w, cons
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::call_once(once[dev], [&] {
         once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, rows);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, rows + det_rows);
         if (once_err[dev] == cudaSuccess)
             once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, false>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * rows);
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 2 * rows + det_rows);
     });
     if (once_err[dev] != cudaSuccess) return once_err[dev];
-    if (vs.n == 1) k_project_bwd<DEG, VD, RED, true><<<(unsigned)nb, bs, rows, s>>>(g, vs, w, grec, out, det_sb);
-    else k_project_bwd<DEG, VD, RED, false><<<(unsigned)nb, bs, 2 * rows, s>>>(g, vs, w, grec, out, det_sb);
+    if (vs.n == 1) k_project_bwd<DEG, VD, RED, true><<<(unsigned)nb, bs, rows + more, s>>>(g, vs, w, grec, out, det_sb);
+    else k_project_bwd<DEG, VD, RED, false><<<(unsigned)nb, bs, 2 * rows + more, s>>>(g, vs, w, grec, out, det_sb);
     if (det_sb) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

@@ -386,6 +386,28 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// x 2^s rounded to the nearest integer (halves to even), as __double2ll_rn(ldexp((double)x, s)) gives it, from the
+// float's bits: the deterministic mode forms nine of them per Gaussian and tile, and the double-precision pipe is 64
+// times slower than the others.  With the sums added by consecutive lanes: 237 -> 185 us for 250k Gaussians at
+// 1280x720 (each lane adding its Gaussian's nine words took 237 us with either conversion).
+__device__ __forceinline__ long long fixed_point(const float x, const int s) {
+    const unsigned bits = __float_as_uint(x);
+    const int ex = (int)((bits >> 23) & 0xffu);
+    if (ex == 0xff) return __double2ll_rn(ldexp((double)x, s));         // infinities and NaN
+    const unsigned m = (bits & 0x7fffffu) | (ex ? 0x800000u : 0u);
+    const int sh = (ex ? ex : 1) - 150 + s;                             // |x| 2^s = m 2^sh
+    long long q;
+    if (sh >= 0) {
+        if (sh > 38) return __double2ll_rn(ldexp((double)x, s));        // beyond 2^62
+        q = (long long)((unsigned long long)m << sh);
+    } else {
+        const int n = min(-sh, 31);                                     // from 26 on everything rounds to zero
+        const unsigned r = m >> n, rest = m & ((1u << n) - 1u), half = 1u << (n - 1);
+        q = (long long)(r + ((rest > half || (rest == half && (r & 1u))) ? 1u : 0u));
+    }
+    return (bits >> 31) ? -q : q;
+}
+
 // Backward, one block per tile, a group of lanes per Gaussian.
 //
 // The tile's pixel terms P = (G/D, -(G.C)/D) sit in shared memory by column
@@ -436,6 +458,7 @@ constexpr float kMagic = 12582912.0f;       // 1.5 x 2^23
 constexpr int kFewWalk = 64;
 // Chunks per part of a tile's list (1 for few tiles): claiming each chunk on its own costs 20 us at 1M Gaussians.
 constexpr unsigned kPartChunks = 4;
+constexpr int kNoBound = 127;               // deterministic mode: a bound of zero (frexpf gives at most 100 here)
 constexpr int kHelpTiles = 1024;            // tiles whose chunks idle blocks look for (a power of two)
 
 // Schedule: as many blocks as fit on the device take the tiles through *counter (in the order given, longest first,
@@ -483,6 +506,10 @@ __global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::
     __shared__ unsigned shist[NK];
     __shared__ unsigned snext[2];               // per class: the next position of the order a warp takes
     __shared__ float4 sbg[NW];                  // background terms per warp
+    // deterministic mode: a warp's Gaussians' sums on their way out, the exponents of their bounds, their records
+    __shared__ float s_val[DET ? NW : 1][DET ? 32 : 1][9];
+    __shared__ signed char s_exp[DET ? NW : 1][DET ? 32 : 1][9];
+    __shared__ unsigned s_rec[DET ? NW : 1][DET ? 32 : 1];
     __shared__ int4 s_cur;                      // the tile (-1: none left) and its ends
     __shared__ unsigned s_part;
 
@@ -715,41 +742,59 @@ __global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::
                         for (int off = LT / 2; off > 0; off >>= 1)
 #pragma unroll
                             for (int c = 0; c < 9; ++c) vals[c] += __shfl_xor_sync(0xffffffffu, vals[c], off);
-                        if (act && lane % LT == 0 && steps > 0) {
-                            if constexpr (!DET) {
+                        const bool add = act && lane % LT == 0 && steps > 0;        // the group's lane with its sums
+                        if constexpr (!DET) {
+                            if (add) {
                                 float4* o = reinterpret_cast<float4*>(grec + (size_t)WSR_GRAD_RECORD_FLOATS * sidx[j]);
                                 atomicAdd(o, make_float4(vals[0], vals[1], vals[2], vals[3]));
                                 atomicAdd(o + 1, make_float4(vals[4], vals[5], vals[6], vals[7]));
                                 atomicAdd(reinterpret_cast<float*>(o + 2), vals[8]);
-                            } else {
-                                // deterministic mode: a 128-byte record holds 9 int64 sums, then the 9 bounds (float
-                                // bits) that fix their units.  A term's bound caps the sum of its absolute pixel
-                                // terms over the whole footprint, the same in every tile of the Gaussian: at most
-                                // (2 hx + 2)(2 hy + 2) pixels (hx, hy its half-extents), each with e <= 1, every
-                                // pixel-table entry at most pmax, |r| <= sqrt(QM), |dx| <= hx inside the cutoff.
-                                float* o = grec + (size_t)kDetRecordFloats * sidx[j];
-                                int* mag = reinterpret_cast<int*>(o + 18);
+                            }
+                        } else {
+                            // deterministic mode: a 128-byte record holds 9 int64 sums, then the 9 bounds (float
+                            // bits) that fix their units.  A term's bound caps the sum of its absolute pixel
+                            // terms over the whole footprint, the same in every tile of the Gaussian: at most
+                            // (2 hx + 2)(2 hy + 2) pixels (hx, hy its half-extents), each with e <= 1, every
+                            // pixel-table entry at most pmax, |r| <= sqrt(QM), |dx| <= hx inside the cutoff.
+                            // The sums go out through shared memory, so that consecutive lanes form and add consecutive
+                            // words of a record.
+                            if (add) {
                                 constexpr float QM = kQMax * 1.0001f + 1e-4f;
                                 const float qd = b.x, hx = sqrtf(QM / qd);
                                 const float hy = sqrtf(QM * fmaf(a.w, a.w, qd) / (qd * a.z * a.z));
                                 const float npx = fminf((2.0f * hx + 2.0f) * (2.0f * hy + 2.0f), 1e12f);
                                 const float gqm = pmax * kLn2 * 1.0001f * (fabsf(b.z) + fabsf(b.w) + fabsf(c2.x) + fabsf(b.y));
                                 const float sq = sqrtf(QM);
-                                const float bound[9] = {npx * gqm * sq, npx * gqm * hx, npx * gqm * QM, npx * gqm * sq * hx,
-                                                        npx * gqm * hx * hx, npx * pmax, npx * pmax, npx * pmax, npx * pmax};
-                                unsigned long long* sum = reinterpret_cast<unsigned long long*>(o);
+                                float* const o = grec + (size_t)kDetRecordFloats * sidx[j] + 18;
+                                auto bound = [&](int c, float m) {
+                                    m = fminf(m, 1e30f);
+                                    int e = kNoBound;
+                                    if (m > 0.0f) frexpf(m, &e);    // m < 2^e
+                                    s_exp[warp][grp][c] = (signed char)e;
+                                    return m;
+                                };
 #pragma unroll
-                                for (int c = 0; c < 9; ++c) {
-                                    const float m = fminf(bound[c], 1e30f);
-                                    mag[c] = __float_as_int(m);     // every tile of the Gaussian writes the same value
-                                    if (m > 0.0f) {
-                                        int e;
-                                        frexpf(m, &e);              // m < 2^e
-                                        const long long q = __double2ll_rn(ldexp((double)vals[c], kDetBits - e));
-                                        atomicAdd(sum + c, (unsigned long long)q);
-                                    }
-                                }
+                                for (int c = 0; c < 9; ++c) s_val[warp][grp][c] = vals[c];
+                                // every tile of the Gaussian writes the same bounds (and a zero in the padding)
+                                *reinterpret_cast<float2*>(o) = f2(bound(0, npx * gqm * sq), bound(1, npx * gqm * hx));
+                                *reinterpret_cast<float4*>(o + 2) = make_float4(bound(2, npx * gqm * QM),
+                                                                                bound(3, npx * gqm * sq * hx),
+                                                                                bound(4, npx * gqm * hx * hx),
+                                                                                bound(5, npx * pmax));
+                                const float m = bound(6, npx * pmax);
+                                *reinterpret_cast<float4*>(o + 6) = make_float4(m, bound(7, npx * pmax), bound(8, npx * pmax),
+                                                                                0.0f);
                             }
+                            if (lane % LT == 0) s_rec[warp][grp] = add ? sidx[j] : 0xffffffffu;
+                            __syncwarp();
+                            for (int k = lane; k < 9 * GW; k += 32) {
+                                const int gi = k / 9, c = k - 9 * gi, e = s_exp[warp][gi][c];
+                                const unsigned ri = s_rec[warp][gi];
+                                if (ri != 0xffffffffu && e != kNoBound)
+                                    atomicAdd(reinterpret_cast<unsigned long long*>(grec + (size_t)kDetRecordFloats * ri) + c,
+                                              (unsigned long long)fixed_point(s_val[warp][gi][c], kDetBits - e));
+                            }
+                            __syncwarp();
                         }
                     }
                 };
@@ -798,17 +843,26 @@ __global__ void __launch_bounds__(256) k_det_pmax(const float* __restrict__ out_
 // Deterministic mode: the tiles' background terms summed in a fixed order.
 __global__ void __launch_bounds__(256) k_det_bg_reduce(const float* __restrict__ bg, int n_tiles,
                                                        float* __restrict__ gw) {
-    __shared__ float part[4][256];
+    __shared__ float part[4][8];
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int t = threadIdx.x; t < n_tiles; t += 256)
+#pragma unroll 8
+    for (int t = threadIdx.x; t < n_tiles; t += 256) {
+        const float4 v = reinterpret_cast<const float4*>(bg)[t];
+        acc[0] += v.x;
+        acc[1] += v.y;
+        acc[2] += v.z;
+        acc[3] += v.w;
+    }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[c] += bg[4 * (size_t)t + c];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) part[c][threadIdx.x] = acc[c];
+    for (int c = 0; c < 4; ++c) {
+        const float t = warp_sum(acc[c]);
+        if ((threadIdx.x & 31) == 0) part[c][threadIdx.x >> 5] = t;
+    }
     __syncthreads();
     if (threadIdx.x < 4) {
         float sum = 0.0f;
-        for (int k = 0; k < 256; ++k) sum += part[threadIdx.x][k];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum += part[threadIdx.x][k];
         gw[2 + threadIdx.x] = sum;
     }
 }

@@ -63,7 +63,8 @@ struct WsHeader {
 
 constexpr size_t kWsHeader = 8192;
 constexpr size_t kWsDetSB = 256;       // deterministic mode: sigma/beta per projection-backward block
-constexpr int kDetSBBlocks = (int)((kWsHeader - kWsDetSB) / (2 * sizeof(float)));   // 992
+constexpr int kDetBlocks = 608;        // most of them
+static_assert(kDetBlocks <= (int)((kWsHeader - kWsDetSB) / (2 * sizeof(float))), "sigma/beta sums in the header");
 // Deterministic mode: a record term is added as 64-bit fixed point in units of
 // 2^(e - kDetBits), 2^e above an a-priori bound on the sum of the absolute
 // values of all its partials (over every tile of the Gaussian), so the exact

@@ -51,7 +51,7 @@ struct WeightDev {
 
 cudaError_t launch_project(const GaussPtrs& g, const Views& vs, WeightDev w, float* records,
                            cudaStream_t s);
-// det_sb: nullptr, or (deterministic mode) room for kDetSBBlocks pairs of sigma/beta block sums; the
+// det_sb: nullptr, or (deterministic mode) room for kDetBlocks pairs of sigma/beta block sums; the
 // records are then WSR_GRAD_RECORD_FLOATS_DET floats of fixed-point sums and their scales
 cudaError_t launch_project_bwd(const GaussPtrs& g, const Views& vs, WeightDev w,
                                const float* grad_records, const wsr_grads& out, float* det_sb, cudaStream_t s);

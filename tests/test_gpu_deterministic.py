@@ -157,3 +157,34 @@ def test_deterministic_fixed_point_sums_stay_inside_their_bounds(tile):
     val = np.ldexp(sums[touched].astype(np.float64), e - 60)
     assert np.all(np.abs(val) <= bounds[touched].astype(np.float64) * (1 + 1e-6))
     assert np.all(sums[~touched] == 0)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 255, 256, 257, 512, 513, 1024, 1025, 2048, 2049, 4096, 4097, 8191, 8192])
+def test_lists_of_every_sort_size_are_sorted(n):
+    """Stacks of n Gaussians on one tile, and a list of another size on a tile of the same block of the sort: the
+    lists of the default mode, sorted by record index (a warp per list up to 1024 entries, then the block)."""
+    import torch
+
+    from paper_2410_18931_gb300 import Gaussians, Renderer
+    other = 300
+    sc = ws.random_scene(n + other, 3, sh_degree=0, vd_opacity=False, box=1e-4, log_scale_mu=-9.0, log_scale_sd=0.1)
+    rng = np.random.default_rng(n)
+    first = np.zeros(n + other, bool)
+    first[rng.permutation(n + other)[:n]] = True
+    sc.means[~first, 0] += 0.5                  # a few tiles away, mixed into the record order
+    cam = ws.look_at((0.0, 0.0, -3.0), width=128, height=64)
+    cam.cx, cam.cy = 72.0, 24.0                 # both stacks in the middle of a tile, 48 pixels apart
+    cam.fx = cam.fy = 3.0 / 0.5 * 48.0
+    cam = cam.rounded()
+    w = ws.default_weight(ws.EXP)
+    g = Gaussians.from_scene(sc)
+    wpar = torch.tensor(w.as_array(), device="cuda")
+    r = Renderer([cam], tile=(16, 16), deterministic=True)
+    st = r.forward(g, w.kind, wpar)
+    off, lst = st.tile_offsets.cpu().numpy(), st.tile_list.cpu().numpy()
+    sizes = sorted(int(x) for x in np.diff(off) if x)
+    assert sizes == sorted((n, other))
+    for t in np.nonzero(np.diff(off))[0]:
+        seg = lst[off[t]:off[t + 1]]
+        want = np.nonzero(first if first[seg[0]] else ~first)[0]
+        assert np.array_equal(seg, want)
