@@ -499,22 +499,17 @@ wsr_status wsr_loss_3dgs(const float* rgb, const float* target, const wsr_camera
     if (!(lambda >= 0.0f && lambda <= 1.0f)) return WSR_ERR_INVALID_ARG;
     static thread_local LossViews L;
     memset(&L, 0, sizeof L);
-    const int side = loss_tile_side();
-    long long tiles = 0, pix = 0;
+    long long pix = 0;
     L.n = n_cams;
     for (int v = 0; v < n_cams; ++v) {
         const int W = cams[v].width, H = cams[v].height;
         if (W <= 0 || H <= 0 || W > 32768 || H > 32768) return WSR_ERR_INVALID_ARG;
         L.w[v] = W;
         L.h[v] = H;
-        L.tiles_x[v] = (W + side - 1) / side;
-        L.tile_off[v] = (int)tiles;
         L.pix_off[v] = pix;
-        tiles += (long long)L.tiles_x[v] * ((H + side - 1) / side);
         pix += (long long)W * H;
-        if (tiles > (1ll << 30)) return WSR_ERR_INVALID_ARG;
     }
-    L.tile_off[n_cams] = (int)tiles;
+    if (!loss_plan(L)) return WSR_ERR_INVALID_ARG;
     // the normalised 11-tap Gaussian of standard deviation 1.5
     double g[11], sum = 0.0;
     for (int k = 0; k < 11; ++k) sum += (g[k] = exp(-(double)((k - 5) * (k - 5)) / (2.0 * 1.5 * 1.5)));

@@ -2,15 +2,13 @@
 // trains with (Sec. 4.4: L1 + 0.2 D-SSIM) with its gradient, and the Adam
 // update of the parameters.
 //
-// Loss.  One block per 32 x 32 output tile of one view.  For each channel the
-// block stages the rendered and target pixels of the tile plus a 10-pixel
-// halo in shared memory (zero outside the image), filters the five local
-// statistics (mu_x, mu_y, E[x^2], E[y^2], E[xy]) separably with the 11-tap
-// Gaussian over the tile plus a 5-pixel halo, forms the SSIM map and the three
-// partials of the loss with respect to (mu_x, E[x^2], E[xy]), and filters
-// those back (the window is symmetric, so the filter is its own adjoint) to
-// the gradient of the tile's pixels.  L1 and SSIM sums go to the loss with
-// one atomic per block and quantity.
+// Loss.  A block per strip of pixel columns and segment of rows of one view
+// filters the local statistics (mu_x, mu_y, E[x^2 + y^2], E[xy]) separably
+// with the 11-tap Gaussian (zero outside the image), forms the SSIM map and
+// the three partials of the loss with respect to (mu_x, E[x^2], E[xy]), and
+// filters those back (the window is symmetric, so the filter is its own
+// adjoint) to the gradient of the segment's pixels.  L1 and SSIM sums go to the
+// loss with one atomic per block and quantity.
 //
 // Adam.  One pass over a flat parameter buffer in float4 units, groups of
 // contiguous elements with their own learning rates.  The step count and the
@@ -26,28 +24,29 @@
 namespace wsr {
 namespace {
 
-constexpr int kR = 5;                       // window radius: 11 taps
-constexpr int kLT = 32;                     // output tile side
-constexpr int kIn = kLT + 4 * kR;           // staged input side (52)
-constexpr int kSt = kLT + 2 * kR;           // statistics side (42)
+// Loss: the images are taken as rows of 3 W floats (the channels interleaved, as stored).  A block walks down a strip
+// of kOP pixel columns, kTap rows at a time:
+//   1. a thread per staged float column reads its next rows (coalesced) and filters x, y, x^2 + y^2 and (x - y)^2
+//      vertically, eleven partial sums per quantity in registers.  SSIM's factor (2 cov + c2) / (var + var + c2) is
+//      1 - D / (var + var + c2) with D the variance of x - y, so these four are enough, and where the images are
+//      alike the cancellation in the variances hardly reaches it (gradient against 64 bits on smooth images: 1.3e-5
+//      relative with the covariance, 1.1e-5 so; on noise 1.3e-7 either way);
+//   2. the rows' horizontal filter, five neighbouring pixels of a channel per item, gives the statistics; the SSIM map
+//      and its three partials follow;
+//   3. a thread per statistics column filters the partials vertically, as in 1;
+//   4. their horizontal filter, as in 2; 5. the gradient, a thread per output column.
+// The strip's halo is 20 pixel columns (85 for 65) and the segment's 20 rows, where a 32x32 tile needed 52x52 staged
+// pixels, staged through shared memory once per channel.  Bound by instruction issue (61 % of the cycles of two blocks
+// of eight warps, the rest the batch's five barriers): a filter's tap on two quantities is one instruction, and the
+// instructions fell from 9.4e7 to 6.8e7 at 1920x1080.  Tiles -> strips, us: 1080p 127 -> 96, 720p 66 -> 56,
+// 979x543 43 -> 40, 640x360 24.7 -> 24.5, 320x180 18.1 -> 16.5, 3840x2160 474 -> 352.
+constexpr int kTap = 11;                    // taps of the window, and rows per batch
+constexpr int kOP = 65, kTP = kOP + 10, kSP = kOP + 20;     // output, statistics and staged pixels of a strip
+constexpr int kVW = 91, kPW = 75;           // pixels per channel and row in shared memory (3 mod 8: a thread per
+                                            // column writes three channels side by side without bank conflicts)
 constexpr int kLossThreads = 256;
-constexpr int kStage = (kIn * kIn + kLossThreads - 1) / kLossThreads;   // staged pixels per thread
-// Shared memory, in floats: the staged (rendered, target) pairs, then the horizontally filtered
-// statistics as (mu_x, mu_y) and (E[x^2], E[y^2]) pairs and E[xy].  The loss partials with
-// respect to (mu_x, E[x^2]) as pairs and E[xy] reuse the staged pixels (no longer needed after
-// the statistics); the filtered partials reuse the statistics.  The partials' rows are kMP
-// apart and the filtered partials' kFP apart (odd numbers of 8-byte words): the horizontal
-// pass reads them a row per lane, and its lanes then fall on distinct banks.
-constexpr int kMP = kSt + 1, kFP = kLT + 1;
-constexpr int kStatOff = ((3 * kSt * kMP > 2 * kIn * kIn ? 3 * kSt * kMP : 2 * kIn * kIn) + 3) / 4 * 4;
-constexpr int kLossSmemFloats = kStatOff + 5 * kIn * kSt;      // the statistics start at kStatOff
-static_assert(3 * kSt * kFP <= 5 * kIn * kSt, "layout");
-// register blocking of the four filter passes (outputs per item along the filtered axis)
-constexpr int kH1 = kSt / 3;                // horizontal statistics: 3 columns
-constexpr int kV2 = 7, kS2 = kSt / kV2;     // vertical statistics: 7 rows
-constexpr int kH3 = 4, kB3 = kLT / kH3;     // horizontal partials: 4 columns
-constexpr int kV4 = 4, kS4 = kLT / kV4;     // vertical partials: 4 rows
-static_assert(kH1 * 3 == kSt && kS2 * kV2 == kSt && kB3 * kH3 == kLT && kS4 * kV4 == kLT, "exact blocking");
+constexpr int kLossSmem = (kTap * 3 * (kVW + kPW)) * (int)sizeof(float4);
+static_assert(3 * kSP <= kLossThreads && kTP % 5 == 0 && kOP % 5 == 0 && kVW >= kSP && kPW >= kTP, "layout");
 
 __device__ __forceinline__ float block_sum_to(float x, float* red) {
 #pragma unroll
@@ -61,222 +60,186 @@ __device__ __forceinline__ float block_sum_to(float x, float* red) {
     return t;   // valid in thread 0
 }
 
-// Every filter step runs on two quantities at once where it can (paired FP32 ops on float2):
-// the rendered and target values, their squares, and the first two loss partials; the cross
-// terms E[xy] and its partial go alone.
-__global__ void __launch_bounds__(kLossThreads, 3) k_loss_3dgs(const float* __restrict__ rgb,
+__global__ void __launch_bounds__(kLossThreads, 2) k_loss_3dgs(const float* __restrict__ rgb,
                                                                const float* __restrict__ tgt, const LossViews L,
                                                                float* __restrict__ loss, float* __restrict__ grad) {
-    extern __shared__ __align__(16) float sm[];
-    float2* sxy = reinterpret_cast<float2*>(sm);                   // [kIn][kIn] (rendered, target)
-    float2* h01 = reinterpret_cast<float2*>(sm + kStatOff);        // [kIn][kSt] filtered (x, y)
-    float2* h23 = h01 + kIn * kSt;                                 // [kIn][kSt] filtered (x^2, y^2)
-    float* h4 = reinterpret_cast<float*>(h23 + kIn * kSt);         // [kIn][kSt] filtered x y
-    float2* m01 = reinterpret_cast<float2*>(sm);                   // [kSt][kMP] partials: mu_x, E[x^2]
-    float* m2 = reinterpret_cast<float*>(m01 + kSt * kMP);         // [kSt][kMP] partial: E[xy]
-    float2* f01 = h01;                                             // [kSt][kFP] horizontally filtered
-    float* f2s = reinterpret_cast<float*>(f01 + kSt * kFP);        // [kSt][kFP]
+    extern __shared__ __align__(16) float4 sm[];
+    float4* const sv = sm;                          // [kTap][3][kVW] vertically filtered; at the end F of the outputs
+    float4* const sp = sm + kTap * 3 * kVW;         // [kTap][3][kPW] partials, then vertically filtered
     __shared__ float red[kLossThreads / 32];
     const int tid = threadIdx.x;
-
     int v = 0;
     while (v + 1 < L.n && (int)blockIdx.x >= L.tile_off[v + 1]) ++v;
     const int t = (int)blockIdx.x - L.tile_off[v];
     const int W = L.w[v], H = L.h[v];
-    const int x0 = (t % L.tiles_x[v]) * kLT, y0 = (t / L.tiles_x[v]) * kLT;
-    const long long base = L.pix_off[v];
+    const int seg = t / L.tiles_x[v], x0 = (t - seg * L.tiles_x[v]) * kOP;
+    const int r0 = seg * L.rows, rows = min(L.rows, H - r0);        // output rows r0 .. r0 + rows - 1
+    const float* const img = rgb + L.pix_off[v] * 3;
+    const float* const ref = tgt + L.pix_off[v] * 3;
+    float* const out = grad + L.pix_off[v] * 3;
     const float gs = -L.lam * L.inv_count;                 // dL / d(SSIM map value)
     const float gl1 = (1.0f - L.lam) * L.inv_count;        // dL / d|x - y|
+    const int px = tid / 3, ch = tid - 3 * px;             // this thread's column in steps 1, 3 and 5
+    const int in_x = x0 - 10 + px;
+    const bool in_col = px < kSP && in_x >= 0 && in_x < W;
+    const long long in_at = 3ll * in_x + ch;
+    const long long pitch = 3ll * W;
+    float g[kTap];
+#pragma unroll
+    for (int k = 0; k < kTap; ++k) g[k] = L.g[k];
+    // row q's partial sums lie in slot q mod 11; a batch's first row is a multiple of 11, so every slot is known here
+    float2 a01[kTap], a23[kTap], b01[kTap];
+    float b2[kTap];
+#pragma unroll
+    for (int k = 0; k < kTap; ++k) {
+        a01[k] = a23[k] = b01[k] = f2(0.f, 0.f);
+        b2[k] = 0.f;
+    }
     float l1 = 0.f, ss = 0.f;
-    float2 g2[2 * kR + 1];                                 // the window's taps, paired
+    const int batches = (rows + 20 + kTap - 1) / kTap;
+    // a batch's first rows are loaded before the last one's steps 4 and 5, the others while the first are filtered
+    constexpr int kAhead = 5;
+    float2 xy[kTap];
+    auto load_row = [&](int t) {
+        const int y = r0 - 10 + t;
+        if (!in_col || y < 0 || y >= H) return f2(0.f, 0.f);
+        return f2(__ldg(img + (y * pitch + in_at)), __ldg(ref + (y * pitch + in_at)));
+    };
 #pragma unroll
-    for (int k = 0; k < 2 * kR + 1; ++k) g2[k] = f2(L.g[k], L.g[k]);
-
-    for (int c = 0; c < 3; ++c) {
-        {
-            // all of a thread's loads first, then the stores: kStage independent loads in flight
-            float2 ab[kStage];
+    for (int i = 0; i < kAhead; ++i) xy[i] = load_row(i);
+    for (int b = 0; b < batches; ++b) {
+        const int t0 = kTap * b;                    // input row t is image row r0 - 10 + t
+        // ---- 1: input row t adds g[d] times itself to statistics row t - d; row t - 10 is then complete ----
 #pragma unroll
-            for (int k = 0; k < kStage; ++k) {
-                const int i = tid + k * kLossThreads;
-                const int iy = i / kIn, ix = i - iy * kIn;
-                const int gx = x0 - 2 * kR + ix, gy = y0 - 2 * kR + iy;
-                ab[k] = f2(0.f, 0.f);
-                if (i < kIn * kIn && gx >= 0 && gx < W && gy >= 0 && gy < H) {
-                    const long long p = (base + (long long)gy * W + gx) * 3 + c;
-                    ab[k] = f2(__ldg(rgb + p), __ldg(tgt + p));
-                }
+        for (int i = kAhead; i < kTap; ++i) xy[i] = load_row(t0 + i);
+#pragma unroll
+        for (int i = 0; i < kTap; ++i) {
+            const float2 x = xy[i];
+            const float dif = x.x - x.y;
+            const float2 m = f2(fmaf(x.x, x.x, x.y * x.y), dif * dif);
+#pragma unroll
+            for (int d = 0; d < kTap; ++d) {
+                const int k = (i - d + kTap) % kTap;
+                a01[k] = d == 0 ? __fmul2_rn(f2(g[0], g[0]), x) : __ffma2_rn(f2(g[d], g[d]), x, a01[k]);
+                a23[k] = d == 0 ? __fmul2_rn(f2(g[0], g[0]), m) : __ffma2_rn(f2(g[d], g[d]), m, a23[k]);
+            }
+            const int k = (i + 1) % kTap;
+            if (px < kSP) sv[(i * 3 + ch) * kVW + px] = make_float4(a01[k].x, a01[k].y, a23[k].x, a23[k].y);
+        }
+        __syncthreads();
+        // ---- 2: statistics row q (image row r0 - 5 + q), pixel j (image column x0 - 5 + j) ----
+        for (int it = tid; it < kTap * 3 * (kTP / 5); it += kLossThreads) {
+            const int i = it / (3 * (kTP / 5)), rest = it - i * (3 * (kTP / 5));
+            const int c = rest / (kTP / 5), j0 = 5 * (rest - c * (kTP / 5));
+            const int q = t0 + i - 10, y = r0 - 5 + q;
+            const bool row_in = q >= 0 && q < rows + 10 && y >= 0 && y < H;
+            float4* const dst = sp + (i * 3 + c) * kPW + j0;
+            if (!row_in) {
+#pragma unroll
+                for (int o = 0; o < 5; ++o) dst[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+                continue;
+            }
+            float2 s01[5], s23[5];
+#pragma unroll
+            for (int o = 0; o < 5; ++o) s01[o] = s23[o] = f2(0.f, 0.f);
+            const float4* const src = sv + (i * 3 + c) * kVW + j0;
+#pragma unroll
+            for (int k = 0; k < kTap + 4; ++k) {
+                const float4 w = src[k];
+#pragma unroll
+                for (int o = 0; o < 5; ++o)
+                    if (k - o >= 0 && k - o < kTap) {
+                        s01[o] = __ffma2_rn(f2(g[k - o], g[k - o]), f2(w.x, w.y), s01[o]);
+                        s23[o] = __ffma2_rn(f2(g[k - o], g[k - o]), f2(w.z, w.w), s23[o]);
+                    }
             }
 #pragma unroll
-            for (int k = 0; k < kStage; ++k) {
-                const int i = tid + k * kLossThreads;
-                if (i < kIn * kIn) sxy[i] = ab[k];
+            for (int o = 0; o < 5; ++o) {
+                const int x = x0 - 5 + j0 + o;
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (x >= 0 && x < W) {
+                    const float mx = s01[o].x, my = s01[o].y, md = mx - my, mm = fmaf(mx, mx, my * my);
+                    const float a1 = fmaf(2.f, mx * my, L.c1), b1 = mm + L.c1;
+                    const float b2_ = (s23[o].x - mm) + L.c2, a2 = b2_ - fmaf(-md, md, s23[o].y);
+                    const float ib1 = rcp_approx(b1), ib2 = rcp_approx(b2_), i12 = ib1 * ib2;
+                    const float sval = a1 * a2 * i12;
+                    p.x = 2.f * gs * fmaf(my * (a2 - a1), i12, mx * sval * (ib2 - ib1));
+                    p.y = -gs * sval * ib2;
+                    p.z = 2.f * gs * a1 * i12;
+                    if (j0 + o >= 5 && j0 + o < 5 + kOP && q >= 5 && q < 5 + rows) ss += sval;
+                }
+                dst[o] = p;
             }
         }
         __syncthreads();
-        // horizontal statistics: three neighbouring columns per item from one window of 13
-        for (int it = tid; it < kIn * kH1; it += kLossThreads) {
-            const int iy = it / kH1, jx0 = (it - iy * kH1) * 3;
-            const float2* r = sxy + iy * kIn + jx0;
-            float2 ab[2 * kR + 3], sq[2 * kR + 3];
-            float xy[2 * kR + 3];
+        // ---- 3: statistics row q adds to output row q - d; row q - 10 is then complete (in place) ----
+        if (px < kTP) {
 #pragma unroll
-            for (int k = 0; k < 2 * kR + 3; ++k) {
-                ab[k] = r[k];
-                sq[k] = __fmul2_rn(ab[k], ab[k]);
-                xy[k] = ab[k].x * ab[k].y;
-            }
+            for (int i = 0; i < kTap; ++i) {
+                float4* const at = sp + (i * 3 + ch) * kPW + px;
+                const float4 p = *at;
 #pragma unroll
-            for (int o = 0; o < 3; ++o) {
-                float2 s01 = f2(0.f, 0.f), s23 = f2(0.f, 0.f);
-                float s4 = 0.f;
-#pragma unroll
-                for (int k = 0; k < 2 * kR + 1; ++k) {
-                    s01 = __ffma2_rn(g2[k], ab[o + k], s01);
-                    s23 = __ffma2_rn(g2[k], sq[o + k], s23);
-                    s4 = fmaf(g2[k].x, xy[o + k], s4);
+                for (int d = 0; d < kTap; ++d) {
+                    const int k = (i + 1 - d + kTap) % kTap;            // q = 11 b + i - 10 is i + 1 mod 11
+                    b01[k] = d == 0 ? __fmul2_rn(f2(g[0], g[0]), f2(p.x, p.y))
+                                    : __ffma2_rn(f2(g[d], g[d]), f2(p.x, p.y), b01[k]);
+                    b2[k] = d == 0 ? g[0] * p.z : fmaf(g[d], p.z, b2[k]);
                 }
-                const int i = iy * kSt + jx0 + o;
-                h01[i] = s01;
-                h23[i] = s23;
-                h4[i] = s4;
+                const int k = (i + 2) % kTap;
+                *at = make_float4(b01[k].x, b01[k].y, b2[k], 0.f);
             }
         }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) xy[i] = load_row(t0 + kTap + i);
+        if (t0 + kTap <= 20) continue;              // the first batch completes no output row
         __syncthreads();
-        // vertical statistics, SSIM map and the loss partials: seven rows per item
-        for (int it = tid; it < kSt * kS2; it += kLossThreads) {
-            const int strip = it / kSt, jx = it - strip * kSt, jy0 = strip * kV2;
-            float2 st01[kV2], st23[kV2];
-            float st4[kV2];
-            {
-                float2 h[kV2 + 2 * kR];
+        // ---- 4: output row n (image row r0 + n), pixel j (image column x0 + j) ----
+        for (int it = tid; it < kTap * 3 * (kOP / 5); it += kLossThreads) {
+            const int i = it / (3 * (kOP / 5)), rest = it - i * (3 * (kOP / 5));
+            const int c = rest / (kOP / 5), j0 = 5 * (rest - c * (kOP / 5));
+            const int n = t0 + i - 20;
+            if (n < 0 || n >= rows) continue;
+            float2 f01[5];
+            float fz[5];
 #pragma unroll
-                for (int r = 0; r < kV2 + 2 * kR; ++r) h[r] = h01[(jy0 + r) * kSt + jx];
+            for (int o = 0; o < 5; ++o) f01[o] = f2(0.f, 0.f), fz[o] = 0.f;
+            const float4* const src = sp + (i * 3 + c) * kPW + j0;
 #pragma unroll
-                for (int o = 0; o < kV2; ++o) {
-                    float2 acc = f2(0.f, 0.f);
+            for (int k = 0; k < kTap + 4; ++k) {
+                const float4 w = src[k];
 #pragma unroll
-                    for (int k = 0; k < 2 * kR + 1; ++k) acc = __ffma2_rn(g2[k], h[o + k], acc);
-                    st01[o] = acc;
-                }
-#pragma unroll
-                for (int r = 0; r < kV2 + 2 * kR; ++r) h[r] = h23[(jy0 + r) * kSt + jx];
-#pragma unroll
-                for (int o = 0; o < kV2; ++o) {
-                    float2 acc = f2(0.f, 0.f);
-#pragma unroll
-                    for (int k = 0; k < 2 * kR + 1; ++k) acc = __ffma2_rn(g2[k], h[o + k], acc);
-                    st23[o] = acc;
-                }
+                for (int o = 0; o < 5; ++o)
+                    if (k - o >= 0 && k - o < kTap) {
+                        f01[o] = __ffma2_rn(f2(g[k - o], g[k - o]), f2(w.x, w.y), f01[o]);
+                        fz[o] = fmaf(g[k - o], w.z, fz[o]);
+                    }
             }
-            {
-                float h[kV2 + 2 * kR];
+            float4* const dst = sv + (i * 3 + c) * kVW + j0;
 #pragma unroll
-                for (int r = 0; r < kV2 + 2 * kR; ++r) h[r] = h4[(jy0 + r) * kSt + jx];
+            for (int o = 0; o < 5; ++o) dst[o] = make_float4(f01[o].x, f01[o].y, fz[o], 0.f);
+        }
+        const bool out_col = px < kOP && x0 + px < W;
+        const long long out_at = 3ll * (x0 + px) + ch;
+        float2 ab[kTap];                                // step 5's pixels, loaded across the barrier
 #pragma unroll
-                for (int o = 0; o < kV2; ++o) {
-                    float acc = 0.f;
-#pragma unroll
-                    for (int k = 0; k < 2 * kR + 1; ++k) acc = fmaf(g2[k].x, h[o + k], acc);
-                    st4[o] = acc;
-                }
-            }
-            const int gx = x0 - kR + jx;
-            const bool col_in = gx >= 0 && gx < W;
-            const bool col_own = jx >= kR && jx < kR + kLT;
-#pragma unroll
-            for (int o = 0; o < kV2; ++o) {
-                const int jy = jy0 + o, gy = y0 - kR + jy;
-                float2 p01 = f2(0.f, 0.f);
-                float p2 = 0.f;
-                if (col_in && gy >= 0 && gy < H) {
-                    const float mx = st01[o].x, my = st01[o].y;
-                    const float sxx = st23[o].x - mx * mx, syy = st23[o].y - my * my, sxy_ = st4[o] - mx * my;
-                    const float a1 = 2.f * mx * my + L.c1, a2 = 2.f * sxy_ + L.c2;
-                    const float b1 = mx * mx + my * my + L.c1, b2 = sxx + syy + L.c2;
-                    const float ib1 = rcp_approx(b1), ib2 = rcp_approx(b2);
-                    const float sv = a1 * a2 * ib1 * ib2;
-                    p01 = f2(gs * (2.f * my * (a2 - a1) * ib1 * ib2 + 2.f * mx * sv * (ib2 - ib1)), gs * (-sv * ib2));
-                    p2 = gs * (2.f * a1 * ib1 * ib2);
-                    if (col_own && jy >= kR && jy < kR + kLT) ss += sv;
-                }
-                const int i = jy * kMP + jx;
-                m01[i] = p01;
-                m2[i] = p2;
-            }
+        for (int i = 0; i < kTap; ++i) {
+            const int n = t0 + i - 20;
+            ab[i] = f2(0.f, 0.f);
+            if (out_col && n >= 0 && n < rows)
+                ab[i] = f2(__ldg(img + ((r0 + n) * pitch + out_at)), __ldg(ref + ((r0 + n) * pitch + out_at)));
         }
         __syncthreads();
-        // horizontal pass of the partials: four columns per item, consecutive lanes on consecutive rows
-        for (int it = tid; it < kSt * kB3; it += kLossThreads) {
-            const int blk = it / kSt, jy = it - blk * kSt, ox0 = blk * kH3;
-            float2 r[kH3 + 2 * kR];
-            float r2[kH3 + 2 * kR];
+        // ---- 5: the gradient ----
+        if (out_col) {
 #pragma unroll
-            for (int k = 0; k < kH3 + 2 * kR; ++k) {
-                r[k] = m01[jy * kMP + ox0 + k];
-                r2[k] = m2[jy * kMP + ox0 + k];
-            }
-#pragma unroll
-            for (int o = 0; o < kH3; ++o) {
-                float2 acc = f2(0.f, 0.f);
-                float acc2 = 0.f;
-#pragma unroll
-                for (int k = 0; k < 2 * kR + 1; ++k) {
-                    acc = __ffma2_rn(g2[k], r[o + k], acc);
-                    acc2 = fmaf(g2[k].x, r2[o + k], acc2);
-                }
-                f01[jy * kFP + ox0 + o] = acc;
-                f2s[jy * kFP + ox0 + o] = acc2;
-            }
-        }
-        __syncthreads();
-        // vertical pass of the partials and the gradient: four rows per item
-        for (int it = tid; it < kLT * kS4; it += kLossThreads) {
-            const int strip = it / kLT, ox = it - strip * kLT, oy0 = strip * kV4;
-            const int gx = x0 + ox;
-            float2 cc[kV4 + 2 * kR];
-            float c2[kV4 + 2 * kR];
-#pragma unroll
-            for (int r = 0; r < kV4 + 2 * kR; ++r) {
-                cc[r] = f01[(oy0 + r) * kFP + ox];
-                c2[r] = f2s[(oy0 + r) * kFP + ox];
-            }
-            float av[kV4], bv[kV4];            // the staged copies are overwritten by now: read them again
-#pragma unroll
-            for (int o = 0; o < kV4; ++o) {
-                const int gy = y0 + oy0 + o;
-                av[o] = bv[o] = 0.f;
-                if (gx < W && gy < H) {
-                    const long long pix = (base + (long long)gy * W + gx) * 3 + c;
-                    av[o] = __ldg(rgb + pix);
-                    bv[o] = __ldg(tgt + pix);
-                }
-            }
-            float2 f[kV4];
-            float fx[kV4];
-#pragma unroll
-            for (int o = 0; o < kV4; ++o) {
-                float2 acc = f2(0.f, 0.f);
-                float acc2 = 0.f;
-#pragma unroll
-                for (int k = 0; k < 2 * kR + 1; ++k) {
-                    acc = __ffma2_rn(g2[k], cc[o + k], acc);
-                    acc2 = fmaf(g2[k].x, c2[o + k], acc2);
-                }
-                f[o] = acc;
-                fx[o] = acc2;
-            }
-            if (gx >= W) continue;
-#pragma unroll
-            for (int o = 0; o < kV4; ++o) {
-                const int oy = oy0 + o, gy = y0 + oy;
-                if (gy >= H) break;
-                const long long pix = (base + (long long)gy * W + gx) * 3 + c;
-                const float a = av[o], b = bv[o];
-                const float d = a - b;
+            for (int i = 0; i < kTap; ++i) {
+                const int n = t0 + i - 20;
+                if (n < 0 || n >= rows) continue;
+                const float4 f = sv[(i * 3 + ch) * kVW + px];
+                const float x = ab[i].x, y = ab[i].y, d = x - y;
                 l1 += fabsf(d);
                 const float gd = d > 0.f ? gl1 : (d < 0.f ? -gl1 : 0.f);
-                grad[pix] = f[o].x + 2.f * a * f[o].y + b * fx[o] + gd;
+                out[(r0 + n) * pitch + out_at] = f.x + 2.f * x * f.y + y * f.z + gd;
             }
         }
         __syncthreads();
@@ -359,7 +322,7 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ p, const float
 
 cudaError_t launch_loss_3dgs(const float* rgb, const float* target, const LossViews& L, float* loss, float* grad,
                              cudaStream_t s) {
-    const size_t smem = (size_t)kLossSmemFloats * sizeof(float);
+    constexpr int smem = kLossSmem;
     // the shared-memory opt-in is a per-device function attribute: set it once per device (thread-safe)
     static std::once_flag once[64];
     static cudaError_t once_err[64];
@@ -368,7 +331,7 @@ cudaError_t launch_loss_3dgs(const float* rgb, const float* target, const LossVi
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::call_once(once[dev], [&] {
-        once_err[dev] = cudaFuncSetAttribute(k_loss_3dgs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        once_err[dev] = cudaFuncSetAttribute(k_loss_3dgs, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     });
     if (once_err[dev] != cudaSuccess) return once_err[dev];
     e = cudaMemsetAsync(loss, 0, 3 * sizeof(float), s);
@@ -379,7 +342,32 @@ cudaError_t launch_loss_3dgs(const float* rgb, const float* target, const LossVi
     return cudaGetLastError();
 }
 
-int loss_tile_side() { return kLT; }
+// Strips and segments of the views (tiles_x, tile_off, rows).  A segment takes as many batches of 11 rows as its
+// rows and 20 more need, so the rows are 11 k - 20; k is the one whose last wave of 304 blocks (two per SM) ends
+// first: a batch of 11 rows costs about the same wherever it lies, so the waves times k are the time.  False when the views hold too many.
+bool loss_plan(LossViews& L) {
+    long long best = 0;
+    for (int k = 3; k <= 32; ++k) {
+        const int rows = kTap * k - 20;
+        long long blocks = 0;
+        for (int v = 0; v < L.n; ++v)
+            blocks += (long long)((L.w[v] + kOP - 1) / kOP) * ((L.h[v] + rows - 1) / rows);
+        const long long cost = (blocks + 303) / 304 * k;
+        if (best == 0 || cost < best) {
+            best = cost;
+            L.rows = rows;
+        }
+    }
+    long long blocks = 0;
+    for (int v = 0; v < L.n; ++v) {
+        L.tiles_x[v] = (L.w[v] + kOP - 1) / kOP;
+        L.tile_off[v] = (int)blocks;
+        blocks += (long long)L.tiles_x[v] * ((L.h[v] + L.rows - 1) / L.rows);
+        if (blocks > (1ll << 30)) return false;
+    }
+    L.tile_off[L.n] = (int)blocks;
+    return true;
+}
 
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, const AdamGroups& G, double beta1,
                         double beta2, AdamState* st, const WsHeader* guard, cudaStream_t s) {

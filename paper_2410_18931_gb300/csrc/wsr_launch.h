@@ -137,10 +137,12 @@ cudaError_t launch_count_pairs(const float* records, const unsigned* tile_offset
 cudaError_t launch_loss_l1(const float* rgb, const float* target, long long count,
                            float* loss, float* grad, cudaStream_t s);
 
-// Views of the 3DGS loss: tiles of loss_tile_side() square per view, in view
-// order; the Gaussian window taps g[] are normalised to sum 1.
+// Views of the 3DGS loss: strips (tiles_x of them) and segments of `rows` rows
+// per view, in view order (loss_plan); the Gaussian window taps g[] are normalised
+// to sum 1.
 struct LossViews {
     int n;
+    int rows;
     int tile_off[WSR_MAX_VIEWS + 1];
     int tiles_x[WSR_MAX_VIEWS];
     int w[WSR_MAX_VIEWS];
@@ -150,7 +152,7 @@ struct LossViews {
     float lam, inv_count, c1, c2;
 };
 
-int loss_tile_side();
+bool loss_plan(LossViews& L);
 cudaError_t launch_loss_3dgs(const float* rgb, const float* target, const LossViews& L, float* loss,
                              float* grad, cudaStream_t s);
 
