@@ -71,6 +71,10 @@ enum { WSR_OPACITY_LOGIT = 0, WSR_OPACITY_SH = 1 };
 #define WSR_GRAD_RECORD_FLOATS_DET 32 /* one record in deterministic mode: 128 bytes */
 #define WSR_DET_MAX_SEGMENT 8192  /* deterministic mode: most instances one tile may hold */
 #define WSR_SCAN_ONE_BLOCK_TILES 32768  /* wsr_bin scans (and orders) up to this many tiles in one kernel */
+/* wsr_bin makes one launch for a small scene: at most WSR_BIN_ONE_TILES tiles over all views and
+ * WSR_BIN_ONE_GAUSSIANS Gaussians times views (half as many beyond 1024 tiles) */
+#define WSR_BIN_ONE_TILES 4096
+#define WSR_BIN_ONE_GAUSSIANS 8192
 
 /* Pinhole camera (passed by value through host memory). */
 typedef struct {

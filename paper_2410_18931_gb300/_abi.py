@@ -24,6 +24,8 @@ WSR_GRAD_RECORD_FLOATS = 12
 WSR_GRAD_RECORD_FLOATS_DET = 32      # deterministic mode: 9 int64 sums and their 9 bounds per record
 WSR_DET_MAX_SEGMENT = 8192
 WSR_SCAN_ONE_BLOCK_TILES = 32768     # wsr_bin scans (and orders) up to this many tiles in one kernel
+WSR_BIN_ONE_TILES = 4096             # wsr_bin makes one launch for at most this many tiles over all views
+WSR_BIN_ONE_GAUSSIANS = 8192         # and this many Gaussians times views (half as many beyond 1024 tiles)
 WSR_BIN_STATIC_MAX_TILES = 65536     # tiles over all views that wsr_bin_static handles
 WSR_BIN_STATIC_BYTES = 270848        # its fixed scratch array, held by every GPU that loads the library
 

@@ -315,10 +315,15 @@ wsr_status wsr_bin(const float* records, int64_t n, const wsr_camera* cams, int3
     if ((unsigned long long)n * (unsigned long long)n_cams > 0xffffffffull) return WSR_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const WsLayout L = ws_layout(vs);
-    WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, workspace, L, s));
     char* ws = (char*)workspace;
-    WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), bin_base(L, ws), tile_list, list_capacity,
-                                (WsHeader*)ws, s));
+    if (bin_in_one(n, vs.n, vs.total_tiles)) {
+        unsigned* order = vs.schedule == WSR_SCHEDULE_PERSISTENT ? (unsigned*)(ws + L.order) : nullptr;
+        WSR_CUDA(launch_bin_one(records, n, vs, tile_offsets, tile_list, list_capacity, (WsHeader*)ws, order, s));
+    } else {
+        WSR_TRY(bin_count_impl(records, n, vs, tile_offsets, list_capacity, workspace, L, s));
+        WSR_CUDA(launch_bin_scatter(records, n, vs, (unsigned*)(ws + L.cursor), bin_base(L, ws), tile_list,
+                                    list_capacity, (WsHeader*)ws, s));
+    }
     if (vs.det) WSR_CUDA(launch_sort_segments(vs, tile_offsets, tile_list, (WsHeader*)ws, s));
     if (total_dev)
         WSR_CUDA(cudaMemcpyAsync(total_dev, &((WsHeader*)ws)->total, sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));

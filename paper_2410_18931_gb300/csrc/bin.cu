@@ -11,9 +11,12 @@
 //                  block, with the persistent schedule's tile order, for up
 //                  to kSmallScanTiles tiles)
 //   k_bin<true>    scatter: claim a slot per (Gaussian, tile) and store
+//   k_bin_one      all of these in one launch, for small scenes
 // A tile is listed when a pixel-centre column of it meets the footprint
 // q <= 9 within the tile's band of pixel-centre rows (the ellipse's exact
 // extent per tile row), not merely when it meets the bounding box.
+#include <cooperative_groups.h>
+
 #include <mutex>
 
 #include "wsr_launch.h"
@@ -448,15 +451,16 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_small(unsigned* __res
 // same bucket by matching lanes, so that neither pass over the tiles queues on a bucket's counter.  It is bound by
 // the latency of its chain of loads, shuffles and three barriers: 12 -> 6 us for 8160 tiles with the order.
 // With SCAN false it only orders the tiles of given offsets.
-template <int I, bool SCAN>
-__global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __restrict__ cursor, int n,
-                                                                unsigned* __restrict__ offsets,
-                                                                unsigned long long capacity, WsHeader* hdr,
-                                                                unsigned* __restrict__ order) {
-    __shared__ unsigned long long s_sum[32];
-    __shared__ unsigned s_hist[32][33];         // per warp and bucket: tiles, then the first place among the bucket's
-    __shared__ unsigned s_total[33];            // per bucket: tiles, then the bucket's first place in the order
-    const unsigned long long lim = capacity < 0xffffffffull ? capacity : 0xffffffffull;
+struct ScanShared {
+    unsigned long long sum[32];
+    unsigned hist[32][33];              // per warp and bucket: tiles, then the first place among the bucket's
+    unsigned total[33];                 // per bucket: tiles, then the bucket's first place in the order
+};
+
+// load(t): a tile's count; SCAN: store(t, o) takes its offset (at most lim), finish(total) the sum, once
+template <int I, bool SCAN, typename Load, typename Store, typename Finish>
+__device__ __forceinline__ void scan_order_rows(const int n, const unsigned long long lim, unsigned* __restrict__ order,
+                                                ScanShared& sh, Load&& load, Store&& store, Finish&& finish) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     const int t0 = warp * 32 * I + lane;
@@ -464,20 +468,20 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
 #pragma unroll
     for (int r = 0; r < I; ++r) {
         const int t = t0 + 32 * r;
-        c[r] = t >= n ? 0u : SCAN ? cursor[t] : offsets[t + 1] - offsets[t];
+        c[r] = t >= n ? 0u : load(t);
     }
     if (order) {
-        s_hist[warp][lane] = 0u;
-        if (lane == 0) s_hist[warp][32] = 0u;
+        sh.hist[warp][lane] = 0u;
+        if (lane == 0) sh.hist[warp][32] = 0u;
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < I; ++r) {
             const int b = t0 + 32 * r < n ? cost_bucket(c[r]) : 33;
             const unsigned same = __match_any_sync(0xffffffffu, b);
             unsigned h = 0u;
-            if (b < 33) h = s_hist[warp][b];
+            if (b < 33) h = sh.hist[warp][b];
             __syncwarp();
-            if (b < 33 && (same & below) == 0u) s_hist[warp][b] = h + __popc(same);
+            if (b < 33 && (same & below) == 0u) sh.hist[warp][b] = h + __popc(same);
             __syncwarp();
             rank[r] = h + __popc(same & below);
         }
@@ -499,9 +503,9 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
             inc[r] += sum - c[r];                   // exclusive within the warp's tiles
             sum += row;
         }
-        if (lane == 0) s_sum[warp] = sum;
+        if (lane == 0) sh.sum[warp] = sum;
         __syncthreads();
-        unsigned long long x = s_sum[lane], scan = x;
+        unsigned long long x = sh.sum[lane], scan = x;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const unsigned long long y = __shfl_up_sync(0xffffffffu, scan, off);
@@ -514,43 +518,36 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
             const int t = t0 + 32 * r;
             const unsigned long long run = first + inc[r];
             const unsigned o = (unsigned)(run < lim ? run : lim);
-            if (t < n) {
-                offsets[t] = o;
-                cursor[t] = o;                      // the scatter's cursor starts at the tile's offset
-            }
+            if (t < n) store(t, o);
         }
-        if (threadIdx.x == 0) {
-            offsets[n] = (unsigned)(tot < lim ? tot : lim);
-            hdr->total = tot;
-            hdr->err = tot > lim ? WSR_ERR_CAPACITY : 0;        // a binning starts from no error
-        }
+        if (threadIdx.x == 0) finish(tot);
     } else {
         __syncthreads();
     }
     if (!order) return;
     // warp b takes bucket b (warp 0 also bucket 32), a lane per warp's count; then warp 0 the buckets
     for (int b = warp; b < 33; b += 32) {
-        const unsigned h = s_hist[lane][b];
+        const unsigned h = sh.hist[lane][b];
         unsigned hi = h;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const unsigned y = __shfl_up_sync(0xffffffffu, hi, off);
             if (lane >= off) hi += y;
         }
-        s_hist[lane][b] = hi - h;
-        if (lane == 31) s_total[b] = hi;
+        sh.hist[lane][b] = hi - h;
+        if (lane == 31) sh.total[b] = hi;
     }
     __syncthreads();
     if (warp == 0) {
-        const unsigned most = s_total[32], h = s_total[lane];   // bucket 32 comes first
+        const unsigned most = sh.total[32], h = sh.total[lane];   // bucket 32 comes first
         unsigned hi = h;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const unsigned y = __shfl_down_sync(0xffffffffu, hi, off);
             if (lane + off < 32) hi += y;
         }
-        s_total[lane] = most + hi - h;
-        if (lane == 0) s_total[32] = 0u;
+        sh.total[lane] = most + hi - h;
+        if (lane == 0) sh.total[32] = 0u;
     }
     __syncthreads();
 #pragma unroll
@@ -558,9 +555,98 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __rest
         const int t = t0 + 32 * r;
         if (t < n) {
             const int b = cost_bucket(c[r]);
-            order[s_total[b] + s_hist[warp][b] + rank[r]] = (unsigned)t;
+            order[sh.total[b] + sh.hist[warp][b] + rank[r]] = (unsigned)t;
         }
     }
+}
+
+template <int I, bool SCAN>
+__global__ void __launch_bounds__(kScanBlock) k_scan_order_rows(unsigned* __restrict__ cursor, int n,
+                                                                unsigned* __restrict__ offsets,
+                                                                unsigned long long capacity, WsHeader* hdr,
+                                                                unsigned* __restrict__ order) {
+    __shared__ ScanShared sh;
+    const unsigned long long lim = capacity < 0xffffffffull ? capacity : 0xffffffffull;
+    scan_order_rows<I, SCAN>(
+        n, lim, order, sh, [&](int t) { return SCAN ? cursor[t] : offsets[t + 1] - offsets[t]; },
+        [&](int t, unsigned o) {
+            offsets[t] = o;
+            cursor[t] = o;                          // the scatter's cursor starts at the tile's offset
+        },
+        [&](unsigned long long tot) {
+            offsets[n] = (unsigned)(tot < lim ? tot : lim);
+            hdr->total = tot;
+            hdr->err = tot > lim ? WSR_ERR_CAPACITY : 0;        // a binning starts from no error
+        });
+}
+
+// Count, scan, order and scatter of a small scene in one launch: a cluster of kOneBlocks blocks, every tile's counter
+// in each block's shared memory.  Warp w of block r takes the batches of 32 Gaussians r + kOneBlocks (w + 32 i) of all
+// views in both passes; between them each block reads all blocks' counters (distributed shared memory) and scans
+// them, so that its cursors start at a tile's offset plus what the blocks before it hold there.  Nothing else than
+// the list, the offsets, the header and the order is written.
+//   Latency bounds it (launch, records, prefix, segments, tiles, twice): 1000 Gaussians at 128x128, 17.7 us for the
+// clear and three kernels -> 8.4; bin_in_one has the limits.
+template <int I>
+__global__ void __cluster_dims__(kOneBlocks, 1, 1) __launch_bounds__(1024, 1)
+    k_bin_one(const float4* __restrict__ rec, long long n, const Views vs, unsigned* __restrict__ offsets,
+              unsigned* __restrict__ list, unsigned long long capacity, WsHeader* hdr, unsigned* __restrict__ order) {
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ ScanShared sh;
+    BinScratch* const scratch = reinterpret_cast<BinScratch*>(s_dyn);
+    const int T = vs.total_tiles;
+    unsigned* const cnt = reinterpret_cast<unsigned*>(s_dyn + sizeof(BinScratch) * 32);
+    unsigned* const cur = cnt + T;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank(), warp = threadIdx.x >> 5;
+    const int lw = __ffs(vs.tile_w) - 1, lh = __ffs(vs.tile_h) - 1;     // tile sides are powers of two
+    const unsigned long long lim = capacity < 0xffffffffull ? capacity : 0xffffffffull;
+    for (int t = threadIdx.x; t < T; t += 1024) cnt[t] = 0u;
+    __syncthreads();
+    const long long nb = (n + 31) >> 5;                                 // batches per view
+    auto pass = [&](auto&& emit) {
+        for (long long b = rank + kOneBlocks * warp; b < nb * vs.n; b += kOneBlocks * 32) {
+            const int v = (int)(b / nb);
+            const long long i0 = (b - v * nb) << 5;
+            const View& V = vs.v[v];
+            bin_batch(rec, n, V, v, i0, lw, lh, scratch[warp],
+                      [&](int tile, int owner) { emit(V.tile_base + tile, (unsigned)(v * n + i0 + owner)); });
+        }
+    };
+    pass([&](int tile, unsigned) { atomicAdd(cnt + tile, 1u); });
+    cluster.sync();
+    const unsigned* all[kOneBlocks];
+#pragma unroll
+    for (int c = 0; c < kOneBlocks; ++c) all[c] = cluster.map_shared_rank(cnt, c);
+    scan_order_rows<I, true>(
+        T, lim, rank == kOneBlocks - 1 ? order : nullptr, sh,
+        [&](int t) {
+            unsigned sum = 0u, before = 0u;
+#pragma unroll
+            for (int c = 0; c < kOneBlocks; ++c) {
+                if (c == rank) before = sum;
+                sum += all[c][t];
+            }
+            cur[t] = before;
+            return sum;
+        },
+        [&](int t, unsigned o) {
+            cur[t] += o;
+            if (rank == 0) offsets[t] = o;
+        },
+        [&](unsigned long long tot) {
+            if (rank != 0) return;
+            offsets[T] = (unsigned)(tot < lim ? tot : lim);
+            hdr->total = tot;
+            hdr->err = tot > lim ? WSR_ERR_CAPACITY : 0;                // a binning starts from no error
+        });
+    cluster.sync();                 // the cursors stand, every block is done with the others' counters
+    pass([&](int tile, unsigned at) {
+        const unsigned slot = atomicAdd(cur + tile, 1u);
+        if (slot < capacity) list[slot] = at;
+        else set_error(hdr, WSR_ERR_CAPACITY);
+    });
 }
 
 __global__ void __launch_bounds__(256) k_order_hist(const unsigned* __restrict__ offsets, int n,
@@ -752,6 +838,33 @@ static cudaError_t launch_bin_local(const LocalBin& L, const float* records, lon
     k_bin_local<NT, SCATTER><<<dim3((unsigned)L.blocks, (unsigned)vs.n), NT, L.smem, s>>>(
         reinterpret_cast<const float4*>(records), n, vs, cursor, base, list, capacity, hdr);
     return cudaGetLastError();
+}
+
+template <int I>
+static cudaError_t launch_one(const float* records, long long n, const Views& vs, unsigned* offsets, unsigned* list,
+                              unsigned long long capacity, WsHeader* hdr, unsigned* order, cudaStream_t s) {
+    // the shared-memory opt-in is a per-device function attribute: set once per device (thread-safe)
+    static std::once_flag once[64];
+    static cudaError_t once_err[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    constexpr size_t fixed = sizeof(BinScratch) * 32;
+    std::call_once(once[dev], [&] {
+        once_err[dev] = cudaFuncSetAttribute(k_bin_one<I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(fixed + 2 * sizeof(unsigned) * 1024 * I));
+    });
+    if (once_err[dev] != cudaSuccess) return once_err[dev];
+    k_bin_one<I><<<kOneBlocks, 1024, fixed + 2 * sizeof(unsigned) * (size_t)vs.total_tiles, s>>>(
+        reinterpret_cast<const float4*>(records), n, vs, offsets, list, capacity, hdr, order);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_bin_one(const float* records, long long n, const Views& vs, unsigned* offsets, unsigned* list,
+                           unsigned long long capacity, WsHeader* hdr, unsigned* order, cudaStream_t s) {
+    static_assert(WSR_BIN_ONE_TILES == 4096, "four tiles per thread at most");
+    return (vs.total_tiles <= 1024 ? launch_one<1> : launch_one<4>)(records, n, vs, offsets, list, capacity, hdr, order, s);
 }
 
 cudaError_t launch_bin_count(const float* records, long long n, const Views& vs, unsigned* cursor, unsigned* base,

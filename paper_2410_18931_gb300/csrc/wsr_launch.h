@@ -74,6 +74,18 @@ inline int bin_blocks_per_view(int n_views, int t_max) {
     return all / n_views > 1 ? all / n_views : 1;
 }
 
+// A small scene's whole binning in one launch (k_bin_one): beyond these sizes its eight blocks take longer than the
+// launches they save.  Clear, count, scan and scatter -> one kernel, us, over all views together: 17.8 -> 8.5 at 1000
+// Gaussians and 104 tiles, 18.4 -> 12.5 at 8000 and 104, 21.3 -> 18.5 at 8000 and 920, 18.6 -> 20.6 at 16000 and 920;
+// 31.1 -> 26.0 at 3000 and 3600, 30.8 -> 33.0 at 8000 and 3600; 42.0 -> 39.1 at 1000 and 8160 (not taken).
+constexpr int kOneBlocks = 8;               // blocks of its cluster, the largest portable one
+inline bool bin_in_one(long long n, int n_views, int total_tiles) {
+    return total_tiles <= WSR_BIN_ONE_TILES &&
+           n * n_views <= (total_tiles <= 1024 ? WSR_BIN_ONE_GAUSSIANS : WSR_BIN_ONE_GAUSSIANS / 2);
+}
+cudaError_t launch_bin_one(const float* records, long long n, const Views& vs, unsigned* offsets, unsigned* tile_list,
+                           unsigned long long capacity, WsHeader* hdr, unsigned* order, cudaStream_t s);
+
 // base: nullptr (global counters only), or total_tiles x bin_blocks_per_view words that carry each block's
 // places from the count to the scatter (pass the same to both)
 cudaError_t launch_bin_count(const float* records, long long n, const Views& vs,

@@ -93,7 +93,7 @@ class Renderer:
         self.chunk = int(chunk)
         self.tile = tuple(tile)
         self.num_tiles = int(self.lib.wsr_num_tiles(self.cams_c, self.n_cams, ctypes.byref(self.tiles_c)))
-        # kernels one wsr_bin launches: the count; the scan, in one kernel (with the persistent schedule's
+        # kernels one wsr_bin launches (bin_launches: small scenes make fewer): the count; the scan, in one kernel (with the persistent schedule's
         # tile order) up to WSR_SCAN_ONE_BLOCK_TILES tiles, else three (and three for the order); the
         # scatter; in the deterministic mode the sort of each tile's list
         if self.num_tiles <= A.WSR_SCAN_ONE_BLOCK_TILES:
@@ -112,6 +112,13 @@ class Renderer:
         self.headroom = headroom
         self.capacity = 0
         self.last_total = 0
+
+    def bin_launches(self, n: int) -> int:
+        """Kernels one ``wsr_bin`` of n Gaussians launches: one for a small scene (and the deterministic sort)."""
+        most = A.WSR_BIN_ONE_GAUSSIANS if self.num_tiles <= 1024 else A.WSR_BIN_ONE_GAUSSIANS // 2
+        if self.num_tiles <= A.WSR_BIN_ONE_TILES and n * self.n_cams <= most:
+            return 2 if self.deterministic else 1
+        return self.bin_kernels
 
     # -- raw C-ABI calls (same names as include/wsr.h) --------------------
     def wsr_project(self, g: Gaussians, kind: int, wparams: torch.Tensor, records: torch.Tensor, stream=None):

@@ -198,9 +198,9 @@ class TrainStep:
 
     @property
     def kernels_per_step(self) -> int:
-        # project 1, bin (Renderer.bin_kernels), fwd 1, loss 1, bwd 1 (and its tile order, where the binning has none),
+        # project 1, bin (Renderer.bin_launches), fwd 1, loss 1, bwd 1 (and its tile order, where the binning has none),
         # project bwd 1, Adam 2; deterministic: + the largest-pixel-term kernel and two ordered reductions
-        return 7 + self.r.bin_kernels + (0 if self.persistent else self.r.order_kernels) + (3 if self.deterministic else 0)
+        return 7 + self.r.bin_launches(self.g.n) + (0 if self.persistent else self.r.order_kernels) + (3 if self.deterministic else 0)
 
     def train(self, steps: int, check_every: int = 10) -> torch.Tensor:
         """Make ``steps`` Adam updates; returns the loss triples {L, L1, SSIM}
