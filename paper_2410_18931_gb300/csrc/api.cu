@@ -385,7 +385,7 @@ wsr_status wsr_render_fwd(const float* records, int64_t n, const uint32_t* tile_
     if (!aligned16(records) || !aligned4(tile_list) || !aligned4(tile_offsets) || !aligned4(out_rgb) ||
         !aligned4(out_den))
         return WSR_ERR_INVALID_ARG;
-    return cuda_status(launch_render_fwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den,
+    return cuda_status(launch_render_fwd(records, n, tile_offsets, tile_list, vs, wd, out_rgb, out_den,
                                          sched_of(vs, workspace), (cudaStream_t)stream));
 }
 

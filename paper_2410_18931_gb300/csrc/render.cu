@@ -111,6 +111,8 @@ struct TileShape {
 // staging and a warp per region.  One block per tile: 566 -> 399 us, 95 -> 60 us for 200k at 1280x720.
 //   20 warps per SM (at most 96 registers a thread): 363 us against 367 at 16, 379 at 24 and 389 at 28.
 constexpr int kFwdWarpsPerSM = 20;
+// The kernel for sparse views: 48 registers a thread, about as fast with 32 and 48 warps.
+constexpr int kLightWarpsPerSM = 40;
 
 template <int TW, int TH>
 struct FwdShape {
@@ -158,6 +160,44 @@ struct FwdStage {
     unsigned short list[NR][4][8 * NR + 2];         // per region and quarter warp: byte offsets into g
 };
 
+// C = (c_B w_B + N) / D and D = w_B + sum of a pixel, from its sums (N, D) = (x, y, z, w)
+__device__ __forceinline__ float4 pixel_out(const float4 n, const float* __restrict__ wparams) {
+    const float wB = __ldg(wparams + 2), D = wB + n.w, inv = 1.0f / D;
+    return make_float4((__ldg(wparams + 3) * wB + n.x) * inv, (__ldg(wparams + 4) * wB + n.y) * inv,
+                       (__ldg(wparams + 5) * wB + n.z) * inv, D);
+}
+
+// Whether two neighbouring pixels, the first at an even column, start on eight bytes in every row of the view.
+__device__ __forceinline__ bool pairs_aligned(const View& V, const float* out_rgb, const float* out_den) {
+    return (((V.pix_base | V.W) & 1) | ((reinterpret_cast<size_t>(out_rgb) | reinterpret_cast<size_t>(out_den)) & 7)) == 0;
+}
+
+// Two neighbouring pixels of a row, the first at an even column, in eight-byte stores where they are aligned: the
+// stores of a sparse view bound it otherwise (an empty 1920x1920 image 33 -> 25 us, 200k at 1280x720 58 -> 57).
+__device__ __forceinline__ void store_pair(const View& V, const bool aligned, const int x, const int y, const float4 p0,
+                                           const float4 p1, float* __restrict__ out_rgb, float* __restrict__ out_den) {
+    if (x >= V.W || y >= V.H) return;
+    const long long pix = V.pix_base + (long long)y * V.W + x;
+    float* const o = out_rgb + 3 * pix;
+    if (aligned) {                                  // (the width is even: both pixels exist)
+        reinterpret_cast<float2*>(o)[0] = f2(p0.x, p0.y);
+        reinterpret_cast<float2*>(o)[1] = f2(p0.z, p1.x);
+        reinterpret_cast<float2*>(o)[2] = f2(p1.y, p1.z);
+        *reinterpret_cast<float2*>(out_den + pix) = f2(p0.w, p1.w);
+        return;
+    }
+    o[0] = p0.x;
+    o[1] = p0.y;
+    o[2] = p0.z;
+    out_den[pix] = p0.w;
+    if (x + 1 < V.W) {
+        o[3] = p1.x;
+        o[4] = p1.y;
+        o[5] = p1.z;
+        out_den[pix + 1] = p1.w;
+    }
+}
+
 template <int TW, int TH, int S>
 __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restrict__ rec,
                                          const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
@@ -174,8 +214,6 @@ __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restric
     // The slice's batches of list entries, each thread staging one; the next batch's records are loaded while
     // this one is walked, and the list entries of the one after that.
     const unsigned start = offsets[tile], end = offsets[tile + 1];
-    const float wB = __ldg(wparams + 2);
-    const float cB0 = __ldg(wparams + 3) * wB, cB1 = __ldg(wparams + 4) * wB, cB2 = __ldg(wparams + 5) * wB;
     const TileCoord tc = tile_coord(vs, tile);
     const View& V = vs.v[tc.v];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = lane >> 3, o8 = lane & 7;
@@ -335,18 +373,121 @@ __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restric
             }
     }
     if (S > 1 && slice > 0) return;
+    store_pair(V, pairs_aligned(V, out_rgb, out_den), x_org + lx, y_org + ly, pixel_out(sum[0], wparams),
+               pixel_out(sum[1], wparams), out_rgb, out_den);
+}
+
+// Forward for sparse views, where a tile's time is the latency of its chain (offsets, list, records, pixels) and not
+// its arithmetic: a warp per 8x8 region as above, two pixels of a row per thread, the region's Gaussians one after
+// another.  Eight accumulators instead of 32 and no loads ahead, so
+// that twice the warps fit on an SM: 8000 Gaussians at 1920x1920 43 -> 27 us, 32,000 55 -> 47 us.
+template <int TW, int TH>
+__device__ __forceinline__ void fwd_tile_light(const int tile, const float4* __restrict__ rec,
+                                               const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
+                                               const Views& vs, const float* __restrict__ wparams,
+                                               float* __restrict__ out_rgb, float* __restrict__ out_den) {
+    using F = FwdShape<TW, TH>;
+    constexpr int RX = F::RX, NR = F::NR, BATCH = 32 * NR;
+    __shared__ float4 g[BATCH][3];                      // walk constants, as in FwdStage
+    __shared__ unsigned hits[NR][NR];
+    const unsigned start = offsets[tile], end = offsets[tile + 1];
+    const TileCoord tc = tile_coord(vs, tile);
+    const View& V = vs.v[tc.v];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int x_org = tc.tx * TW, y_org = tc.ty * TH;
+    const int lx = 8 * (w % RX) + 2 * (lane & 3), ly = 8 * (w / RX) + (lane >> 2);
+    const float2 ox = f2((float)lx, (float)(lx + 1));
+    const float oy = (float)ly;
+    auto sync = [&] {
+        if constexpr (NR == 1) __syncwarp();
+        else __syncthreads();
+    };
+    float2 rg[2], bd[2];                                // per column: (N_r, N_g) and (N_b, D)
+    rg[0] = rg[1] = bd[0] = bd[1] = f2(0.f, 0.f);
+    for (unsigned base = start; base < end; base += BATCH) {
+        if (base != start) sync();                      // the batch before is walked
+        if (base + 32 * w < end) {
+            const bool in = base + threadIdx.x < end;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            float cb = 0.f;
+            if (in) {
+                const float4* p = rec + 3ull * list[base + threadIdx.x];
+                a = __ldg(p);
+                b = __ldg(p + 1);
+                cb = __ldg(reinterpret_cast<const float*>(p + 2));
+            }
+            const float gx = (float)x_org + 0.5f - a.x, gy = (float)y_org + 0.5f - a.y;
+            g[threadIdx.x][0] = make_float4(a.z, a.w, fmaf(a.z, gy, a.w * gx), b.x);
+            g[threadIdx.x][1] = make_float4(b.x * gx * gx, 2.0f * b.x * gx, b.z, b.w);
+            *reinterpret_cast<float2*>(&g[threadIdx.x][2]) = f2(cb, b.y);
+            const unsigned hit = in ? regions_hit<RX, F::RY>(a, b.x, gx, gy) : 0u;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const int x = x_org + lx + c, y = y_org + ly;
-        if (x < V.W && y < V.H) {
-            const long long pix = V.pix_base + (long long)y * V.W + x;
-            const float D = wB + sum[c].w;
-            const float inv = 1.0f / D;
-            out_rgb[3 * pix + 0] = (cB0 + sum[c].x) * inv;
-            out_rgb[3 * pix + 1] = (cB1 + sum[c].y) * inv;
-            out_rgb[3 * pix + 2] = (cB2 + sum[c].z) * inv;
-            out_den[pix] = D;
+            for (int k = 0; k < NR; ++k) {
+                const unsigned bal = __ballot_sync(0xffffffffu, (hit >> k) & 1u);
+                if (lane == 0) hits[k][w] = bal;
+            }
         }
+        sync();
+        for (int k = 0; k < NR && base + 32 * k < end; ++k) {
+            for (unsigned bal = hits[w][k]; bal; bal &= bal - 1) {
+                const float4* e = g[32 * k + __ffs(bal) - 1];
+                const float4 u = e[0], t = e[1];
+                const float2 cbuw = *reinterpret_cast<const float2*>(e + 2);
+                const float2 crg = f2(t.z, t.w);
+                // q' in the same operations as above
+                const float2 P = __ffma2_rn(ox, __ffma2_rn(ox, f2(u.w, u.w), f2(t.y, t.y)), f2(t.x, t.x));
+                float2 rr;
+                if constexpr (TW == 8) {
+                    rr = __ffma2_rn(f2(u.x, u.x), f2(oy, oy), __ffma2_rn(f2(u.y, u.y), ox, f2(u.z, u.z)));
+                } else {
+                    const float ry = fmaf(u.x, oy, u.z);
+                    rr = __ffma2_rn(f2(u.y, u.y), ox, f2(ry, ry));
+                }
+                const float2 q = __ffma2_rn(rr, rr, P);
+                if (q.x <= kQMax) {
+                    const float e0 = ex2_approx(-q.x);
+                    rg[0] = __ffma2_rn(crg, f2(e0, e0), rg[0]);
+                    bd[0] = __ffma2_rn(cbuw, f2(e0, e0), bd[0]);
+                }
+                if (q.y <= kQMax) {
+                    const float e1 = ex2_approx(-q.y);
+                    rg[1] = __ffma2_rn(crg, f2(e1, e1), rg[1]);
+                    bd[1] = __ffma2_rn(cbuw, f2(e1, e1), bd[1]);
+                }
+            }
+        }
+    }
+    const float4 p0 = pixel_out(make_float4(rg[0].x, rg[0].y, bd[0].x, bd[0].y), wparams);
+    const float4 p1 = pixel_out(make_float4(rg[1].x, rg[1].y, bd[1].x, bd[1].y), wparams);
+    if (pairs_aligned(V, out_rgb, out_den)) {
+        store_pair(V, true, x_org + lx, y_org + ly, p0, p1, out_rgb, out_den);
+        return;
+    }
+    // the region's rows through shared memory, consecutive words to consecutive lanes: 39 -> 31 us at 1919x1919
+    __shared__ float s_px[NR][256];                     // 8 x 8 colours, then 8 x 8 densities
+    float* const px = s_px[w];
+    const int at = 8 * (lane >> 2) + 2 * (lane & 3);
+    __syncwarp();                                       // (the tile before has been read)
+    px[3 * at] = p0.x;
+    px[3 * at + 1] = p0.y;
+    px[3 * at + 2] = p0.z;
+    px[3 * at + 3] = p1.x;
+    px[3 * at + 4] = p1.y;
+    px[3 * at + 5] = p1.z;
+    px[192 + at] = p0.w;
+    px[193 + at] = p1.w;
+    __syncwarp();
+    const int xr = x_org + 8 * (w % RX), yr = y_org + 8 * (w / RX), xn = V.W - xr, yn = V.H - yr;   // may be negative
+    const long long pix = V.pix_base + (long long)yr * V.W + xr;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const int e = lane + 32 * k, row = e / 24, c = e - 24 * row;
+        if (row < yn && c < 3 * xn) out_rgb[3 * (pix + (long long)row * V.W) + c] = px[e];
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int e = lane + 32 * k, row = e >> 3, c = e & 7;
+        if (row < yn && c < xn) out_den[pix + (long long)row * V.W + c] = px[192 + e];
     }
 }
 
@@ -377,6 +518,17 @@ __global__ void __launch_bounds__(32 * S * FwdShape<TW, TH>::NR, kFwdWarpsPerSM 
                  unsigned* __restrict__ counter) {
     for_each_tile(order, counter, vs.total_tiles, [&](int tile) {
         fwd_tile<TW, TH, S>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den);
+    });
+}
+
+template <int TW, int TH>
+__global__ void __launch_bounds__(32 * FwdShape<TW, TH>::NR, kLightWarpsPerSM / FwdShape<TW, TH>::NR)
+    k_render_fwd_light(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
+                       const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
+                       float* __restrict__ out_rgb, float* __restrict__ out_den, const unsigned* __restrict__ order,
+                       unsigned* __restrict__ counter) {
+    for_each_tile(order, counter, vs.total_tiles, [&](int tile) {
+        fwd_tile_light<TW, TH>(tile, rec, offsets, list, vs, wparams, out_rgb, out_den);
     });
 }
 
@@ -879,29 +1031,42 @@ cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks
     });
 }
 
+// Records per 1024 pixels up to which the kernel for sparse views is taken (the lists' lengths are not known on the
+// host).  It against the other, us: 27 and 43 at 2.2 (8000 Gaussians at 1920x1920), 21 and 27 at 7.9 (16k at
+// 1920x1080), 48 and 56 at 8.9 (32k at 1920x1920), 78 and 73 at 18 (64k); in 8x8 tiles 33 and 40, 23 and 27, 58 and 56,
+// 88 and 78.
+constexpr long long kSparse = 9;
+
+// S slices, or 0: the kernel for sparse views
 template <int TW, int TH, int S>
 cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
-    constexpr int NT = 32 * S * FwdShape<TW, TH>::NR;
+    constexpr int NT = 32 * (S ? S : 1) * FwdShape<TW, TH>::NR;
+    auto kernel = [] {
+        if constexpr (S == 0) return k_render_fwd_light<TW, TH>;
+        else return k_render_fwd<TW, TH, S>;
+    }();
     static PerDevice known;
     int grid = vs.total_tiles;
     if (sched.order) {
         int most = 0;
-        cudaError_t e = resident_blocks(known, k_render_fwd<TW, TH, S>, NT, most);
+        cudaError_t e = resident_blocks(known, kernel, NT, most);
         if (e == cudaSuccess) e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
         grid = min(grid, most);
     }
-    k_render_fwd<TW, TH, S><<<(unsigned)grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb, den,
-                                                sched.order, sched.counter);
+    kernel<<<(unsigned)grid, NT, 0, s>>>(reinterpret_cast<const float4*>(rec), off, list, vs, w.params, rgb, den, sched.order,
+                                         sched.counter);
     return cudaGetLastError();
 }
 
 template <int TW, int TH>
-cudaError_t fwd_t(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
+cudaError_t fwd_t(const float* rec, long long n_records, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
     // Two slices where the tiles alone leave the SMs idle: 14.4 -> 10.4 us at 240 tiles, 14.5 -> 13.7 at 475
     // (40k Gaussians), 14.4 -> 15.1 at 920, 39 -> 70 at 8160.
+    if (vs.total_tiles > kFewTiles && n_records * 1024 <= kSparse * vs.total_tiles * (TW * TH))
+        return fwd_s<TW, TH, 0>(rec, off, list, vs, w, rgb, den, sched, s);
     return vs.total_tiles <= kFewTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
                                             : fwd_s<TW, TH, 1>(rec, off, list, vs, w, rgb, den, sched, s);
 }
@@ -1067,13 +1232,13 @@ cudaError_t sm_count(int& sms) {
     });
 }
 
-cudaError_t launch_render_fwd(const float* rec, const unsigned* off, const unsigned* list, const Views& vs,
+cudaError_t launch_render_fwd(const float* rec, long long n, const unsigned* off, const unsigned* list, const Views& vs,
                               WeightDev w, float* rgb, float* den, Sched sc, cudaStream_t s) {
     if (vs.total_tiles == 0) return cudaSuccess;
-    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8>(rec, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8>(rec, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
     return cudaErrorInvalidValue;
 }
 

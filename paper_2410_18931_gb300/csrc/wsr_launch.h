@@ -115,7 +115,7 @@ struct Sched {
     unsigned* counter;
 };
 
-cudaError_t launch_render_fwd(const float* records, const unsigned* tile_offsets,
+cudaError_t launch_render_fwd(const float* records, long long n, const unsigned* tile_offsets,
                               const unsigned* tile_list, const Views& vs, WeightDev w,
                               float* out_rgb, float* out_den, Sched sched, cudaStream_t s);
 
