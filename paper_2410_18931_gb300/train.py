@@ -162,6 +162,7 @@ class TrainStep:
         dev = self.flat.device
         self.r = Renderer(self.cams, tile=self.tile, persistent=self.persistent, headroom=self.headroom,
                           chunk=self.chunk, deterministic=self.deterministic)
+        self.r.bin_kernels = self.r.bin_launches(self.g.n)
         self.st = self.r.forward(self.g, self.kind, self.wparams)
         self.grad_rgb = torch.empty_like(self.st.rgb)
         self.grad_records = torch.empty(self.r.n_cams * self.g.n * self.r.record_floats, device=dev)
@@ -198,9 +199,9 @@ class TrainStep:
 
     @property
     def kernels_per_step(self) -> int:
-        # project 1, bin (Renderer.bin_launches), fwd 1, loss 1, bwd 1 (and its tile order, where the binning has none),
+        # project 1, bin (bin_kernels), fwd 1, loss 1, bwd 1 (and its tile order, where the binning has none),
         # project bwd 1, Adam 2; deterministic: + the largest-pixel-term kernel and two ordered reductions
-        return 7 + self.r.bin_launches(self.g.n) + (0 if self.persistent else self.r.order_kernels) + (3 if self.deterministic else 0)
+        return 7 + self.r.bin_kernels + (0 if self.persistent else self.r.order_kernels) + (3 if self.deterministic else 0)
 
     def train(self, steps: int, check_every: int = 10) -> torch.Tensor:
         """Make ``steps`` Adam updates; returns the loss triples {L, L1, SSIM}
