@@ -162,7 +162,7 @@ enum {
  *     terms are reduced in tile order;
  *   - wsr_project_bwd, given the same tiles, reads those records and reduces
  *     its sigma/beta terms in a fixed order.
- * The backward then takes about 1.4 times as long.
+ * The backward then takes about 1.25 times as long.
  */
 typedef struct {
     int32_t tile_w, tile_h;
