@@ -621,7 +621,10 @@ constexpr float kMagic = 12582912.0f;       // 1.5 x 2^23
 constexpr int kFewWalk = 64;
 // Chunks per part of a tile's list (1 for few tiles): claiming each chunk on its own costs 20 us at 1M Gaussians.
 constexpr unsigned kPartChunks = 4;
-constexpr int kNoBound = 127;               // deterministic mode: a bound of zero (frexpf gives at most 100 here)
+// Deterministic mode: a bound's exponent in a byte, kExpBias above frexpf's (-148 for the smallest subnormal, at most
+// 100 here), and the byte of a bound of zero.
+constexpr int kExpBias = 24, kNoBound = 127;
+static_assert(-148 + kExpBias >= -128 && 100 + kExpBias < kNoBound, "exponents and kNoBound fit in a byte");
 constexpr int kHelpTiles = 1024;            // tiles whose chunks idle blocks look for (a power of two)
 
 // Schedule: as many blocks as fit on the device take the tiles through *counter (in the order given, longest first,
@@ -931,8 +934,9 @@ __global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::
                                 float* const o = grec + (size_t)kDetRecordFloats * sidx[j] + 18;
                                 auto bound = [&](int c, float m) {
                                     m = fminf(m, 1e30f);
-                                    int e = kNoBound;
+                                    int e = kNoBound - kExpBias;
                                     if (m > 0.0f) frexpf(m, &e);    // m < 2^e
+                                    e += kExpBias;
                                     s_exp[warp][grp][c] = (signed char)e;
                                     return m;
                                 };
@@ -955,7 +959,7 @@ __global__ void __launch_bounds__(BwdThreads<CH>::value, 1024 / BwdThreads<CH>::
                                 const unsigned ri = s_rec[warp][gi];
                                 if (ri != 0xffffffffu && e != kNoBound)
                                     atomicAdd(reinterpret_cast<unsigned long long*>(grec + (size_t)kDetRecordFloats * ri) + c,
-                                              (unsigned long long)fixed_point(s_val[warp][gi][c], kDetBits - e));
+                                              (unsigned long long)fixed_point(s_val[warp][gi][c], kDetBits + kExpBias - e));
                             }
                             __syncwarp();
                         }
