@@ -282,7 +282,7 @@ static wsr_status bin_count_impl(const float* records, int64_t n, const Views& v
     WsHeader* hdr = (WsHeader*)ws;
     unsigned* cursor = (unsigned*)(ws + L.cursor);
     unsigned* bsum = (unsigned*)(ws + L.block_sums);
-    WSR_CUDA(launch_bin_count(records, n, vs, cursor, bin_base(L, workspace), s));
+    WSR_CUDA(launch_bin_count(records, n, vs, cursor, bin_base(L, workspace), capacity, s));
     const bool persistent = vs.schedule == WSR_SCHEDULE_PERSISTENT;
     WSR_CUDA(launch_scan(vs, cursor, bsum, tile_offsets, capacity, hdr, (unsigned*)(ws + L.buckets),
                          persistent ? (unsigned*)(ws + L.order) : nullptr, s));

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ rec, lon
 // every tile of its view.  Block b of a view takes the batches of 32 Gaussians b, b + B, ... (its warps
 // one after another as they come free) in both passes.  COUNT: the block's counts per tile, then one
 // global atomic per tile that it reaches; what that returns, the block's first place among the tile's
-// instances, is kept in `base` (a row of T entries per block).  SCATTER: the block's cursors start at
+// instances, is kept in `base` (a row of T entries per block; nullptr: not asked for).  SCATTER: the block's cursors start at
 // the tile's offset plus that place, so a slot costs one shared atomic.
 //   The global counters bound the plain pass: neighbouring tiles share 32-byte sectors, and a view's
 // counters are only a few kilobytes, so the atomics of all SMs queue at a few L2 lines.  Measured, count,
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(NT, NT > 768 ? 1 : 2)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lw = __ffs(vs.tile_w) - 1, lh = __ffs(vs.tile_h) - 1;   // tile sides are powers of two
     cursor += V.tile_base;
-    base += (size_t)V.tile_base * gridDim.x + (size_t)blockIdx.x * T;
+    if (base) base += (size_t)V.tile_base * gridDim.x + (size_t)blockIdx.x * T;
     if (threadIdx.x == 0) s_next = 0;
     // (four tiles per thread at a time, so that their loads, or below their atomics, are in flight together)
     for (int t0 = threadIdx.x; t0 < T; t0 += 4 * NT) {
@@ -259,6 +259,11 @@ __global__ void __launch_bounds__(NT, NT > 768 ? 1 : 2)
     }
     if constexpr (!SCATTER) {
         __syncthreads();
+        if (base == nullptr) {
+            for (int t = threadIdx.x; t < T; t += NT)
+                if (const unsigned c = cnt[t]) atomicAdd(cursor + t, c);
+            return;
+        }
         for (int t0 = threadIdx.x; t0 < T; t0 += 4 * NT) {
             unsigned c[4], b[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
@@ -800,16 +805,18 @@ cudaError_t launch_tile_order(const Views& vs, const unsigned* offsets, unsigned
 // Blocks per view and threads of k_bin_local, 0 blocks when its counters do not fit in shared memory.
 struct LocalBin {
     int blocks, threads;
+    bool scatter;               // the scatter too takes its counters (scatter_local)
     size_t smem;
 };
 
-static LocalBin local_bin(const Views& vs, long long n) {
-    LocalBin L{0, 0, 0};
+static LocalBin local_bin(const Views& vs, long long n, unsigned long long capacity) {
+    LocalBin L{0, 0, false, 0};
     int t_max = 0;
     for (int v = 0; v < vs.n; ++v) t_max = max(t_max, vs.v[v].tiles_x * vs.v[v].tiles_y);
     L.blocks = bin_blocks_per_view(vs.n, t_max);
     if (L.blocks == 0) return L;
     L.threads = t_max <= kLocalTilesTwo ? 768 : 1024;
+    L.scatter = scatter_local(t_max, capacity);
     // a small scene is spread over more SMs: eight batches of 32 per block
     const long long want = (n + 255) / 256;
     if (want < L.blocks) L.blocks = (int)max(want, 1ll);
@@ -868,11 +875,12 @@ cudaError_t launch_bin_one(const float* records, long long n, const Views& vs, u
 }
 
 cudaError_t launch_bin_count(const float* records, long long n, const Views& vs, unsigned* cursor, unsigned* base,
-                             cudaStream_t s) {
+                             unsigned long long capacity, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned) * (size_t)vs.total_tiles, s);
     if (e != cudaSuccess || n == 0) return e;
-    const LocalBin L = local_bin(vs, n);
+    const LocalBin L = local_bin(vs, n, capacity);
     if (base && L.blocks) {
+        if (!L.scatter) base = nullptr;
         return L.threads == 768
                    ? launch_bin_local<768, false>(L, records, n, vs, cursor, base, nullptr, 0ull, nullptr, s)
                    : launch_bin_local<1024, false>(L, records, n, vs, cursor, base, nullptr, 0ull, nullptr, s);
@@ -927,8 +935,8 @@ cudaError_t launch_bin_scatter(const float* records, long long n, const Views& v
                                unsigned* base, unsigned* list, unsigned long long capacity, WsHeader* hdr,
                                cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    const LocalBin L = local_bin(vs, n);
-    if (base && L.blocks && capacity <= kLocalList) {
+    const LocalBin L = local_bin(vs, n, capacity);
+    if (base && L.blocks && L.scatter) {
         return L.threads == 768 ? launch_bin_local<768, true>(L, records, n, vs, cursor, base, list, capacity, hdr, s)
                                 : launch_bin_local<1024, true>(L, records, n, vs, cursor, base, list, capacity, hdr, s);
     }

@@ -62,10 +62,20 @@ cudaError_t launch_project_bwd(const GaussPtrs& g, const Views& vs, WeightDev w,
 constexpr int kLocalTilesTwo = 12288;
 constexpr int kLocalTiles = 40960;
 constexpr int kLocalSMs = 152;
-// Its scatter serves lists of up to 2^25 entries, the size of L2: each block fills its own run of a tile's
-// segment, so every line of the list stays open for the whole pass.  Measured against the scatter with global
-// counters: 304 and 399 us for 25M instances, 645 and 524 us for 38M (1920x1080), 569 and 283 us for 34M (3840x2160).
+// Its scatter fills a run of a tile's segment per block, so every run's line stays open for the whole pass: past the
+// size of L2 it loses to the scatter with global counters.  At two blocks per SM that is a list of 2^25 entries.  At
+// one the runs count too, a third of their 32-byte sectors beside the list: both take as long at 27M entries in 14400
+// tiles and at 20M to 22M in 32400 (the rule: 26.8M and 20.4M).  Whole binning, us, these counters and the global
+// ones: 1920x1080 410 and 509 for 25M, 661 and 649 for 33M, 645 and 524 for 38M; 2560x1440 268 and 331 for 20M, 587
+// and 488 for 33M; 3840x2160 120 and 156 for 10M, 270 and 264 for 20M, 377 and 329 for 25M, 678 and 435 for 33M (2^25
+// entries whatever the tiles: 657, 447 with global counters in both passes).  The list's length is not known when the
+// launch is made: its capacity is taken as a quarter above it there, as callers leave it room to grow.
 constexpr unsigned long long kLocalList = 1ull << 25;
+inline bool scatter_local(int t_max, unsigned long long capacity) {
+    if (t_max <= kLocalTilesTwo) return capacity <= kLocalList;
+    const unsigned long long l2 = 134000000ull, runs = 32ull * kLocalSMs * (unsigned)t_max;
+    return capacity <= kLocalList && capacity / 5 * 16 <= l2 - runs / 3;
+}
 
 // Blocks per view of k_bin_local for views of at most t_max tiles (0: not used)
 inline int bin_blocks_per_view(int n_views, int t_max) {
@@ -87,9 +97,10 @@ cudaError_t launch_bin_one(const float* records, long long n, const Views& vs, u
                            unsigned long long capacity, WsHeader* hdr, unsigned* order, cudaStream_t s);
 
 // base: nullptr (global counters only), or total_tiles x bin_blocks_per_view words that carry each block's
-// places from the count to the scatter (pass the same to both)
-cudaError_t launch_bin_count(const float* records, long long n, const Views& vs,
-                             unsigned* cursor, unsigned* base, cudaStream_t s);
+// places from the count to the scatter (pass the same base and capacity to both; a count that no scatter follows
+// passes the largest capacity)
+cudaError_t launch_bin_count(const float* records, long long n, const Views& vs, unsigned* cursor, unsigned* base,
+                             unsigned long long capacity, cudaStream_t s);
 // the scan of the per-tile counts into offsets (and the scatter's cursors); with `order`, also
 // the persistent schedule's longest-first tile order (`buckets`: 66 words of scratch)
 cudaError_t launch_scan(const Views& vs, unsigned* cursor, unsigned* block_sums,
