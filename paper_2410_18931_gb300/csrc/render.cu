@@ -111,8 +111,9 @@ struct TileShape {
 // staging and a warp per region.  One block per tile: 566 -> 399 us, 95 -> 60 us for 200k at 1280x720.
 //   20 warps per SM (at most 96 registers a thread): 363 us against 367 at 16, 379 at 24 and 389 at 28.
 constexpr int kFwdWarpsPerSM = 20;
-// The kernel for sparse views: 48 registers a thread, about as fast with 32 and 48 warps.
-constexpr int kLightWarpsPerSM = 40;
+// The kernel for sparse views, 64 registers a thread: with 40 warps (48 registers, 8 bytes spilled) 8000 Gaussians at
+// 1920x1080 take 13.2 us instead of 12.1, wide ones 65 instead of 57.
+constexpr int kLightWarpsPerSM = 32;
 
 template <int TW, int TH>
 struct FwdShape {
@@ -120,13 +121,13 @@ struct FwdShape {
     static_assert(TW % 8 == 0 && TH % 8 == 0 && NR <= 4, "whole regions");
 };
 
-// Which of the tile's 8x8 regions a footprint q' <= kQMax can reach, one bit each (row by row); (gx, gy) is the
-// tile's first pixel centre less the mean.  Eight pixel rows cut the ellipse in a convex part whose x-extent
+// Which of RX x RY regions of RW x 8 pixels a footprint q' <= kQMax can reach, one bit each (row by row); (gx, gy) is
+// the first region's first pixel centre less the mean.  Eight pixel rows cut the ellipse in a convex part whose x-extent
 // [x_l, x_r] has a closed form (as in the binning: x(dy) = (-B' dy +- sqrt(A' QM - det' dy^2)) / A' at the row
 // of the band nearest the ellipse's rightmost and leftmost point); a region is reached when that extent,
 // widened far beyond its rounding, meets the region's pixel-centre columns.  Every comparison is "not outside":
 // NaN counts as reached.
-template <int RX, int RY>
+template <int RX, int RY, int RW = 8>
 __device__ __forceinline__ unsigned regions_hit(const float4 a, const float qd, const float gx, const float gy) {
     const float QM = kQMax * 1.0001f + 1e-4f;
     const float A = fmaf(a.w, a.w, qd), ia = rcp_approx(A), det = qd * a.z * a.z, aq = A * QM;
@@ -144,7 +145,7 @@ __device__ __forceinline__ unsigned regions_hit(const float4 a, const float qd, 
         const bool out = det * dn * dn > aq * 1.001f;
 #pragma unroll
         for (int c = 0; c < RX; ++c)
-            if (!(out || xl > gx + (float)(8 * c + 7) || xr < gx + (float)(8 * c))) hit |= 1u << (b * RX + c);
+            if (!(out || xl > gx + (float)(RW * c + RW - 1) || xr < gx + (float)(RW * c))) hit |= 1u << (b * RX + c);
     }
     return hit;
 }
@@ -195,6 +196,45 @@ __device__ __forceinline__ void store_pair(const View& V, const bool aligned, co
         o[4] = p1.y;
         o[5] = p1.z;
         out_den[pix + 1] = p1.w;
+    }
+}
+
+// The same where not every row starts on eight bytes (an odd width or an odd first pixel), by all lanes of a warp: rows
+// that start at an odd pixel pair their columns one further on.  `next` is the lane that holds the columns to the
+// right, and for the last lane of a row (`last`) the first, WIDTH columns before those.
+template <int WIDTH>
+__device__ __forceinline__ void store_shifted(const View& V, const int next, const bool last, const int x, const int y,
+                                              const float4 p0, const float4 p1, float* __restrict__ out_rgb,
+                                              float* __restrict__ out_den) {
+    const long long row = V.pix_base + (long long)y * V.W;
+    const bool aligned = ((reinterpret_cast<size_t>(out_rgb) | reinterpret_cast<size_t>(out_den)) & 7) == 0;
+    const bool off = ((row + x) & 1) != 0;
+    const float4 nx = make_float4(__shfl_sync(0xffffffffu, p0.x, next), __shfl_sync(0xffffffffu, p0.y, next),
+                                  __shfl_sync(0xffffffffu, p0.z, next), __shfl_sync(0xffffffffu, p0.w, next));
+    if (y >= V.H) return;
+    const float4 a = off ? p1 : p0, b = off ? nx : p1;
+    const int xa = off ? x + 1 : x, xb = off ? (last ? x + 2 - WIDTH : x + 2) : x + 1;
+    if (aligned && xb == xa + 1 && xb < V.W) {
+        float2* const o = reinterpret_cast<float2*>(out_rgb + 3 * (row + xa));
+        o[0] = f2(a.x, a.y);
+        o[1] = f2(a.z, b.x);
+        o[2] = f2(b.y, b.z);
+        *reinterpret_cast<float2*>(out_den + row + xa) = f2(a.w, b.w);
+        return;
+    }
+    if (xa < V.W) {
+        float* const o = out_rgb + 3 * (row + xa);
+        o[0] = a.x;
+        o[1] = a.y;
+        o[2] = a.z;
+        out_den[row + xa] = a.w;
+    }
+    if (xb < V.W) {
+        float* const o = out_rgb + 3 * (row + xb);
+        o[0] = b.x;
+        o[1] = b.y;
+        o[2] = b.z;
+        out_den[row + xb] = b.w;
     }
 }
 
@@ -377,128 +417,135 @@ __device__ __forceinline__ void fwd_tile(const int tile, const float4* __restric
                pixel_out(sum[1], wparams), out_rgb, out_den);
 }
 
+// The kernel for sparse views: a warp per 16x8 pixels (8x8 in tiles of that width).
+template <int TW, int TH>
+struct LightShape {
+    static constexpr int RW = TW == 8 ? 8 : 16, RX = TW / RW, NR = RX * (TH / 8);
+    static constexpr int COLS = RW / 8;     // columns per thread, of two rows; eight lanes across
+    static_assert(TW % RW == 0 && TH % 8 == 0, "whole regions");
+};
+
 // Forward for sparse views, where a tile's time is the latency of its chain (offsets, list, records, pixels) and not
-// its arithmetic: a warp per 8x8 region as above, two pixels of a row per thread, the region's Gaussians one after
-// another.  Eight accumulators instead of 32 and no loads ahead, so
-// that twice the warps fit on an SM: 8000 Gaussians at 1920x1920 43 -> 27 us, 32,000 55 -> 47 us.
+// its arithmetic: a warp per region, each staging the tile's list on its own (no barrier between warps), two rows and
+// one or two columns per thread, the Gaussians that reach the region one after another.  A quarter to a half of the
+// kernel above's accumulators, so that 32 warps fit on an SM.
+//   With a warp per 8x8 pixels, two columns of one row per thread and batches staged by the block it took 1920x1080,
+// us: 8000 Gaussians 15.7 -> 12.1, 16000 19.7 -> 16.4 (and 22.2 -> 17.8 at 1919x1079), 4.5 times as wide 70 -> 57 and
+// 133 -> 108, 12 times as wide 394 -> 303; 16000 at 3840x2160 66 -> 48; in 8x8 tiles 16000 22 -> 19.3, wide 144 -> 109.
 template <int TW, int TH>
 __device__ __forceinline__ void fwd_tile_light(const int tile, const float4* __restrict__ rec,
                                                const unsigned* __restrict__ offsets, const unsigned* __restrict__ list,
                                                const Views& vs, const float* __restrict__ wparams,
                                                float* __restrict__ out_rgb, float* __restrict__ out_den) {
-    using F = FwdShape<TW, TH>;
-    constexpr int RX = F::RX, NR = F::NR, BATCH = 32 * NR;
-    __shared__ float4 g[BATCH][3];                      // walk constants, as in FwdStage
-    __shared__ unsigned hits[NR][NR];
+    using F = LightShape<TW, TH>;
+    constexpr int COLS = F::COLS;
+    __shared__ float4 s_g[F::NR][32][3];                // walk constants, as in FwdStage
     const unsigned start = offsets[tile], end = offsets[tile + 1];
     const TileCoord tc = tile_coord(vs, tile);
     const View& V = vs.v[tc.v];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float4(*const g)[3] = s_g[w];
     const int x_org = tc.tx * TW, y_org = tc.ty * TH;
-    const int lx = 8 * (w % RX) + 2 * (lane & 3), ly = 8 * (w / RX) + (lane >> 2);
+    const int rx = F::RW * (w % F::RX), ry = 8 * (w / F::RX);               // the warp's region
+    const int lx = rx + COLS * (lane & 7), ly = ry + 2 * (lane >> 3);
     const float2 ox = f2((float)lx, (float)(lx + 1));
     const float oy = (float)ly;
-    auto sync = [&] {
-        if constexpr (NR == 1) __syncwarp();
-        else __syncthreads();
-    };
-    float2 rg[2], bd[2];                                // per column: (N_r, N_g) and (N_b, D)
-    rg[0] = rg[1] = bd[0] = bd[1] = f2(0.f, 0.f);
-    for (unsigned base = start; base < end; base += BATCH) {
-        if (base != start) sync();                      // the batch before is walked
-        if (base + 32 * w < end) {
-            const bool in = base + threadIdx.x < end;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            float cb = 0.f;
-            if (in) {
-                const float4* p = rec + 3ull * list[base + threadIdx.x];
-                a = __ldg(p);
-                b = __ldg(p + 1);
-                cb = __ldg(reinterpret_cast<const float*>(p + 2));
-            }
-            const float gx = (float)x_org + 0.5f - a.x, gy = (float)y_org + 0.5f - a.y;
-            g[threadIdx.x][0] = make_float4(a.z, a.w, fmaf(a.z, gy, a.w * gx), b.x);
-            g[threadIdx.x][1] = make_float4(b.x * gx * gx, 2.0f * b.x * gx, b.z, b.w);
-            *reinterpret_cast<float2*>(&g[threadIdx.x][2]) = f2(cb, b.y);
-            const unsigned hit = in ? regions_hit<RX, F::RY>(a, b.x, gx, gy) : 0u;
+    float2 rg[2][COLS], bd[2][COLS];                    // per row and column: (N_r, N_g) and (N_b, D)
 #pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const unsigned bal = __ballot_sync(0xffffffffu, (hit >> k) & 1u);
-                if (lane == 0) hits[k][w] = bal;
-            }
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) rg[r][c] = bd[r][c] = f2(0.f, 0.f);
+    auto add = [&](const float q, const float2 crg, const float2 cbuw, float2& o_rg, float2& o_bd) {
+        if (q <= kQMax) {
+            const float e = ex2_approx(-q);
+            o_rg = __ffma2_rn(crg, f2(e, e), o_rg);
+            o_bd = __ffma2_rn(cbuw, f2(e, e), o_bd);
         }
-        sync();
-        for (int k = 0; k < NR && base + 32 * k < end; ++k) {
-            for (unsigned bal = hits[w][k]; bal; bal &= bal - 1) {
-                const float4* e = g[32 * k + __ffs(bal) - 1];
-                const float4 u = e[0], t = e[1];
-                const float2 cbuw = *reinterpret_cast<const float2*>(e + 2);
-                const float2 crg = f2(t.z, t.w);
-                // q' in the same operations as above
+    };
+    // the next batch's records are loaded while this one is walked, and the list entries of the one after that
+    unsigned nidx = start + lane < end ? list[start + lane] : 0u;
+    float4 na, nb;
+    float ncb;
+    auto fetch = [&](unsigned b) {
+        na = nb = make_float4(0.f, 0.f, 0.f, 0.f);
+        ncb = 0.f;
+        if (b + lane < end) {
+            const float4* p = rec + 3ull * nidx;
+            na = __ldg(p);
+            nb = __ldg(p + 1);
+            ncb = __ldg(reinterpret_cast<const float*>(p + 2));
+        }
+        nidx = b + 32 + lane < end ? list[b + 32 + lane] : 0u;
+    };
+    fetch(start);
+    for (unsigned base = start; base < end; base += 32) {
+        const float4 a = na, b = nb;
+        const float gx = (float)x_org + 0.5f - a.x, gy = (float)y_org + 0.5f - a.y;
+        // (the binning has tested a tile that is one region)
+        const bool hit = base + lane < end &&
+                         (F::NR == 1 || regions_hit<1, 1, F::RW>(a, b.x, gx + (float)rx, gy + (float)ry));
+        const unsigned bal = __ballot_sync(0xffffffffu, hit);
+        if (hit) {
+            float4* const o = g[__popc(bal & ((1u << lane) - 1u))];
+            o[0] = make_float4(a.z, a.w, fmaf(a.z, gy, a.w * gx), b.x);
+            o[1] = make_float4(b.x * gx * gx, 2.0f * b.x * gx, b.z, b.w);
+            *reinterpret_cast<float2*>(o + 2) = f2(ncb, b.y);
+        }
+        fetch(base + 32);
+        __syncwarp();
+        const int nj = __popc(bal);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
+            const float4 u = g[j][0], t = g[j][1];
+            const float2 cbuw = *reinterpret_cast<const float2*>(&g[j][2]);
+            const float2 crg = f2(t.z, t.w);
+            // q' by the operations of the kernel above (and so the same pairs): there the columns are paired in tiles
+            // of every width, here the rows where a thread has one column
+            if constexpr (COLS == 1) {
+                const float P = fmaf(ox.x, fmaf(ox.x, u.w, t.y), t.x), rx = fmaf(u.y, ox.x, u.z);
+                const float2 rr = __ffma2_rn(f2(u.x, u.x), f2(oy, oy + 1.0f), f2(rx, rx));
+                const float2 q = __ffma2_rn(rr, rr, f2(P, P));
+                add(q.x, crg, cbuw, rg[0][0], bd[0][0]);
+                add(q.y, crg, cbuw, rg[1][0], bd[1][0]);
+            } else {
                 const float2 P = __ffma2_rn(ox, __ffma2_rn(ox, f2(u.w, u.w), f2(t.y, t.y)), f2(t.x, t.x));
-                float2 rr;
-                if constexpr (TW == 8) {
-                    rr = __ffma2_rn(f2(u.x, u.x), f2(oy, oy), __ffma2_rn(f2(u.y, u.y), ox, f2(u.z, u.z)));
-                } else {
-                    const float ry = fmaf(u.x, oy, u.z);
-                    rr = __ffma2_rn(f2(u.y, u.y), ox, f2(ry, ry));
-                }
-                const float2 q = __ffma2_rn(rr, rr, P);
-                if (q.x <= kQMax) {
-                    const float e0 = ex2_approx(-q.x);
-                    rg[0] = __ffma2_rn(crg, f2(e0, e0), rg[0]);
-                    bd[0] = __ffma2_rn(cbuw, f2(e0, e0), bd[0]);
-                }
-                if (q.y <= kQMax) {
-                    const float e1 = ex2_approx(-q.y);
-                    rg[1] = __ffma2_rn(crg, f2(e1, e1), rg[1]);
-                    bd[1] = __ffma2_rn(cbuw, f2(e1, e1), bd[1]);
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float ry = fmaf(u.x, oy + (float)r, u.z);
+                    const float2 rr = __ffma2_rn(f2(u.y, u.y), ox, f2(ry, ry));
+                    const float2 q = __ffma2_rn(rr, rr, P);
+                    add(q.x, crg, cbuw, rg[r][0], bd[r][0]);
+                    add(q.y, crg, cbuw, rg[r][COLS - 1], bd[r][COLS - 1]);
                 }
             }
         }
+        __syncwarp();                                   // the batch is walked: the next may be written
     }
-    const float4 p0 = pixel_out(make_float4(rg[0].x, rg[0].y, bd[0].x, bd[0].y), wparams);
-    const float4 p1 = pixel_out(make_float4(rg[1].x, rg[1].y, bd[1].x, bd[1].y), wparams);
-    if (pairs_aligned(V, out_rgb, out_den)) {
-        store_pair(V, true, x_org + lx, y_org + ly, p0, p1, out_rgb, out_den);
-        return;
-    }
-    // Rows that start at an odd pixel pair their columns one further on; the last lane's two pixels stand alone.  At
-    // 1919x1919, word stores -> these: an empty image 39 -> 25 us, 8000 Gaussians 39 -> 33, 32k 53 -> 53, in 8x8 tiles
-    // 58 -> 59 (the rows through shared memory instead: 23, 33, 58 and 66).
-    const int x = x_org + lx, y = y_org + ly;
-    const long long pix = V.pix_base + (long long)y * V.W + x;
-    const bool off = (pix & 1) != 0 || ((reinterpret_cast<size_t>(out_rgb) | reinterpret_cast<size_t>(out_den)) & 7) != 0;
-    const int from = (lane & ~3) | ((lane + 1) & 3);
-    const float4 nx = make_float4(__shfl_sync(0xffffffffu, p0.x, from), __shfl_sync(0xffffffffu, p0.y, from),
-                                  __shfl_sync(0xffffffffu, p0.z, from), __shfl_sync(0xffffffffu, p0.w, from));
-    if (y >= V.H) return;
-    const bool last = (lane & 3) == 3;
-    const float4 a = off ? p1 : p0, b = off ? nx : p1;
-    const int xa = off ? x + 1 : x, xb = off ? (last ? x - 6 : x + 2) : x + 1;
-    const long long row = V.pix_base + (long long)y * V.W;
-    const bool aligned = ((reinterpret_cast<size_t>(out_rgb) | reinterpret_cast<size_t>(out_den)) & 7) == 0;
-    if (aligned && xb == xa + 1 && xb < V.W) {
-        float2* const o = reinterpret_cast<float2*>(out_rgb + 3 * (row + xa));
-        o[0] = f2(a.x, a.y);
-        o[1] = f2(a.z, b.x);
-        o[2] = f2(b.y, b.z);
-        *reinterpret_cast<float2*>(out_den + row + xa) = f2(a.w, b.w);
-        return;
-    }
-    if (xa < V.W) {
-        float* const o = out_rgb + 3 * (row + xa);
-        o[0] = a.x;
-        o[1] = a.y;
-        o[2] = a.z;
-        out_den[row + xa] = a.w;
-    }
-    if (xb < V.W) {
-        float* const o = out_rgb + 3 * (row + xb);
-        o[0] = b.x;
-        o[1] = b.y;
-        o[2] = b.z;
-        out_den[row + xb] = b.w;
+    const bool pairs = pairs_aligned(V, out_rgb, out_den);
+    float4 px[2][COLS];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < COLS; ++c)
+            px[r][c] = pixel_out(make_float4(rg[r][c].x, rg[r][c].y, bd[r][c].x, bd[r][c].y), wparams);
+    if constexpr (COLS == 1) {
+        // two lanes side by side: the even one takes both columns of the first row, the odd one of the second
+        const bool odd = lane & 1;
+        const float4 give = odd ? px[0][0] : px[1][0], mine = odd ? px[1][0] : px[0][0];
+        const float4 got = make_float4(__shfl_xor_sync(0xffffffffu, give.x, 1), __shfl_xor_sync(0xffffffffu, give.y, 1),
+                                       __shfl_xor_sync(0xffffffffu, give.z, 1), __shfl_xor_sync(0xffffffffu, give.w, 1));
+        const float4 p0 = odd ? got : mine, p1 = odd ? mine : got;
+        const int x = x_org + (lx & ~1), y = y_org + ly + odd;
+        if (pairs) store_pair(V, true, x, y, p0, p1, out_rgb, out_den);
+        else store_shifted<8>(V, (lane & ~7) | ((lane + 2) & 7), (lane & 7) >= 6, x, y, p0, p1, out_rgb, out_den);
+    } else {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const float4 p0 = px[r][0], p1 = px[r][COLS - 1];
+            const int x = x_org + lx, y = y_org + ly + r;
+            if (pairs) store_pair(V, true, x, y, p0, p1, out_rgb, out_den);
+            else store_shifted<16>(V, (lane & ~7) | ((lane + 1) & 7), (lane & 7) == 7, x, y, p0, p1, out_rgb, out_den);
+        }
     }
 }
 
@@ -533,7 +580,7 @@ __global__ void __launch_bounds__(32 * S * FwdShape<TW, TH>::NR, kFwdWarpsPerSM 
 }
 
 template <int TW, int TH>
-__global__ void __launch_bounds__(32 * FwdShape<TW, TH>::NR, kLightWarpsPerSM / FwdShape<TW, TH>::NR)
+__global__ void __launch_bounds__(32 * LightShape<TW, TH>::NR, kLightWarpsPerSM / LightShape<TW, TH>::NR)
     k_render_fwd_light(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
                        const unsigned* __restrict__ list, const Views vs, const float* __restrict__ wparams,
                        float* __restrict__ out_rgb, float* __restrict__ out_den, const unsigned* __restrict__ order,
@@ -1047,16 +1094,23 @@ cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks
 }
 
 // Records per 1024 pixels up to which the kernel for sparse views is taken (the lists' lengths are not known on the
-// host).  It against the other, us: 27 and 43 at 2.2 (8000 Gaussians at 1920x1920), 21 and 27 at 7.9 (16k at
-// 1920x1080), 48 and 56 at 8.9 (32k at 1920x1920), 78 and 73 at 18 (64k); in 8x8 tiles 33 and 40, 23 and 27, 58 and 56,
-// 88 and 78.
+// host).  It against the other at 1920x1080, us, for Gaussians of three sizes (the second and third 4.5 and 12 times as
+// wide as the first):
+//   500 (0.25 per 1024)   9.4 and 17.5   11.4 and 24    26.5 and 36
+//   8000 (4)             12.1 and 23     57 and 56      303 and 264
+//   16000 (8)            16.4 and 26    108 and 95
+//   32000 (16)           25.7 and 31    213 and 174     (not taken)
+// in 8x8 tiles 19.3 and 25 and 109 and 106 at 16000, 26 and 32 and 209 and 193 at 32000; 16000 in two clusters of a
+// hundred tiles 151 and 85.  So where it is taken it loses at most a seventh to lists of hundreds of entries, and past
+// the limit wide Gaussians would lose more than narrow ones gain.  Deciding per tile (lists past 64 entries left to a
+// second launch of the other kernel) gives the clusters 79 us, and takes 1.7 to 2 us from every sparse view.
 constexpr long long kSparse = 9;
 
 // S slices, or 0: the kernel for sparse views
 template <int TW, int TH, int S>
 cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
-    constexpr int NT = 32 * (S ? S : 1) * FwdShape<TW, TH>::NR;
+    constexpr int NT = S ? 32 * S * FwdShape<TW, TH>::NR : 32 * LightShape<TW, TH>::NR;
     auto kernel = [] {
         if constexpr (S == 0) return k_render_fwd_light<TW, TH>;
         else return k_render_fwd<TW, TH, S>;
