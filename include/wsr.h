@@ -465,11 +465,15 @@ wsr_status wsr_bin_static(const float* records, int64_t n, const wsr_camera* cam
  *   [1] (pixel, Gaussian) slots wsr_render_fwd evaluates: it walks the
  *       Gaussians that reach an 8x8 region of a tile four at a time, so 256
  *       slots per round of four (of each batch of the tile's list), the last
- *       round's idle quarters included; 64 per Gaussian in 8x8 tiles;
+ *       round's idle quarters included but in 8x8 tiles (64 per Gaussian);
+ *       in sparse views (few records for their pixels, more than 608 tiles)
+ *       it walks them one at a time: 128 slots for each 16x8 region that a
+ *       Gaussian of the tile reaches, 64 per Gaussian in 8x8 tiles;
  *   [2] (pixel, Gaussian) slots wsr_render_bwd evaluates: for each Gaussian
  *       of a tile, the rows that its footprint reaches, each of tile width
  *       columns, or of half the tile width when no row needs more.
- * Arguments as for wsr_render_fwd.  Not part of a timed step.
+ * Arguments as for wsr_render_fwd (n selects the kernel there, and its count
+ * here).  Not part of a timed step.
  */
 wsr_status wsr_count_pairs(const float* records, int64_t n, const uint32_t* tile_offsets,
                            const uint32_t* tile_list, const wsr_camera* cams, int32_t n_cams,

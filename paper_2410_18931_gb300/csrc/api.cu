@@ -486,7 +486,7 @@ wsr_status wsr_count_pairs(const float* records, int64_t n, const uint32_t* tile
     if (!aligned16(records) || !aligned4(tile_list) || !aligned4(tile_offsets) || ((uintptr_t)count_dev & 7u))
         return WSR_ERR_INVALID_ARG;
     WSR_TRY(make_views(cams, n_cams, tiles, &vs));
-    return cuda_status(launch_count_pairs(records, tile_offsets, tile_list, vs, (unsigned long long*)count_dev,
+    return cuda_status(launch_count_pairs(records, n, tile_offsets, tile_list, vs, (unsigned long long*)count_dev,
                                           (cudaStream_t)stream));
 }
 

@@ -1105,6 +1105,9 @@ cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks
 // the limit wide Gaussians would lose more than narrow ones gain.  Deciding per tile (lists past 64 entries left to a
 // second launch of the other kernel) gives the clusters 79 us, and takes 1.7 to 2 us from every sparse view.
 constexpr long long kSparse = 9;
+inline bool sparse_view(const Views& vs, const long long n_records) {
+    return vs.total_tiles > kFewTiles && n_records * 1024 <= kSparse * vs.total_tiles * (vs.tile_w * vs.tile_h);
+}
 
 // S slices, or 0: the kernel for sparse views
 template <int TW, int TH, int S>
@@ -1134,7 +1137,7 @@ cudaError_t fwd_t(const float* rec, long long n_records, const unsigned* off, co
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
     // Two slices where the tiles alone leave the SMs idle: 14.4 -> 10.4 us at 240 tiles, 14.5 -> 13.7 at 475
     // (40k Gaussians), 14.4 -> 15.1 at 920, 39 -> 70 at 8160.
-    if (vs.total_tiles > kFewTiles && n_records * 1024 <= kSparse * vs.total_tiles * (TW * TH))
+    if (sparse_view(vs, n_records))
         return fwd_s<TW, TH, 0>(rec, off, list, vs, w, rgb, den, sched, s);
     return vs.total_tiles <= kFewTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
                                             : fwd_s<TW, TH, 1>(rec, off, list, vs, w, rgb, den, sched, s);
@@ -1176,15 +1179,19 @@ cudaError_t bwd_t(const float* rec, const unsigned* off, const unsigned* list, c
 //       within rounding of the cutoff differently);
 //   [1] the (pixel, Gaussian) slots the forward evaluates: per batch of a
 //       tile's list and 8x8 region, rounds of four Gaussians that reach the
-//       region (its own test), 256 slots each; 64 per Gaussian in 8x8 tiles;
+//       region (its own test), 256 slots each, in 8x8 tiles without the idle
+//       quarters of the last one; in sparse views (`light`) the pixels of
+//       each region of that kernel that a Gaussian reaches;
 //   [2] the backward's pixel slots (per tile instance, the rows its footprint
 //       reaches, TW columns each, or TW / 2 when no row needs more), from the
 //       backward's own arithmetic.
 template <int TW, int TH, int PPT>
 __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
     k_count_pairs(const float4* __restrict__ rec, const unsigned* __restrict__ offsets,
-                  const unsigned* __restrict__ list, const Views vs, unsigned long long* __restrict__ count) {
+                  const unsigned* __restrict__ list, const Views vs, const bool light,
+                  unsigned long long* __restrict__ count) {
     using S = TileShape<TW, TH, PPT>;
+    using G = LightShape<TW, TH>;
     constexpr int NT = S::NT;
     using F = FwdShape<TW, TH>;
     static_assert(NT == 32 * F::NR, "the forward's batches");
@@ -1214,7 +1221,13 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
             const float qd = __ldg(reinterpret_cast<const float*>(p + 1));
             s0[tid] = a;
             s1[tid] = qd;
-            hit = regions_hit<F::RX, F::RY>(a, qd, (float)x_org + 0.5f - a.x, (float)y_org + 0.5f - a.y);
+            const float gx = (float)x_org + 0.5f - a.x, gy = (float)y_org + 0.5f - a.y;
+            if (!light) hit = regions_hit<F::RX, F::RY>(a, qd, gx, gy);
+            else if (G::NR == 1) cnt_fwd += G::RW * 8;
+            else
+                for (int k = 0; k < G::NR; ++k)         // one region at a time, as its warps do
+                    cnt_fwd += G::RW * 8 * regions_hit<1, 1, G::RW>(a, qd, gx + (float)(G::RW * (k % G::RX)),
+                                                                    gy + (float)(8 * (k / G::RX)));
             // the backward's pixel slots: the rows its footprint reaches, TW or TW / 2 columns each
             int first, nst;
             bool wide;
@@ -1229,7 +1242,7 @@ __global__ void __launch_bounds__(TileShape<TW, TH, PPT>::NT)
             if ((tid & 31) == 0 && bal) atomicAdd(&s_n[k], (unsigned)__popc(bal));
         }
         __syncthreads();
-        // the forward's rounds over this batch: 256 slots each (one region per tile: 64 per Gaussian)
+        // the forward's rounds over this batch: 256 slots each (one region per tile: 64 per Gaussian; none if light)
         if (tid < F::NR) cnt_fwd += F::NR > 1 ? 256ull * ((s_n[tid] + 3u) >> 2) : 64ull * s_n[tid];
         if (x >= V.W) continue;
         for (int j = 0; j < cnt; ++j) {
@@ -1344,15 +1357,16 @@ cudaError_t launch_det_bg_reduce(const float* bg_tiles, int n_tiles, float* gw, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_count_pairs(const float* rec, const unsigned* off, const unsigned* list, const Views& vs,
+cudaError_t launch_count_pairs(const float* rec, long long n, const unsigned* off, const unsigned* list, const Views& vs,
                                unsigned long long* count, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(unsigned long long), s);
     if (e != cudaSuccess || vs.total_tiles == 0) return e;
     const float4* r = reinterpret_cast<const float4*>(rec);
-    if (vs.tile_w == 16 && vs.tile_h == 16) k_count_pairs<16, 16, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 8 && vs.tile_h == 8) k_count_pairs<8, 8, 2><<<vs.total_tiles, 32, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 32 && vs.tile_h == 8) k_count_pairs<32, 8, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, count);
-    else if (vs.tile_w == 16 && vs.tile_h == 8) k_count_pairs<16, 8, 2><<<vs.total_tiles, 64, 0, s>>>(r, off, list, vs, count);
+    const bool light = sparse_view(vs, n * vs.n);
+    if (vs.tile_w == 16 && vs.tile_h == 16) k_count_pairs<16, 16, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, light, count);
+    else if (vs.tile_w == 8 && vs.tile_h == 8) k_count_pairs<8, 8, 2><<<vs.total_tiles, 32, 0, s>>>(r, off, list, vs, light, count);
+    else if (vs.tile_w == 32 && vs.tile_h == 8) k_count_pairs<32, 8, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, light, count);
+    else if (vs.tile_w == 16 && vs.tile_h == 8) k_count_pairs<16, 8, 2><<<vs.total_tiles, 64, 0, s>>>(r, off, list, vs, light, count);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }

@@ -154,7 +154,7 @@ cudaError_t launch_det_pmax(const float* out_rgb, const float* out_den, const fl
                             unsigned* pmax, cudaStream_t s);
 cudaError_t launch_det_bg_reduce(const float* bg_tiles, int n_tiles, float* grad_wparams, cudaStream_t s);
 
-cudaError_t launch_count_pairs(const float* records, const unsigned* tile_offsets, const unsigned* tile_list,
+cudaError_t launch_count_pairs(const float* records, long long n, const unsigned* tile_offsets, const unsigned* tile_list,
                                const Views& vs, unsigned long long* count, cudaStream_t s);
 
 cudaError_t launch_loss_l1(const float* rgb, const float* target, long long count,
