@@ -75,6 +75,10 @@ enum { WSR_OPACITY_LOGIT = 0, WSR_OPACITY_SH = 1 };
  * WSR_BIN_ONE_GAUSSIANS Gaussians times views (half as many beyond 1024 tiles) */
 #define WSR_BIN_ONE_TILES 4096
 #define WSR_BIN_ONE_GAUSSIANS 8192
+/* wsr_render_bwd orders the tiles itself with the per-tile schedule beyond WSR_ORDER_MIN_TILES of them, in one kernel
+ * up to WSR_ORDER_ONE_BLOCK_TILES, else in two */
+#define WSR_ORDER_MIN_TILES 1024
+#define WSR_ORDER_ONE_BLOCK_TILES 16384
 
 /* Pinhole camera (passed by value through host memory). */
 typedef struct {

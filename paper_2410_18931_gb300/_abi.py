@@ -26,6 +26,8 @@ WSR_DET_MAX_SEGMENT = 8192
 WSR_SCAN_ONE_BLOCK_TILES = 32768     # wsr_bin scans (and orders) up to this many tiles in one kernel
 WSR_BIN_ONE_TILES = 4096             # wsr_bin makes one launch for at most this many tiles over all views
 WSR_BIN_ONE_GAUSSIANS = 8192         # and this many Gaussians times views (half as many beyond 1024 tiles)
+WSR_ORDER_MIN_TILES = 1024           # the backward orders the per-tile schedule's tiles beyond this many
+WSR_ORDER_ONE_BLOCK_TILES = 16384    # in one kernel up to this many, else in two
 WSR_BIN_STATIC_MAX_TILES = 65536     # tiles over all views that wsr_bin_static handles
 WSR_BIN_STATIC_BYTES = 270848        # its fixed scratch array, held by every GPU that loads the library
 

@@ -93,15 +93,19 @@ struct WsLayout {
 WsLayout ws_layout(const Views& vs, bool render = true) {
     WsLayout L;
     const size_t nb = (size_t)(vs.total_tiles + kScanTile - 1) / kScanTile;
-    L.cursor = kWsHeader;
-    L.block_sums = L.cursor + align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
-    L.total = L.block_sums + align256(sizeof(unsigned long long) * (nb + 1));
+    const size_t per_tile = align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
     L.order = L.buckets = L.bg_tiles = L.bwd_work = L.bin_base = 0;
+    L.cursor = kWsHeader;
+    if (render) {
+        L.buckets = kWsHeader;
+        L.bwd_work = L.buckets + align256(sizeof(unsigned) * 66);
+        L.cursor = L.bwd_work + per_tile;
+    }
+    L.block_sums = L.cursor + per_tile;
+    L.total = L.block_sums + align256(sizeof(unsigned long long) * (nb + 1));
     if (!render) return L;
     L.order = L.total;
-    L.buckets = L.order + align256(sizeof(unsigned) * (size_t)vs.total_tiles);
-    L.bwd_work = L.buckets + align256(sizeof(unsigned) * 66);
-    L.total = L.bwd_work + align256(sizeof(unsigned) * ((size_t)vs.total_tiles + 1));
+    L.total = L.order + align256(sizeof(unsigned) * (size_t)vs.total_tiles);
     if (vs.det) {
         L.bg_tiles = L.total;
         L.total = L.bg_tiles + align256(4 * sizeof(float) * (size_t)vs.total_tiles);
@@ -408,28 +412,30 @@ wsr_status wsr_render_bwd_tiles(const float* records, int64_t n, const uint32_t*
         return WSR_ERR_INVALID_ARG;
     if ((unsigned long long)n * (unsigned long long)n_cams > 0xffffffffull) return WSR_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    WsHeader* hdr = (WsHeader*)workspace;
-    WSR_CUDA(cudaMemsetAsync(hdr->gw, 0, sizeof hdr->gw, s));
-    const size_t rec_floats = vs.det ? WSR_GRAD_RECORD_FLOATS_DET : WSR_GRAD_RECORD_FLOATS;
-    if (n > 0) WSR_CUDA(cudaMemsetAsync(grad_records, 0, sizeof(float) * rec_floats * (size_t)n * n_cams, s));
     const WsLayout L = ws_layout(vs);
     char* const ws = (char*)workspace;
+    WsSums* const sums = (WsSums*)(ws + kWsSums);
+    // the sums, the order's buckets and the counters of tiles and parts in one clear
+    WSR_CUDA(cudaMemsetAsync(sums, 0, L.bwd_work - kWsSums + sizeof(unsigned) * ((size_t)vs.total_tiles + 1), s));
+    const size_t rec_floats = vs.det ? WSR_GRAD_RECORD_FLOATS_DET : WSR_GRAD_RECORD_FLOATS;
+    if (n > 0) WSR_CUDA(cudaMemsetAsync(grad_records, 0, sizeof(float) * rec_floats * (size_t)n * n_cams, s));
     // the binning leaves the tile order only for the persistent schedule
-    BwdSched sched{vs.total_tiles > kFewTiles ? (const unsigned*)(ws + L.order) : nullptr, (unsigned*)(ws + L.bwd_work)};
+    BwdSched sched{vs.total_tiles > WSR_ORDER_MIN_TILES ? (const unsigned*)(ws + L.order) : nullptr,
+                   (unsigned*)(ws + L.bwd_work)};
     if (vs.schedule != WSR_SCHEDULE_PERSISTENT && sched.order)
         WSR_CUDA(launch_tile_order(vs, tile_offsets, (unsigned*)(ws + L.buckets), (unsigned*)(ws + L.order), s));
     if (!vs.det) {
         WSR_CUDA(launch_render_bwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den, grad_rgb, grad_records,
-                                   hdr->gw, false, nullptr, nullptr, sched, s));
+                                   sums->gw, false, nullptr, nullptr, sched, s));
         return WSR_OK;
     }
     // deterministic: the largest pixel term over the image, then the record terms as exact fixed-point sums
     // in units that a per-Gaussian bound fixes; the background terms per tile, then summed in tile order
     float* bg_tiles = (float*)(ws + L.bg_tiles);
-    WSR_CUDA(launch_det_pmax(out_rgb, out_den, grad_rgb, vs.total_pix, &hdr->det_pmax, s));
+    WSR_CUDA(launch_det_pmax(out_rgb, out_den, grad_rgb, vs.total_pix, &sums->det_pmax, s));
     WSR_CUDA(launch_render_bwd(records, tile_offsets, tile_list, vs, wd, out_rgb, out_den, grad_rgb, grad_records,
-                               hdr->gw, true, bg_tiles, &hdr->det_pmax, sched, s));
-    WSR_CUDA(launch_det_bg_reduce(bg_tiles, vs.total_tiles, hdr->gw, s));
+                               sums->gw, true, bg_tiles, &sums->det_pmax, sched, s));
+    WSR_CUDA(launch_det_bg_reduce(bg_tiles, vs.total_tiles, sums->gw, s));
     return WSR_OK;
 }
 
@@ -447,13 +453,13 @@ wsr_status wsr_project_bwd(const wsr_gaussians* g, const wsr_camera* cams, int32
     WSR_TRY(check_gauss(g, n_cams, wd.kind, &gp));
     if (gp.n > 0 && (!grad_records || !aligned16(grad_records))) return WSR_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    WsHeader* hdr = (WsHeader*)workspace;
+    float* const gw = ((WsSums*)((char*)workspace + kWsSums))->gw;
     wsr_grads inner = *grads;
-    inner.weight_params = hdr->gw;
+    inner.weight_params = gw;
     float* sb = det ? (float*)((char*)workspace + kWsDetSB) : nullptr;   // sigma/beta per block
     WSR_CUDA(launch_project_bwd(gp, vs, wd, grad_records, inner, sb, s));
     if (grads->weight_params)
-        WSR_CUDA(cudaMemcpyAsync(grads->weight_params, hdr->gw, 6 * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        WSR_CUDA(cudaMemcpyAsync(grads->weight_params, gw, 6 * sizeof(float), cudaMemcpyDeviceToDevice, s));
     return WSR_OK;
 }
 

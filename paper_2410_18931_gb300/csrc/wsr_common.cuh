@@ -45,26 +45,34 @@ struct Views {
     View v[WSR_MAX_VIEWS];
 };
 
-// Workspace layout: [header 8 KB][cursor: total_tiles + 1 u32][block sums]
-//                   [tile order: total_tiles u32][order buckets: 66 u32]
-//                   [backward: counter and chunks taken per tile, total_tiles + 1 u32]
+// Workspace layout: [header 8 KB]
+//                   [order buckets: 66 u32]
+//                   [backward: counter and parts taken per tile, total_tiles + 1 u32]
+//                   [cursor: total_tiles + 1 u32][block sums]
+//                   [tile order: total_tiles u32]
 //                   [deterministic mode: background terms per tile, 4 floats]
 //                   [binning: a row of counters per block of k_bin_local]
-// The header's first 256 bytes are the struct below; in deterministic mode the
-// projection backward keeps its per-block sigma/beta sums after it.
+// The header's first 256 bytes are the first struct below; in deterministic
+// mode the projection backward keeps its per-block sigma/beta sums after it.
+// Its last 64 bytes are the second struct, so that one clear zeroes it and
+// the backward's regions behind it.
 struct WsHeader {
     int err;                   // first device-side error (wsr_status), 0 if none
     int pad0;
-    float gw[8];               // gradient accumulators of sigma, beta, w_B, c_B (6 used)
     unsigned long long total;  // tile instances counted by the last binning
     unsigned int work[4];      // [0] the forward's persistent-schedule counter
+};
+struct WsSums {
+    float gw[8];               // gradient accumulators of sigma, beta, w_B, c_B (6 used)
     unsigned int det_pmax;     // deterministic mode: the largest |pixel term| G/D, (G.C)/D (float bits)
+    unsigned int pad[7];
 };
 
 constexpr size_t kWsHeader = 8192;
+constexpr size_t kWsSums = kWsHeader - sizeof(WsSums);
 constexpr size_t kWsDetSB = 256;       // deterministic mode: sigma/beta per projection-backward block
 constexpr int kDetBlocks = 608;        // most of them
-static_assert(kDetBlocks <= (int)((kWsHeader - kWsDetSB) / (2 * sizeof(float))), "sigma/beta sums in the header");
+static_assert(kDetBlocks <= (int)((kWsSums - kWsDetSB) / (2 * sizeof(float))), "sigma/beta sums in the header");
 // Deterministic mode: a record term is added as 64-bit fixed point in units of
 // 2^(e - kDetBits), 2^e above an a-priori bound on the sum of the absolute
 // values of all its partials (over every tile of the Gaussian), so the exact

@@ -115,7 +115,9 @@ cudaError_t launch_sort_segments(const Views& vs, const unsigned* tile_offsets, 
                                  WsHeader* hdr, cudaStream_t s);
 
 // Views of at most this many tiles (four per SM) leave SMs idle with a block per tile: the forward then splits each
-// tile's list in two, and the backward takes smaller chunks and needs no order.
+// tile's list in two, and the backward takes smaller chunks.  (It needs no order up to WSR_ORDER_MIN_TILES: few blocks
+// take a second tile, and idle ones look at every tile's parts.  640 tiles of 10000 Gaussians 31 -> 20 us, of which
+// the order was 4.)
 constexpr int kFewTiles = 608;
 
 // Work distribution of a forward launch: order == nullptr means one block per
@@ -130,12 +132,12 @@ cudaError_t launch_render_fwd(const float* records, long long n, const unsigned*
                               const unsigned* tile_list, const Views& vs, WeightDev w,
                               float* out_rgb, float* out_den, Sched sched, cudaStream_t s);
 
-// The longest-first tile order of a binning's offsets (`buckets`: 66 words of scratch).
+// The longest-first tile order of a binning's offsets (`buckets`: 66 words, zero).
 cudaError_t launch_tile_order(const Views& vs, const unsigned* tile_offsets, unsigned* buckets, unsigned* order,
                               cudaStream_t s);
 
-// Work distribution of a backward launch: the tile order (nullptr: as numbered), and total_tiles + 1 words that the
-// launcher clears: the counter of tiles taken, then each tile's counter of chunks taken.
+// Work distribution of a backward launch: the tile order (nullptr: as numbered), and total_tiles + 1 words, zero: the
+// counter of tiles taken past the blocks' first ones, then each tile's counter of parts taken.
 struct BwdSched {
     const unsigned* order;
     unsigned* counter;

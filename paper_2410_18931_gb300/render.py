@@ -94,16 +94,16 @@ class Renderer:
         self.tile = tuple(tile)
         self.num_tiles = int(self.lib.wsr_num_tiles(self.cams_c, self.n_cams, ctypes.byref(self.tiles_c)))
         # kernels one wsr_bin launches (bin_launches: small scenes make fewer): the count; the scan, in one kernel (with the persistent schedule's
-        # tile order) up to WSR_SCAN_ONE_BLOCK_TILES tiles, else three (and three for the order); the
+        # tile order) up to WSR_SCAN_ONE_BLOCK_TILES tiles, else three (and two for the order); the
         # scatter; in the deterministic mode the sort of each tile's list
         if self.num_tiles <= A.WSR_SCAN_ONE_BLOCK_TILES:
             self.bin_kernels = 3
         else:
-            self.bin_kernels = 5 + (3 if persistent else 0)
+            self.bin_kernels = 5 + (2 if persistent else 0)
         self.bin_kernels += 1 if self.deterministic else 0
-        # kernels the backward launches to order the tiles when the binning has not (the per-tile schedule): none for
-        # few tiles, one up to 16384, else three
-        self.order_kernels = 0 if persistent or self.num_tiles <= 608 else 1 if self.num_tiles <= 16384 else 3
+        # kernels the backward launches to order the tiles when the binning has not (the per-tile schedule)
+        self.order_kernels = (0 if persistent or self.num_tiles <= A.WSR_ORDER_MIN_TILES else
+                              1 if self.num_tiles <= A.WSR_ORDER_ONE_BLOCK_TILES else 2)
         self.num_pix = int(self.lib.wsr_num_pixels(self.cams_c, self.n_cams))
         ws = int(self.lib.wsr_workspace_size(self.cams_c, self.n_cams, ctypes.byref(self.tiles_c)))
         if self.num_tiles <= 0 or ws == 0:
