@@ -330,8 +330,12 @@ __device__ __forceinline__ void rows_out(float* __restrict__ g, const float* __r
 // several views add theirs in rows beside them.  Below degree 2 the rows are short and stay in registers.
 //   One view, 1M Gaussians of degree 3 with view-dependent opacity: 138 -> 117 us (636 MB, 80% of the copy rate);
 // 400k of degree 2: 82 -> 37 us (rows of 27 floats took 4-byte accesses); six views of 300k, degree 2: 128 -> 84 us.
-// Blocks per SM: at degree 3 four, for five the registers spill (136 us).
-template <int DEG, bool VD, bool RED, bool ONE>
+// Blocks per SM: at degree 3 four, which spills up to 36 bytes with view-dependent opacity; five spill more (136 us).
+// Small scenes of degree 3 pay for the way through shared memory: one view of 2000 6.0 -> 6.5 us, of 100k 16.4 -> 17.7
+// (three views 26 -> 23.6); 20k 8.1 -> 7.4.
+//   The deterministic mode's records are a kernel of their own (DET): as a branch they cost the others 0.3 to 1.5 us,
+// 2000 of degree 0 in three views 7.3 -> 6.6, 100k of degree 1 12.2 -> 10.7.
+template <int DEG, bool VD, bool RED, bool ONE, bool DET>
 __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) : (DEG == 3 ? 3 : DEG == 2 ? 4 : 1))
     k_project_bwd(const GaussPtrs g, const Views vs, const WeightDev wd, const float* __restrict__ grec,
                   const wsr_grads out, float* __restrict__ det_sb) {
@@ -350,8 +354,8 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
     float* const s_det = ROWS ? s_ga + 128 * PA : s_rows;
     float gsig = 0.0f, gbeta = 0.0f;
     const float sigma = __ldg(wd.params + 0), beta = __ldg(wd.params + 1);
-    // det_sb != nullptr: deterministic mode (fixed-point records, a bounded grid striding over the
-    // Gaussians, sigma/beta summed per block in a fixed order into det_sb)
+    // DET: deterministic mode (fixed-point records, a bounded grid striding over the Gaussians, sigma/beta
+    // summed per block in a fixed order into det_sb)
     for (long long i0 = 128ll * blockIdx.x; i0 < g.n; i0 += 128ll * gridDim.x) {
         const int cnt = (int)min(128ll, g.n - i0);
         const long long i = i0 + threadIdx.x;
@@ -389,7 +393,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
                              "l"(from + (c / 7 * 8 + c % 7)) : "memory");
             }
         };
-        if (det_sb) copy_det(0);
+        if constexpr (DET) copy_det(0);
         else if (mine) load_record(0);
         auto get_h = [&](float (&h)[3 * K], float (&ha)[KA]) {
             if constexpr (ROWS) {
@@ -426,7 +430,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
         };
         const float zero_h[3 * K] = {}, zero_a[KA] = {};
         if constexpr (!ONE || !ROWS) put_g(zero_h, zero_a);
-        if (ROWS || det_sb) {
+        if constexpr (ROWS || DET) {
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
         }
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
 
         const int nv = ONE ? 1 : vs.n;
         for (int v = 0; v < nv; ++v) {
-            if (det_sb && v > 0) {
+            if (DET && v > 0) {
                 __syncthreads();                // the last view's records are read
                 copy_det(v);
                 asm volatile("cp.async.wait_all;" ::: "memory");
@@ -451,7 +455,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
             const View& V = vs.v[v];
             float g9[9];
             bool any = false;
-            if (det_sb == nullptr) {
+            if constexpr (!DET) {
                 g9[0] = ra.x, g9[1] = ra.y, g9[2] = ra.z, g9[3] = ra.w;
                 g9[4] = rb.x, g9[5] = rb.y, g9[6] = rb.z, g9[7] = rb.w;
                 g9[8] = rc;
@@ -661,7 +665,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
             if (out.sh) rows_out<3 * K>(out.sh + 3ll * K * i0, s_gh, cnt);
             if (out.opacity) rows_out<KA>(out.opacity + (long long)KA * i0, s_ga, cnt);
         }
-        if (ROWS || det_sb) __syncthreads();    // the rows and records are read
+        if constexpr (ROWS || DET) __syncthreads();    // the rows and records are read
     }
     // global weight parameters: warp reduce, then one atomic per warp, or (deterministic) the block's sums
     // in warp order
@@ -670,7 +674,7 @@ __global__ void __launch_bounds__(128, ONE ? (DEG == 3 ? 4 : DEG == 2 ? 6 : 3) :
         gsig += __shfl_xor_sync(0xffffffffu, gsig, off);
         gbeta += __shfl_xor_sync(0xffffffffu, gbeta, off);
     }
-    if (det_sb != nullptr) {
+    if constexpr (DET) {
         __shared__ float swb[2][4];
         if ((threadIdx.x & 31) == 0) {
             swb[0][threadIdx.x >> 5] = gsig;
@@ -740,16 +744,20 @@ cudaError_t project_bwd_t(const GaussPtrs& g, const Views& vs, WeightDev w, cons
     if (e0 != cudaSuccess) return e0;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::call_once(once[dev], [&] {
-        once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, rows + det_rows);
-        if (once_err[dev] == cudaSuccess)
-            once_err[dev] = cudaFuncSetAttribute(k_project_bwd<DEG, VD, RED, false>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 2 * rows + det_rows);
+        auto most = [&](auto kernel, int bytes) {
+            if (once_err[dev] == cudaSuccess && bytes)
+                once_err[dev] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        };
+        once_err[dev] = cudaSuccess;
+        most(k_project_bwd<DEG, VD, RED, true, false>, rows);
+        most(k_project_bwd<DEG, VD, RED, false, false>, 2 * rows);
+        most(k_project_bwd<DEG, VD, RED, true, true>, rows + det_rows);
+        most(k_project_bwd<DEG, VD, RED, false, true>, 2 * rows + det_rows);
     });
     if (once_err[dev] != cudaSuccess) return once_err[dev];
-    if (vs.n == 1) k_project_bwd<DEG, VD, RED, true><<<(unsigned)nb, bs, rows + more, s>>>(g, vs, w, grec, out, det_sb);
-    else k_project_bwd<DEG, VD, RED, false><<<(unsigned)nb, bs, 2 * rows + more, s>>>(g, vs, w, grec, out, det_sb);
+    auto kernel = vs.n == 1 ? det_sb ? k_project_bwd<DEG, VD, RED, true, true> : k_project_bwd<DEG, VD, RED, true, false>
+                            : det_sb ? k_project_bwd<DEG, VD, RED, false, true> : k_project_bwd<DEG, VD, RED, false, false>;
+    kernel<<<(unsigned)nb, bs, (vs.n == 1 ? rows : 2 * rows) + more, s>>>(g, vs, w, grec, out, det_sb);
     if (det_sb) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
