@@ -358,7 +358,10 @@ cudaError_t launch_loss_3dgs(const float* rgb, const float* target, const LossVi
 
 // Strips and segments of the views (tiles_x, tile_off, rows).  A segment takes as many batches of 11 rows as its
 // rows and 20 more need, so the rows are 11 k - 20; k is the one whose last wave of 304 blocks (two per SM) ends
-// first: a batch of 11 rows costs about the same wherever it lies, so the waves times k are the time.  False when the views hold too many.
+// first: a batch of 11 rows costs about the same wherever it lies, 8.0 us for two blocks on an SM and 4.9 for one
+// (and 2.5 to begin with), which a last wave of at most 152 blocks has.  Weighed as whole waves, 640x360 took 24.8
+// instead of 22.7 us (k 3 instead of 4), 801x601 40.5 instead of 37.0 (5, 7), 65x5000 33 instead of 27 (4, 5), 32
+// views of 64x64 24.8 instead of 22.7 (3, 4).  False when the views hold too many.
 bool loss_plan(LossViews& L) {
     long long best = 0;
     for (int k = 3; k <= 32; ++k) {
@@ -366,7 +369,8 @@ bool loss_plan(LossViews& L) {
         long long blocks = 0;
         for (int v = 0; v < L.n; ++v)
             blocks += (long long)((L.w[v] + kOP - 1) / kOP) * ((L.h[v] + rows - 1) / rows);
-        const long long cost = (blocks + 303) / 304 * k;
+        const long long rest = blocks % 304;
+        const long long cost = (blocks / 304 + (rest > 152)) * 80 * k + (rest > 0 && rest <= 152 ? 49 * k + 25 : 0);
         if (best == 0 || cost < best) {
             best = cost;
             L.rows = rows;
