@@ -1132,19 +1132,24 @@ cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks
 }
 
 // Records per 1024 pixels up to which the kernel for sparse views is taken (the lists' lengths are not known on the
-// host).  It against the other at 1920x1080, us, for Gaussians of three sizes (the second and third 4.5 and 12 times as
-// wide as the first):
-//   500 (0.25 per 1024)   9.4 and 17.5   11.4 and 24    26.5 and 36
-//   8000 (4)             12.1 and 23     57 and 56      303 and 264
-//   16000 (8)            16.4 and 26    108 and 95
-//   32000 (16)           25.7 and 31    213 and 174     (not taken)
-// in 8x8 tiles 19.3 and 25 and 109 and 106 at 16000, 26 and 32 and 209 and 193 at 32000; 16000 in two clusters of a
-// hundred tiles 151 and 85.  So where it is taken it loses at most a seventh to lists of hundreds of entries, and past
-// the limit wide Gaussians would lose more than narrow ones gain.  Deciding per tile (lists past 64 entries left to a
-// second launch of the other kernel) gives the clusters 79 us, and takes 1.7 to 2 us from every sparse view.
-constexpr long long kSparse = 9;
+// host).  It and the other, us, for Gaussians of size exp(-4), five units away, and wider ones:
+//   1920x1080   500 (0.25 per 1024)   9.4, 17.5   exp(-2.5) 11.4, 24   exp(-1.5) 26.5, 36
+//               8000 (4)             12.1, 23     exp(-2.5) 57, 56     exp(-1.5) 303, 264
+//               20000 (10)           18.7, 27     exp(-3.5) 31, 35
+//               32000 (16)           25.7, 31     exp(-2.5) 213, 174
+//               50000 (25)           35.9, 37                           (not taken)
+//   1280x720    10000 (11)            8.5, 12.7   exp(-3) 21.1, 20.7
+//   979x543     8000 (15)             7.7, 9.8    exp(-2.5) 27, 21
+//               10000 (19)            8.4, 9.8    exp(-3) 18.0, 15.2    (not taken)
+// In 8x8 tiles, whose lists are shorter, 32000 at 1920x1080 take 26 and 32, 50000 at 1280x720 (56) 21.9 and 22.4, of
+// exp(-3) 10000 at 979x543 (19) 17.1 and 16.4.  So near the limits Gaussians of a trained scene's size gain a fifth,
+// and wide ones lose up to a third (the two cases of 27 and 213 took 30 and 214 before there were two kernels).  16000
+// in two clusters of a hundred tiles take 151 and 85.  Deciding per tile (lists past 64 entries left to a second launch
+// of the other kernel) gives the clusters 79 us, and takes 1.7 to 2 us from every sparse view.
+constexpr long long kSparse = 16, kSparse8 = 40;
 inline bool sparse_view(const Views& vs, const long long n_records) {
-    return vs.total_tiles > kFewTiles && n_records * 1024 <= kSparse * vs.total_tiles * (vs.tile_w * vs.tile_h);
+    const int pixels = vs.tile_w * vs.tile_h;
+    return vs.total_tiles > kFewTiles && n_records * 1024 <= (pixels == 64 ? kSparse8 : kSparse) * vs.total_tiles * pixels;
 }
 
 // S slices, or 0: the kernel for sparse views

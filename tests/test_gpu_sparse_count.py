@@ -44,6 +44,6 @@ def test_sparse_slots(tile):
             dx, dy = x0[:, None, None] + fx, y0[:, None, None] + fy[:, None]
             hi += int(((qs * dy + qw * dx) ** 2 + qd * dx ** 2 <= 9.3 * 0.7213475).any(axis=(1, 2)).sum())
         assert slots % 128 == 0 and lo * 128 <= slots <= hi * 128
-    st.n = 9 * r.num_tiles * tile[0] * tile[1] // 1024 + 1
+    st.n = r.num_pix
     pairs2, slots2, _ = r.wsr_count_pairs(st)
     assert pairs2 == pairs and slots2 != slots if tile != (8, 8) else slots2 <= slots
