@@ -51,7 +51,7 @@ MUFU_PER_SM = 16         # ex2 / rsqrt / rcp results per SM and clock
 SM_MAX_MHZ = 2070.0
 METRIC = "fwd and fwd+bwd Mpix/s at 1M Gaussians 1080p vs plain FP32 path; max err"
 # project 1, fwd 1, loss 1, bwd tiles 1, project bwd 1; plus wsr_bin's and the backward's tile order, where the
-# binning makes none (Renderer.bin_kernels, order_kernels)
+# binning makes none (Renderer.bin_launches, order_kernels)
 KERNELS_PER_STEP = 5
 
 
@@ -464,7 +464,7 @@ def run_ours(args):
     scene, cam, weight, extra, target = build_workload(args, rank, world)
     tile, persistent, chunk, tune_ms = launch_config(args, scene, cam, weight, target)
     S = Step(scene, cam, weight, tile, target, persistent, chunk)
-    kernels_per_step = KERNELS_PER_STEP + S.r.bin_kernels + S.r.order_kernels
+    kernels_per_step = KERNELS_PER_STEP + S.r.bin_launches(S.g.n) + S.r.order_kernels
     A = S.A
     npix = cam.width * cam.height
     flush = torch.empty(512 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
@@ -648,7 +648,7 @@ def run_deterministic(S, scene, cam, weight, target, tile, persistent, chunk, fl
         stages.append([evs[k].elapsed_time(evs[k + 1]) for k in range(6)])
     ms = float(np.mean(times))
     st_ms = np.mean(np.array(stages), axis=0)
-    stage_names, bin_kernels = D.stage_names, D.r.bin_kernels + D.r.order_kernels
+    stage_names, bin_kernels = D.stage_names, D.r.bin_launches(D.g.n) + D.r.order_kernels
     del D, outs
     torch.cuda.empty_cache()
     return {"ms_per_step": round(ms, 4), "fwd_bwd_mpix_s": round(cam.width * cam.height / (ms * 1e-3) / 1e6, 2),

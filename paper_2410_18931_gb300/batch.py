@@ -32,7 +32,6 @@ class GraphStep:
         self.g, self.kind, self.wparams = g, kind, wparams
         self.r = Renderer(cams, tile=tile, persistent=persistent, headroom=headroom, chunk=chunk,
                           deterministic=deterministic)
-        self.r.bin_kernels = self.r.bin_launches(g.n)
         self.st = self.r.forward(g, kind, wparams)           # sizes the tile list exactly (+ headroom)
         self.target = target.reshape(-1, 3).contiguous()
         dev = self.r.device
@@ -81,9 +80,9 @@ class GraphStep:
 
     @property
     def kernels_per_step(self) -> int:
-        # project 1, bin (bin_kernels), fwd 1, loss 1, bwd 1 (and its tile order), project bwd 1;
+        # project 1, bin (bin_launches), fwd 1, loss 1, bwd 1 (and its tile order), project bwd 1;
         # deterministic: + the largest-pixel-term kernel and two ordered reductions
-        return 5 + self.r.bin_kernels + self.r.order_kernels + (3 if self.r.deterministic else 0)
+        return 5 + self.r.bin_launches(self.g.n) + self.r.order_kernels + (3 if self.r.deterministic else 0)
 
 
 def time_step(step: GraphStep, reps: int = 5, warmup: int = 2, flush: torch.Tensor | None = None) -> float:
