@@ -255,8 +255,9 @@ __global__ void __launch_bounds__(kLossThreads, 2) k_loss_3dgs(const float* __re
 }
 
 // The next step's number and bias corrections 1 / (1 - b1^t) and 1 / sqrt(1 - b2^t), a lane each.  One chain of FP64
-// operations bounds it, so the powers are formed by squaring (2 log2 t products; relative error below 1e-14, far under
-// the float results' 6e-8) beside each other: 9.4 us with two calls of pow() one after the other, 3.5 us.
+// operations bounds it, so the powers are formed by squaring (2 log2 t products) beside each other: 9.4 us with two calls
+// of pow() one after the other, 3.5 us.  A power's relative error grows as t 2^-53, and b^t damps it in 1 - b^t: below
+// 2^-52 / (1 - b), 2e-13 for b = 0.999 and 2e-12 for 0.9999, far under the float results' 6e-8.
 __global__ void k_adam_tick(AdamState* st, const WsHeader* guard, double b1, double b2) {
     if (guard && guard->err != 0) {
         if (threadIdx.x == 0) st->skipped += 1;
