@@ -549,7 +549,10 @@ __device__ __forceinline__ void fwd_tile_light(const int tile, const float4* __r
     }
 }
 
-// Persistent schedule: blocks take tiles order[0..n) through *counter.
+// Persistent schedule: block i takes the tile order[i], and then the others through *counter.  Dealt by their numbers
+// the longest tiles spread over the SMs where every block has one (claimed through the counter they lie anywhere: 2108
+// tiles of wide Gaussians in the sparse kernel, 979x543, 39 -> 23 us), and views of no more tiles than blocks need
+// neither counter nor clear (1000 Gaussians at 200x120 8.4 -> 4.1 us, at 500x313 8.4 -> 4.2).
 template <typename F>
 __device__ __forceinline__ void for_each_tile(const unsigned* __restrict__ order, unsigned* __restrict__ counter,
                                               int n_tiles, F&& body) {
@@ -558,13 +561,13 @@ __device__ __forceinline__ void for_each_tile(const unsigned* __restrict__ order
         return;
     }
     __shared__ int s_item;
-    for (;;) {
-        __syncthreads();                      // the previous tile is done with shared memory
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n_tiles) break;
+    for (int item = (int)blockIdx.x; item < n_tiles;) {
         body((int)order[item]);
+        if ((int)gridDim.x >= n_tiles) break;
+        __syncthreads();                      // the tile is done with shared memory
+        if (threadIdx.x == 0) s_item = (int)(gridDim.x + atomicAdd(counter, 1u));
+        __syncthreads();
+        item = s_item;
     }
 }
 
@@ -1166,7 +1169,7 @@ cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, c
     if (sched.order) {
         int most = 0;
         cudaError_t e = resident_blocks(known, kernel, NT, most);
-        if (e == cudaSuccess) e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
+        if (e == cudaSuccess && most < grid) e = cudaMemsetAsync(sched.counter, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
         grid = min(grid, most);
     }
