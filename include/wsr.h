@@ -143,9 +143,9 @@ enum {
  * wsr_render_fwd launches one block per resident slot that takes tiles from
  * that order through a counter in the workspace; the same workspace and tiles
  * must then be passed to wsr_bin and the renderers.  The backward always takes
- * tiles that way (it forms the order itself for the other schedule) and splits
- * the longest lists over blocks.  `chunk` is how many of a tile's Gaussians a
- * block of wsr_render_bwd takes at a time: 64 (blocks of 128 threads), 128, 256
+ * tiles that way (it forms the order itself for the other schedule, beyond
+ * WSR_ORDER_MIN_TILES tiles) and splits the longest lists over blocks.  `chunk`
+ * is how many of a tile's Gaussians a block of wsr_render_bwd takes at a time: 64 (blocks of 128 threads), 128, 256
  * or 512 (blocks of 256 threads), or 0 for the default, 512 (128 for views of
  * at most 608 tiles); other values return WSR_ERR_UNSUPPORTED.  It changes the
  * schedule only, not the result beyond rounding order.

@@ -206,12 +206,12 @@ __global__ void __launch_bounds__(256) k_bin(const float4* __restrict__ rec, lon
 // every tile of its view.  Block b of a view takes the batches of 32 Gaussians b, b + B, ... (its warps
 // one after another as they come free) in both passes.  COUNT: the block's counts per tile, then one
 // global atomic per tile that it reaches; what that returns, the block's first place among the tile's
-// instances, is kept in `base` (a row of T entries per block; nullptr: not asked for).  SCATTER: the block's cursors start at
-// the tile's offset plus that place, so a slot costs one shared atomic.
+// instances, is kept in `base` (a row of T entries per block; nullptr: not asked for).  SCATTER: the block's cursors start
+// at the tile's offset plus that place, so a slot costs one shared atomic.
 //   The global counters bound the plain pass: neighbouring tiles share 32-byte sectors, and a view's
 // counters are only a few kilobytes, so the atomics of all SMs queue at a few L2 lines.  Measured, count,
 // scan and scatter: 171 -> 87 us for 1M Gaussians at 1920x1080 (6.3M instances), 392 -> 126 us for 300k
-// in six views (6.3M instances, the smallest view 920 tiles), 17.5 -> 17.1 us for 1000 at 128x128.  What
+// in six views (6.3M instances, the smallest view 920 tiles), 21 -> 15 us for 10000 at 979x543.  What
 // is left is the latency of a warp's chain (records, prefix, segments, tiles) at 48 warps per SM.
 template <int NT, bool SCATTER>
 __global__ void __launch_bounds__(NT, NT > 768 ? 1 : 2)
