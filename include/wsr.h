@@ -273,7 +273,7 @@ wsr_status wsr_bin_total(const void* workspace, size_t workspace_bytes, uint64_t
 /*
  * wsr_render_fwd — Eq. 7 per pixel, one thread block per tile or (WSR_SCHEDULE_PERSISTENT) one per resident slot.
  * The kernel, and with it the order in which a pixel's terms are added, depends on the number of tiles and on n (the
- * records per view) against the pixels.
+ * records per view) against the views' pixels.
  *   out_rgb  [num_pixels, 3] float32 output, views concatenated in order, each
  *            view row-major (y * width + x)
  *   out_den  [num_pixels] float32 output: the full denominator w_B + sum a_i

@@ -1149,10 +1149,19 @@ cudaError_t resident_blocks(PerDevice& known, K kernel, int threads, int& blocks
 // and wide ones lose up to a third (the two cases of 27 and 213 took 30 and 214 before there were two kernels).  16000
 // in two clusters of a hundred tiles take 151 and 85.  Deciding per tile (lists past 64 entries left to a second launch
 // of the other kernel) gives the clusters 79 us, and takes 1.7 to 2 us from every sparse view.
-constexpr long long kSparse = 16, kSparse8 = 40;
-inline bool sparse_view(const Views& vs, const long long n_records) {
-    const int pixels = vs.tile_w * vs.tile_h;
-    return vs.total_tiles > kFewTiles && n_records * 1024 <= (pixels == 64 ? kSparse8 : kSparse) * vs.total_tiles * pixels;
+//   A view with many records for its pixels has long lists, and they set the end of the whole batch: the sparse
+// kernel's time lost there is about 0.5 us per record and 256 pixels of the densest view, and what it gains elsewhere
+// 1.4 us per 1000 times 256 pixels, so in wide tiles it also needs 480 n <= all pixels / 256 times the densest view's
+// / 256.  Frames of 2832 Gaussians in 846x566, 667x375 and 148x83 104 and 81 us, 4796 in 1334x750 and 222x222 97 and
+// 83, 8569 in 1805x1015 and 539x539 80 and 88 (taken), 1037 in 1389x1389, 1098x1098 and 145x108 105 and 115 (taken).
+constexpr long long kSparse = 16, kSparse8 = 40, kDenseView = 480;
+inline bool sparse_view(const Views& vs, const long long n) {
+    const long long pixels = vs.tile_w * vs.tile_h, all = vs.total_tiles * pixels;
+    if (vs.total_tiles <= kFewTiles || n * vs.n * 1024 > (pixels == 64 ? kSparse8 : kSparse) * all) return false;
+    if (pixels == 64) return true;
+    long long least = all;
+    for (int v = 0; v < vs.n; ++v) least = min(least, vs.v[v].tiles_x * vs.v[v].tiles_y * pixels);
+    return kDenseView * n <= (all / 256) * (least / 256);
 }
 
 // S slices, or 0: the kernel for sparse views
@@ -1179,11 +1188,11 @@ cudaError_t fwd_s(const float* rec, const unsigned* off, const unsigned* list, c
 }
 
 template <int TW, int TH>
-cudaError_t fwd_t(const float* rec, long long n_records, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
+cudaError_t fwd_t(const float* rec, long long n, const unsigned* off, const unsigned* list, const Views& vs, WeightDev w,
                   float* rgb, float* den, Sched sched, cudaStream_t s) {
     // Two slices where the tiles alone leave the SMs idle: 14.4 -> 10.4 us at 240 tiles, 14.5 -> 13.7 at 475
     // (40k Gaussians), 14.4 -> 15.1 at 920, 39 -> 70 at 8160.
-    if (sparse_view(vs, n_records))
+    if (sparse_view(vs, n))
         return fwd_s<TW, TH, 0>(rec, off, list, vs, w, rgb, den, sched, s);
     return vs.total_tiles <= kFewTiles ? fwd_s<TW, TH, 2>(rec, off, list, vs, w, rgb, den, sched, s)
                                             : fwd_s<TW, TH, 1>(rec, off, list, vs, w, rgb, den, sched, s);
@@ -1361,10 +1370,10 @@ cudaError_t sm_count(int& sms) {
 cudaError_t launch_render_fwd(const float* rec, long long n, const unsigned* off, const unsigned* list, const Views& vs,
                               WeightDev w, float* rgb, float* den, Sched sc, cudaStream_t s) {
     if (vs.total_tiles == 0) return cudaSuccess;
-    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
-    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8>(rec, n * vs.n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 16) return fwd_t<16, 16>(rec, n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 8 && vs.tile_h == 8) return fwd_t<8, 8>(rec, n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 32 && vs.tile_h == 8) return fwd_t<32, 8>(rec, n, off, list, vs, w, rgb, den, sc, s);
+    if (vs.tile_w == 16 && vs.tile_h == 8) return fwd_t<16, 8>(rec, n, off, list, vs, w, rgb, den, sc, s);
     return cudaErrorInvalidValue;
 }
 
@@ -1405,7 +1414,7 @@ cudaError_t launch_count_pairs(const float* rec, long long n, const unsigned* of
     cudaError_t e = cudaMemsetAsync(count, 0, 3 * sizeof(unsigned long long), s);
     if (e != cudaSuccess || vs.total_tiles == 0) return e;
     const float4* r = reinterpret_cast<const float4*>(rec);
-    const bool light = sparse_view(vs, n * vs.n);
+    const bool light = sparse_view(vs, n);
     if (vs.tile_w == 16 && vs.tile_h == 16) k_count_pairs<16, 16, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, light, count);
     else if (vs.tile_w == 8 && vs.tile_h == 8) k_count_pairs<8, 8, 2><<<vs.total_tiles, 32, 0, s>>>(r, off, list, vs, light, count);
     else if (vs.tile_w == 32 && vs.tile_h == 8) k_count_pairs<32, 8, 2><<<vs.total_tiles, 128, 0, s>>>(r, off, list, vs, light, count);

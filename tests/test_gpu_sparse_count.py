@@ -47,3 +47,26 @@ def test_sparse_slots(tile):
     st.n = r.num_pix
     pairs2, slots2, _ = r.wsr_count_pairs(st)
     assert pairs2 == pairs and slots2 != slots if tile != (8, 8) else slots2 <= slots
+
+
+def test_a_dense_view_keeps_its_batch_from_the_sparse_kernel():
+    """Few records for all pixels, but many for a small view's: the whole batch takes the other kernel, and the count
+    of its slots is that of one record per pixel (tiles wider than 8; 8x8 ones go by all pixels alone)."""
+    import torch
+
+    from paper_2410_18931_gb300 import Gaussians, Renderer
+    sc = ws.random_scene(700, 9, sh_degree=0, vd_opacity=False, clusters=0, box=1.0, log_scale_mu=-3.0, log_scale_sd=0.8)
+    w = ws.default_weight(ws.EXP)
+    for tile in ((16, 16), (32, 8), (16, 8)):
+        slots = {}
+        for small in (False, True):
+            cams = [ws.look_at((0.1, -0.2, -3.0), width=601, height=403).rounded()]
+            if small:
+                cams.append(ws.look_at((0.1, -0.2, -3.0), width=57, height=43).rounded())
+            r = Renderer(cams, tile=tile)
+            st = r.forward(Gaussians.from_scene(sc), w.kind, torch.tensor(w.as_array(), device="cuda"))
+            own = r.wsr_count_pairs(st)[1]
+            st.n = r.num_pix
+            slots[small] = own, r.wsr_count_pairs(st)[1]
+        assert slots[True][0] == slots[True][1], tile
+        assert slots[False][0] != slots[False][1], tile
